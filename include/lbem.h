@@ -168,9 +168,10 @@ lbem_status lbem_set_receivers(lbem_t *h, int n, const long long *site, const in
  * 9-10), source (Eq. 3), equilibrium (Eq. 8), collision at tau = dt/2 (Eq. 17);
  * receivers sample the pre-collision fields.  One fused kernel launch per step,
  * or per two (three) steps where lbem_set_temporal_blocking enables it (two is
- * the default for 2D), enqueued on the stream (or replayed from
- * a cached CUDA graph when enabled by lbem_set_graphs).  Requires a medium.
- * nsteps >= 0. */
+ * the default for 2D), or, for a call of at least 3 steps of a 2D grid that keeps
+ * that default with no tile shape chosen, per 8 steps (see there), enqueued on the
+ * stream (or replayed from a cached CUDA graph when enabled by lbem_set_graphs).
+ * Requires a medium.  nsteps >= 0. */
 lbem_status lbem_step(lbem_t *h, int nsteps);
 
 /* Walls and absorbing layers (2D and 3D, LBEM_F32 storage; the paper treats
@@ -257,6 +258,10 @@ lbem_status lbem_set_watchdog(lbem_t *h, int every, double max_growth);
  * sites), walls and layers included; a dispersive pole without walls or a mu array with shape 0 at 4 per SM;
  * both bit-identical to their single steps.  With a pole and walls (or a pole with a mu array), and for
  * steps_per_pass = 3, every step of these media is a single step.
+ * With steps_per_pass = 2 and tile_shape = -1 (the default), a call of lbem_step of at least 3 steps on an FP32 grid
+ * of uniform mu without walls, a pole or a tensor runs 8 steps per launch by the marching kernel instead: a warp walks
+ * a strip of columns down its rows with 8 time levels in flight (the last launch of a call takes the steps left), the
+ * same bits again.  A tile shape >= 0 gives launches of two steps.
  * LBEM_ERR_ARG for values outside the current handle's set. */
 lbem_status lbem_set_temporal_blocking(lbem_t *h, int steps_per_pass, int tile_shape);
 
@@ -397,7 +402,8 @@ lbem_status lbem_adjoint(lbem_t *h, const float *trace_cot, float *grad_eps, dou
  * *best (may be NULL) receives the chosen variant id.  Where two steps per
  * launch apply and are enabled (lbem_set_temporal_blocking), every tile shape
  * of that kernel is timed too; the fastest is kept, and two-step launches stay
- * on only if they beat the best single-step kernel. */
+ * on only if they beat the best single-step kernel.  The marching kernel (8 steps per launch) is timed beside them
+ * where it applies; if it wins, the default without a tile shape is kept. */
 lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best);
 lbem_status lbem_set_variant(lbem_t *h, int variant);
 lbem_status lbem_get_variant(const lbem_t *h, int *variant, int *nvariants);

@@ -99,6 +99,9 @@ lbem_status device_input(lbem_t *h, const float *p, size_t count, size_t off, co
     return LBEM_OK;
 }
 
+// Columns per bit of Events::mask.
+static int event_bucket(int nx) { return (nx + 63) / 64; }
+
 StepArgs step_args(const lbem_t *h, int cur_in) {
     StepArgs a;
     a.g = h->grid;
@@ -122,6 +125,8 @@ StepArgs step_args(const lbem_t *h, int cur_in) {
     }
     a.evt.rowptr = h->nev ? h->d_rowptr : nullptr;
     a.evt.ev = h->d_ev;
+    a.evt.mask = h->d_evmask;
+    a.evt.bucket = event_bucket(h->grid.nx);
     a.evt.amp = h->d_amp;
     a.evt.nt = h->nsrc ? h->nt : 0;
     a.evt.traces = h->d_traces;
@@ -137,6 +142,7 @@ static Walls handle_walls(const lbem_t *h) {
     w.fx = h->bc[0] ? h->d_fx : nullptr;
     w.fy = h->bc[1] ? h->d_fy : nullptr;
     w.fz = h->bc[2] ? h->d_fz : nullptr;
+    w.nlayer = h->layer;
     return w;
 }
 
@@ -196,6 +202,13 @@ static int two_step_shape(const lbem_t *h) {
     if (!h->tb_shape_set && big) return h->has_mu ? 2 : 7 + rs2_nshapes() + 1;
     return h->tblock == 2 && h->tb_shape < tb2_nshapes(h->storage, h->has_mu) ? h->tb_shape : 0;
 }
+// Whether calls of at least MARCH_MIN_STEPS steps run by the marching kernel (march.cu), 8 steps a launch: where two
+// steps per launch are the default and no shape was chosen.  Two steps take one two-step launch as before.
+constexpr int MARCH_MIN_STEPS = 3;
+static bool march_ok(const lbem_t *h) {
+    return h->tblock == 2 && !h->tb_shape_set && h->dim == 2 && h->storage == LBEM_F32 && !h->general() && !h->has_mu &&
+           !h->walls();
+}
 static int steps_per_launch(const lbem_t *h) { return three_step_ok(h) ? 3 : two_step_ok(h) ? 2 : 1; }
 
 // Enqueue nsteps steps starting from buffer `cur` at time t0: triples (pairs) of steps with the three-step
@@ -242,6 +255,15 @@ static cudaError_t enqueue_steps(const lbem_t *h, int cur, long long t0, int nst
             if (e != cudaSuccess) return e;
             cur ^= 1;
         }
+    }
+    if (march_ok(h) && nsteps >= MARCH_MIN_STEPS) {
+        StepArgs a = step_args(h, cur);
+        a.t = t0;
+        int launches = 0;
+        cudaError_t e = launch_march_2d(a, handle_walls(h), nsteps, h->stream, &launches);
+        if (e != cudaSuccess) return e;
+        n = nsteps;
+        cur ^= launches & 1;
     }
     if (two_step_ok(h)) {
         const int shape = two_step_shape(h);
@@ -314,6 +336,13 @@ static lbem_status rebuild_events(lbem_t *h) {
     gfree(h, h->d_ev);
     h->d_ev = nullptr;
     h->nev = (int)sorted.size();
+    if (h->nev) {
+        std::vector<unsigned long long> mask(h->grid.nrows, 0);
+        for (size_t i = 0; i < order.size(); i++) mask[rows[order[i]]] |= 1ull << (sorted[i].x / event_bucket(nx));
+        if (!h->d_evmask)
+            LBEM_CUDA(gmalloc(h, (void **)&h->d_evmask, sizeof(unsigned long long) * h->grid.nrows, "event columns"));
+        LBEM_CUDA(cudaMemcpy(h->d_evmask, mask.data(), sizeof(mask[0]) * mask.size(), cudaMemcpyHostToDevice));
+    }
     if (!h->d_rowptr) LBEM_CUDA(gmalloc(h, (void **)&h->d_rowptr, sizeof(int) * (h->grid.nrows + 1), "event rows"));
     LBEM_CUDA(cudaMemcpy(h->d_rowptr, rowptr.data(), sizeof(int) * rowptr.size(), cudaMemcpyHostToDevice));
     if (h->nev) {
@@ -457,7 +486,7 @@ void lbem_destroy(lbem_t *h) {
     drop_graph(h);
     adjoint_free(h);
     for (void *p : {(void *)h->pool, (void *)h->cL2, (void *)h->mu, (void *)h->dlnmu, (void *)h->d_rowptr,
-                    (void *)h->d_ev, (void *)h->d_amp, (void *)h->d_traces, (void *)h->d_partials,
+                    (void *)h->d_ev, (void *)h->d_evmask, (void *)h->d_amp, (void *)h->d_traces, (void *)h->d_partials,
                     (void *)h->d_diag, (void *)h->d_counter, (void *)h->d_stage, (void *)h->d_fx, (void *)h->d_fy,
                     (void *)h->d_fz,
                     (void *)h->d_wp2, (void *)h->d_wr2, (void *)h->d_gam, (void *)h->d_J, (void *)h->d_P,
@@ -1150,6 +1179,28 @@ lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best) {
             }
         }
     }
+    // the marching kernel, where calls of this handle would run by it if no shape were kept
+    bool march = false;
+    if (st == LBEM_OK && max_k == 2 && trial_steps >= MARCH_MIN_STEPS) {
+        const bool set = h->tb_shape_set;
+        h->tb_shape_set = false;
+        if (march_ok(h)) {
+            int n = 0;
+            for (int rep = 0; rep < 2 && st == LBEM_OK; rep++) {
+                StepArgs a = step_args(h, cur0);
+                a.evt.rowptr = nullptr;
+                cudaEventRecord(e0, h->stream);
+                cudaError_t e = launch_march_2d(a, handle_walls(h), trial_steps, h->stream, &n);
+                if (e != cudaSuccess) st = cuda_fail(e, "lbem_autotune");
+                cudaEventRecord(e1, h->stream);
+            }
+            cudaEventSynchronize(e1);
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            march = ms / trial_steps < best_per_step;
+        }
+        h->tb_shape_set = set;
+    }
     if (best_tblock == 1) best_shape = 0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1159,9 +1210,9 @@ lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best) {
     cudaFree(save);
     if (st != LBEM_OK) return st;
     h->variant = best_v;
-    h->tb_shape = best_shape;
-    h->tb_shape_set = true;
-    h->tblock = best_tblock;
+    h->tb_shape = march ? 0 : best_shape;
+    h->tb_shape_set = !march;
+    h->tblock = march ? 2 : best_tblock;
     drop_graph(h);
     if (best) *best = best_v;
     return LBEM_OK;

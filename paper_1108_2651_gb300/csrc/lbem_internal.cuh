@@ -325,6 +325,9 @@ struct Event {
 struct Events {
     const int *rowptr = nullptr;  // [nrows + 1] or null if no events
     const Event *ev = nullptr;
+    // per row a bit for every bucket of `bucket` columns that holds an event (null with rowptr)
+    const unsigned long long *mask = nullptr;
+    int bucket = 1;
     const float *amp = nullptr;   // [nsrc][nt]
     int nt = 0;
     float *traces = nullptr;      // [nrec][cap]
@@ -350,7 +353,7 @@ struct Medium {
     // (time t) and written to Pw (the plane of the output state's parity)
     const float *wp2 = nullptr, *wr2 = nullptr, *gam = nullptr, *Pr = nullptr;
     const float *pc = nullptr, *pb = nullptr, *pa = nullptr;
-    float *J = nullptr, *Pw = nullptr;
+    float *J = nullptr, *Pw = nullptr, *Jw = nullptr;
 };
 
 // Walls and absorbing layers (walls.cu): per axis x, y 0 = periodic, 1 = PEC wall, 2 = PMC wall; layer
@@ -358,6 +361,7 @@ struct Medium {
 struct Walls {
     int kind[3] = {0, 0, 0};
     const float *fx = nullptr, *fy = nullptr, *fz = nullptr;
+    int nlayer = 0;  // width of the layer
 };
 // What the general single-step kernel (general.cu) adds to a step: one Drude-Lorentz pole per site (parameters
 // and state as planes with the grid's pitch, J at t - 1/2 (in place), P at t read from P and written to Pn; wp2
@@ -376,7 +380,7 @@ struct EdgeTile {
     int x0, y0, w, h;
 };
 
-struct StepArgs {
+struct __align__(16) StepArgs {
     Grid g;
     PopBuf in, out;
     Medium med;
@@ -482,6 +486,7 @@ struct lbem {
     // events
     int *d_rowptr = nullptr;
     lbk::Event *d_ev = nullptr;
+    unsigned long long *d_evmask = nullptr;  // Events::mask
     float *d_amp = nullptr;
     float *d_traces = nullptr;
     int nsrc = 0, nrec = 0, nt = 0, cap = 0, nev = 0;
@@ -571,6 +576,9 @@ int tb2_nshapes(int storage, bool has_mu);
 // two steps per launch by register streaming (rstream.cu): FP32 storage, uniform mu
 int rs2_nshapes();
 cudaError_t launch_step_2d_rs2(const StepArgs &a, int shape, cudaStream_t s);
+// up to 8 steps per launch by marching strips down the rows (march.cu): enqueues the launches of nsteps steps from
+// a.in, alternating between the two buffers; *launches of them
+cudaError_t launch_march_2d(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches);
 int ss2_nshapes();  // strip streaming (sstream.cu): two steps per launch, FP32, uniform mu
 cudaError_t launch_step_2d_ss2(const StepArgs &a, int shape, cudaStream_t s);
 cudaError_t launch_step_2d_ss2_an(const StepArgs &a, cudaStream_t s);  // anisotropic medium, no pole

@@ -1,0 +1,62 @@
+"""The marching kernel (8 steps per launch, the default for calls of at least 3 steps) against single steps.
+
+Every site update is the single-step kernel's arithmetic in its order, so E, B and the receiver traces are
+bit-identical for every grid, step count and split of the steps into calls.  The grids lie at the kernel's edges: strips
+of up to 112 columns (4 * 28) with 8 columns of halo, rows whose last group of four is partial, segments of two rows,
+grids smaller than a halo.
+"""
+import numpy as np
+import pytest
+
+from paper_1108_2651_gb300 import lbem, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(shape, seed, nsteps):
+    eps, _ = W.random_medium(shape, seed)
+    p = W.Problem("march", 2, shape, eps, None, nsteps)
+    p.E0, p.B0 = W.random_fields(shape, seed + 1, 0.3)
+    ny, nx = shape
+    n = ny * nx
+    rng = np.random.default_rng(seed + 2)
+    corners = [0, nx - 1, (ny - 1) * nx, n - 1, (ny // 2) * nx + min(nx - 1, 112)]
+    p.src_site = np.unique(np.concatenate([corners, rng.integers(0, n, 3)])).astype(np.int64)
+    p.src_comp = np.full(p.src_site.size, 2, np.int32)
+    p.src_amp = rng.standard_normal((p.src_site.size, nsteps))
+    p.rec_site = np.concatenate([corners, rng.integers(0, n, 20)]).astype(np.int64)  # two may share a site
+    p.rec_comp = np.resize(np.array([2, 3, 4], np.int32), p.rec_site.size)
+    return p
+
+
+def _run(p, calls, steps_per_pass=None, graphs=False):
+    import torch
+
+    stream = torch.cuda.Stream() if graphs else None
+    s = lbem.Solver(p.shape, stream=stream.cuda_stream if stream else None)
+    s.set_problem(p)
+    if steps_per_pass:
+        lbem.lbem_set_temporal_blocking(s.h, steps_per_pass, -1)
+    if graphs:
+        lbem.lbem_set_graphs(s.h, True)
+    for n in calls:
+        s.step(n)
+    E, B = s.fields()
+    tr = s.traces(p.rec_site.size)
+    torch.cuda.synchronize()
+    lbem.lbem_sync(s.h)
+    lbem.lbem_check_guards(s.h)
+    s.close()
+    return E.cpu().numpy(), B.cpu().numpy(), tr.cpu().numpy()
+
+
+@pytest.mark.parametrize("shape", [(1, 1), (1, 300), (2, 3), (3, 112), (5, 113), (9, 116), (17, 224), (40, 225),
+                                   (300, 5), (64, 451), (131, 1000), (700, 337)])
+def test_march_is_bitwise_identical_to_single_steps(lbem, shape):
+    p = _problem(shape, 700 + shape[1], 43)
+    ref = _run(p, [43], steps_per_pass=1)
+    for calls in ([43], [8, 35], [16, 16, 11], [3, 4, 5, 6, 7, 9, 9], [1, 2, 40]):
+        for graphs in (False, True):
+            got = _run(p, calls, graphs=graphs)
+            for a, b in zip(got, ref):
+                np.testing.assert_array_equal(a, b, err_msg=f"{shape}, calls {calls}, graphs {graphs}")
