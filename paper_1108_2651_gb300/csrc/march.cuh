@@ -78,6 +78,19 @@ __device__ __forceinline__ float m_lds1(unsigned a) {
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
     return v;
 }
+__device__ __forceinline__ void m_sts1(unsigned a, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v));
+}
+__device__ __forceinline__ int2 m_lds_int2(unsigned a) {
+    int2 v;
+    asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ int4 m_lds_int4(unsigned a) {
+    int4 v;
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
 __device__ __forceinline__ uint2 m_lds8(unsigned a) {
     uint2 v;
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
@@ -111,8 +124,11 @@ struct MarchCfg {
     static constexpr int NM = MED == MARCH_MU ? 3 : MED == MARCH_POLE ? 4 : 1;  // medium planes
     static constexpr int RB = NM * 512, NR = K + D - 1 <= 8 ? 8 : 16;      // the ring of medium rows
     static_assert(K + D - 1 <= NR && K % 2 == 0, "ring of medium rows");
-    static constexpr int XB = ST == LBEM_F32 ? 0 : 2560;                   // event scratch (FP32: the stage just read)
-    static constexpr int O_RING = D * SB, O_G = O_RING + NR * RB, O_X = O_G + (K - 1) * 1024, smem = O_X + XB;
+    // then plane 2's slots, and the unit's sources and receivers: 32 records, the sources' currents of K steps, and
+    // 32 places for a lane's quads (five planes, a source's S^, the pole's P)
+    static constexpr int QB = MED == MARCH_POLE ? 112 : 96;
+    static constexpr int O_RING = D * SB, O_G = O_RING + NR * RB, O_EV = O_G + (K - 1) * 1024,
+                         O_AMP = O_EV + 512, O_Q = O_AMP + 128 * K, smem = O_Q + 32 * QB;
 };
 
 // The state's storage format <-> FP32 of 4 sites.
@@ -219,6 +235,13 @@ __device__ __forceinline__ void m_collide(float4 g0, float4 g1, float4 g2, float
     o.p4 = quad(o4a, o4b);
 }
 
+struct MarchTrue {
+    static constexpr bool value = true;
+};
+struct MarchFalse {
+    static constexpr bool value = false;
+};
+
 // The march of one unit by one warp: kp steps from a.t.
 template <int ST, int MED, bool WL, int K, int D>
 __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, int kp, int nstrips, int nseg, int strip,
@@ -249,9 +272,6 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
         const unsigned lo = __reduce_or_sync(FULL, (unsigned)smask), hi = __reduce_or_sync(FULL, (unsigned)(smask >> 32));
         smask = ((unsigned long long)hi << 32) | lo;
     }
-    // columns whose update a wall or a layer changes
-    const int edge_x = WL ? max(w.nlayer, 1) : 0;
-    const bool xslow = WL && w.kind[0] && (xs - H < edge_x || xs - H + 128 > G.nx - edge_x);
     const float sx = WL && w.kind[0] == 1 ? -1.f : 1.f, sy = WL && w.kind[1] == 1 ? -1.f : 1.f;
     const float r = MED == MARCH_AN ? a.med.ar : 1.f, ri = MED == MARCH_AN ? __fdiv_rn(1.f, r) : 1.f,
                 fs = MED == MARCH_AN ? __fadd_rn(r, ri) : 2.f;
@@ -343,41 +363,133 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
     for (int j = 0; j < K; j++) A0[j] = A1[j] = A3[j] = PP[j] = JJ[j] = z4;
     unsigned g2a = sl + Cfg::O_G - 1024, g2b = g2a + 512;  // level j's slots of plane 2 at + 1024 j
 
-    // Sources and receivers of row `row` at time tj: receivers written, the sources' part of S^ added to sh.  The
-    // lane's populations are read by column from `scr` (planes 512 bytes apart) and c_L^2 from `mr`.
-    auto events = [&](int row, long long tj, bool rec, unsigned scr, unsigned mr, float4 pz, float4 &sh) {
-        const int e0 = __ldg(a.evt.rowptr + row), e1 = __ldg(a.evt.rowptr + row + 1);
-#pragma unroll 1
-        for (int e = e0; e < e1; e++) {
-            const int4 ev = __ldg(reinterpret_cast<const int4 *>(a.evt.ev + e));  // x, kind, index, comp
-            int d = ev.x - xw;
-            if (d < 0) d += G.nx;
-#pragma unroll 1
-            for (; d < 4; d += G.nx) {
-                if (ev.y == 0) {
-                    if (ev.w == 2 && tj < a.evt.nt) {
-                        float jz = __ldg(a.evt.amp + (long long)ev.z * a.evt.nt + tj);
-                        if (MED == MARCH_MU) jz = __fmul_rn(jz, __ldg(a.med.mu + (long long)row * G.pitch + ev.x));
-                        if (MED == MARCH_AN) jz = __fmul_rn(jz, a.med.amu);
-                        set(sh, d, __fsub_rn(get(sh, d), jz));
+    // Sources and receivers.  A unit lists those of its rows and columns (of the receivers, those it owns) in shared
+    // memory, with the sources' currents of the launch's steps: looked up row by row in global memory they cost a row
+    // several dependent loads at each of its levels (1024^2 with 64 receivers: 5.7 us a step, 2.3 without any).  A record
+    // is {row (unwrapped), lane | column << 5 | receiver << 7 | place << 8, index, component}; lane l keeps the row of
+    // record l; records of one row and lane share a place for the lane's quads.  Units with more than 32 records, or
+    // two sources on a site (`many`), look them up in global memory after all, on rows whose mask has one of the strip's
+    // columns.
+    int erow = -(1 << 30);
+    bool many = false;
+    unsigned fb = 0;  // the flags of such rows: bit 0 that of level K - 1, bit K - 1 that of level 0, then those below
+    if (hasev) {
+        int ne = 0;
+        const unsigned rec = smem + Cfg::O_EV;
+        for (int base = y0 - (kp - 1); base < y1 + (kp - 1) && !many; base += 32) {
+            const int row = base + lane, rw = wrapi(row, G.ny);
+            const int e0 = __ldg(a.evt.rowptr + rw), e1 = __ldg(a.evt.rowptr + rw + 1);
+            const int n = row < y1 + (kp - 1) && (a.evt.mask[rw] & smask) ? e1 - e0 : 0;
+            if (__ballot_sync(FULL, n > 0) == 0) continue;
+            int sum = n;  // inclusive sums over the lanes (rows)
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(FULL, sum, o);
+                if (lane >= o) sum += v;
+            }
+            const int total = __shfl_sync(FULL, sum, 31);
+            for (int i = 0; i < total && !many; i += 32) {
+                // the lane's event: number i + lane of the block's, in the row whose sums it lies between
+                int q = 0;
+#pragma unroll
+                for (int o = 16; o; o >>= 1)
+                    if (__shfl_sync(FULL, sum, q + o - 1) <= i + lane) q += o;
+                const int e = __shfl_sync(FULL, e0, q & 31) + i + lane -
+                              (__shfl_sync(FULL, sum, q & 31) - __shfl_sync(FULL, n, q & 31));
+                const int yu = base + q;
+                int4 ev = make_int4(-1, 0, 0, 0);
+                if (i + lane < total) ev = __ldg(reinterpret_cast<const int4 *>(a.evt.ev + e));  // x, kind, index, comp
+                int dx0 = ev.x - wrapi(xs - H, G.nx);
+                dx0 += dx0 < 0 ? G.nx : 0;
+                for (int k = 0; k < 128; k += G.nx) {  // a narrow grid repeats its columns
+                    int dx = dx0 + k;
+                    bool keep = ev.x >= 0 && dx < 128;
+                    if (ev.y) {
+                        keep = k == 0 && ev.x >= xs && ev.x < xe && yu >= y0 && yu < y1;
+                        dx = ev.x - xs + H;
                     }
-                } else if (rec && X + d < xe && tj < a.evt.cap) {
-                    const float q0 = m_lds1(scr + 4 * d), q1 = m_lds1(scr + 512 + 4 * d),
-                                q2 = m_lds1(scr + 1024 + 4 * d), q3 = m_lds1(scr + 1536 + 4 * d),
-                                q4 = m_lds1(scr + 2048 + 4 * d), cl = m_lds1(mr + 4 * d);
-                    float v = field2d(ev.w, cl, ((q0 + q1) + (q2 + q3)) + q4, q4 - q2, q1 - q3);
-                    if (MED == MARCH_POLE && ev.w == 2) v = __fsub_rn(v, get(pz, d));
-                    if (MED == MARCH_AN && ev.w == 3) v = __fmul_rn(v, r);
-                    if (MED == MARCH_AN && ev.w == 4) v = __fmul_rn(v, ri);
-                    a.evt.traces[(long long)ev.z * a.evt.cap + tj] = v;
+                    const unsigned b = __ballot_sync(FULL, keep);
+                    const int at = ne + __popc(b & ((1u << lane) - 1));
+                    ne += __popc(b);
+                    many = ne > 32;
+                    if (keep && at < 32) {
+                        asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(rec + at * 16), "r"(yu),
+                                     "r"((dx >> 2) | (dx & 3) << 5 | (ev.y ? 128 : 0)), "r"(ev.z), "r"(ev.w));
+                        for (int k = 0; k < kp && ev.y == 0; k++) {
+                            float jz = 0.f;  // a component that does not couple, or past the series: no current
+                            if (ev.w == 2 && a.t + k < a.evt.nt)
+                                jz = __ldg(a.evt.amp + (long long)ev.z * a.evt.nt + a.t + k);
+                            if (MED == MARCH_MU)
+                                jz = __fmul_rn(jz, __ldg(a.med.mu + (long long)wrapi(yu, G.ny) * G.pitch + ev.x));
+                            if (MED == MARCH_AN) jz = __fmul_rn(jz, a.med.amu);
+                            m_sts1(smem + Cfg::O_AMP + (at * K + k) * 4, jz);
+                        }
+                    }
+                    if (many) break;
                 }
             }
         }
+        __syncwarp();
+        if (ne > 0 && !many) {
+            int2 v = make_int2(-1 - lane, 0);
+            if (lane < ne) v = m_lds_int2(rec + lane * 16);
+            const unsigned at = __match_any_sync(FULL, v.x * 32 + (v.y & 31));
+            const unsigned same = __match_any_sync(FULL, v.y & 127) & at & __ballot_sync(FULL, !(v.y & 128));
+            many = __any_sync(FULL, lane < ne && !(v.y & 128) && __popc(same) > 1);
+            if (lane < ne) {
+                erow = v.x;
+                m_sts1(rec + lane * 16 + 4, __int_as_float(v.y | (__ffs(at) - 1) << 8));
+                m_sts(smem + Cfg::O_Q + lane * Cfg::QB + 80, z4);
+            }
+            __syncwarp();
+        }
+    }
+    // An event at column x: the current jz of a source, taken from sh, or a receiver of one of the lane's sites.
+    auto event = [&](int x, bool rcv, int index, int comp, float jz, long long tj, const float4 &g0, const float4 &g1,
+                     const float4 &g2, const float4 &g3, const float4 &g4, const float4 &c, const float4 &pz, float4 &sh) {
+        int d = x - xw;
+        d += d < 0 ? G.nx : 0;
+#pragma unroll 1
+        for (; d < 4; d += G.nx) {
+            if (!rcv) {
+                set(sh, d, __fsub_rn(get(sh, d), jz));
+            } else if (owned && X + d < xe && tj < a.evt.cap) {
+                const float q0 = get(g0, d), q1 = get(g1, d), q2 = get(g2, d), q3 = get(g3, d), q4 = get(g4, d);
+                float v = field2d(comp, get(c, d), ((q0 + q1) + (q2 + q3)) + q4, q4 - q2, q1 - q3);
+                if (MED == MARCH_POLE && comp == 2) v = __fsub_rn(v, get(pz, d));
+                if (MED == MARCH_AN && comp == 3) v = __fmul_rn(v, r);
+                if (MED == MARCH_AN && comp == 4) v = __fmul_rn(v, ri);
+                a.evt.traces[(long long)index * a.evt.cap + tj] = v;
+            }
+        }
+    };
+    // The events of unwrapped row yu at level j by the row's list in global memory; whether a source is among them.
+    auto events = [&](int yu, int j, const float4 &g0, const float4 &g1, const float4 &g2, const float4 &g3,
+                      const float4 &g4, const float4 &c, const float4 &pz, float4 &sh) {
+        const long long tj = a.t + j;
+        bool src = false;
+        if (!((fb >> (K - 1 - j)) & 1)) return false;
+        const int row = wrapi(yu, G.ny);
+        const int e0 = __ldg(a.evt.rowptr + row), e1 = __ldg(a.evt.rowptr + row + 1);
+#pragma unroll 1
+        for (int e = e0; e < e1; e++) {
+            const int4 ev = __ldg(reinterpret_cast<const int4 *>(a.evt.ev + e));
+            float jz = 0.f;
+            if (ev.y == 0) {
+                if (ev.w != 2 || tj >= a.evt.nt) continue;
+                jz = __ldg(a.evt.amp + (long long)ev.z * a.evt.nt + tj);
+                if (MED == MARCH_MU) jz = __fmul_rn(jz, __ldg(a.med.mu + (long long)row * G.pitch + ev.x));
+                if (MED == MARCH_AN) jz = __fmul_rn(jz, a.med.amu);
+                src = true;
+            } else if (yu < y0 || yu >= y1) {
+                continue;
+            }
+            event(ev.x, ev.y != 0, ev.z, ev.w, jz, tj, g0, g1, g2, g3, g4, c, pz, sh);
+        }
+        return src;
     };
 
-    // Event flags of the rows: bit 0 that of level K - 1, bit K - 1 that of level 0, then those below.  yl: the row
-    // of level 0 (unwrapped), st: its stage, rs: its place in the medium ring.
-    unsigned fb = 0;
+    // yl: the row of level 0 (unwrapped), st: its stage, rs: its place in the medium ring.
     int yl = y0 - (kp - 1), st = 0, rs = 0;
     auto ring = [&](int j) {
         return sl + Cfg::O_RING + ((rs - j) & (NR - 1)) * RB;
@@ -447,148 +559,201 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
         pole_update(c.z, sig.z, pc.z, pb.z, pa.z, J.z, P.z);
         pole_update(c.w, sig.w, pc.w, pb.w, pa.w, J.w, P.w);
     };
-    // A row with every level busy and no event or wall, FP32 storage.
-    auto row_plain = [&]() {
+    // With walls (WL): the pulls across them, at row yu, given the lane's unshifted planes 1 and 3 and the plane 2
+    // computed by the previous iteration (row ny - 1's own), and the absorbing layer.
+    auto wall_pulls = [&](int yu, const float4 &h1, const float4 &h3, float4 &g1, float4 &h2, float4 &g3, float4 &h4,
+                          bool lev, unsigned prev2) {
+        if (w.kind[0]) {
+            if (X == 0) g1.x = sx * h3.x;
+            const int k = G.nx - 1 - X;
+            if ((unsigned)k < 4u) set(g3, k, sx * get(h1, k));
+        }
+        if (w.kind[1]) {  // the plane-2 value kept for row 0 is plane 4 of the row itself (see below)
+            if (yu == 0) h2 = make_float4(sy * h2.x, sy * h2.y, sy * h2.z, sy * h2.w);
+            if (yu == G.ny - 1) {
+                if (lev) h4 = m_lds(prev2);
+                h4 = make_float4(sy * h4.x, sy * h4.y, sy * h4.z, sy * h4.w);
+            }
+        }
+    };
+    float4 fx = make_float4(1.f, 1.f, 1.f, 1.f);  // the columns' factors (the table is padded with 1 to the pitch)
+    if (WL && w.fx && X >= 0 && X < G.nx) fx = __ldg(reinterpret_cast<const float4 *>(w.fx + X));
+    auto layer = [&](int yu, Quad5 &n) {
+        const float fy = w.fy && (unsigned)yu < (unsigned)G.ny ? __ldg(w.fy + yu) : 1.f;
+        const float4 f = make_float4(__fmul_rn(fx.x, fy), __fmul_rn(fx.y, fy), __fmul_rn(fx.z, fy), __fmul_rn(fx.w, fy));
+        float4 *v[5] = {&n.p0, &n.p1, &n.p2, &n.p3, &n.p4};
+#pragma unroll
+        for (int p = 0; p < 5; p++)
+            *v[p] = make_float4(__fmul_rn(v[p]->x, f.x), __fmul_rn(v[p]->y, f.y), __fmul_rn(v[p]->z, f.z),
+                                __fmul_rn(v[p]->w, f.w));
+    };
+    // The terms of a source S^ at the lane's sites, added last as collide2d adds them.
+    auto source = [&](const float4 &c, const float4 &S4, Quad5 &n) {
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const float cl = get(c, k), S = get(S4, k);
+            const float w0 = MED == MARCH_AN ? __fsub_rn(1.f, __fmul_rn(fs, cl)) : __fsub_rn(1.f, 2.f * cl);
+            const float Tm = __fmul_rn(-0.5f * cl, S), T0 = __fmul_rn(-w0, S);
+            const float Tx = MED == MARCH_AN ? __fmul_rn(r, Tm) : Tm;
+            const float Ty = MED == MARCH_AN ? __fmul_rn(ri, Tm) : Tm;
+            set(n.p0, k, __fadd_rn(get(n.p0, k), T0));
+            set(n.p1, k, __fadd_rn(get(n.p1, k), Tx));
+            set(n.p2, k, __fadd_rn(get(n.p2, k), Ty));
+            set(n.p3, k, __fadd_rn(get(n.p3, k), Tx));
+            set(n.p4, k, __fadd_rn(get(n.p4, k), Ty));
+        }
+    };
+    // One row, every level one row further.  EV: a row with events or of a launch of fewer than K steps; its straight
+    // line only hands the quads of the lanes concerned to their places in shared memory and adds the sources' terms
+    // (S^ = 0 adds -0 and changes nothing), and the records are gone through once, before and after: with their code at
+    // every level the row was 20 KB that the instruction cache did not hold, 3 us a row against 0.5 us of a plain one.
+    auto row = [&](auto evc) {
+        constexpr bool EV = decltype(evc)::value;
         const unsigned s = smem + st * SB + lane * (PS / 32);
         float4 g0, a1, g2, a3, g4, P = z4, J = z4;
         stage(s, g0, a1, g2, a3, g4, P, J);
         issue();
+        unsigned levels = 0, recs = 0;  // EV: the levels to leave the line at, the records of the row's levels
+        unsigned long long place = 0;   // the lane's place per level (6 bits, 32: none)
+        if (EV) {
+            if (kp < K) levels = 1u << (kp - 1);
+            recs = __ballot_sync(FULL, (unsigned)(yl - erow) < (unsigned)K);
+#pragma unroll 1
+            for (unsigned b = recs; b; b &= b - 1) {
+                const int l = __ffs(b) - 1;
+                const int2 v = m_lds_int2(smem + Cfg::O_EV + l * 16);
+                const int j = yl - v.x;
+                levels |= 1u << j;
+                if ((v.y & 31) == lane) {
+                    const unsigned q = (unsigned)v.y >> 8;
+                    place |= (unsigned long long)(32 | q) << (6 * j);
+                    if (!(v.y & 128))
+                        m_sts1(smem + Cfg::O_Q + q * Cfg::QB + 80 + ((v.y >> 5) & 3) * 4,
+                               __fsub_rn(0.f, m_lds1(smem + Cfg::O_AMP + (l * K + j) * 4)));
+                }
+            }
+        }
         Quad5 o;
-        float4 Po = z4, Jo = z4;
+        float4 Po = z4, Jo = z4;  // the pole's state after the previous level
 #pragma unroll
         for (int j = 0; j < K; j++) {
             Quad5 n;
             const unsigned mr = ring(j);
             const float4 c = m_lds(mr);
-            const float4 h0 = j ? A0[j] : g0, h1 = j ? A1[j] : a1, h2 = j ? m_lds(g2a + 1024 * j) : g2,
-                         h3 = j ? A3[j] : a3, h4 = j ? o.p4 : g4;
-            const float4 g1 = make_float4(__shfl_up_sync(FULL, h1.w, 1), h1.x, h1.y, h1.z);
-            const float4 g3 = make_float4(h3.y, h3.z, h3.w, __shfl_down_sync(FULL, h3.x, 1));
-            float4 sh = z4, sig, Pn = j ? PP[j] : P, Jn = j ? JJ[j] : J;
+            const float4 h0 = j ? A0[j] : g0, h1 = j ? A1[j] : a1, h3 = j ? A3[j] : a3;
+            float4 h2 = j ? m_lds(g2a + 1024 * j) : g2, h4 = j ? o.p4 : g4;
+            float4 g1 = make_float4(__shfl_up_sync(FULL, h1.w, 1), h1.x, h1.y, h1.z);
+            float4 g3 = make_float4(h3.y, h3.z, h3.w, __shfl_down_sync(FULL, h3.x, 1));
+            if (WL) wall_pulls(yl - j, h1, h3, g1, h2, g3, h4, j > 0, g2b + 1024 * j);
+            float4 sh = z4, S = z4, sig, Pn = j ? PP[j] : P, Jn = j ? JJ[j] : J;
+            const bool leave = EV && ((levels >> j) & 1);
             if (MED == MARCH_MU) sh = mu_src(mr, g1, h2, g3, h4);
+            if (EV && leave) {
+                const unsigned v = (unsigned)(place >> (6 * j)) & 63;
+                if (v) {
+                    const unsigned q = smem + Cfg::O_Q + (v & 31) * Cfg::QB;
+                    m_sts(q, h0);
+                    m_sts(q + 16, g1);
+                    m_sts(q + 32, h2);
+                    m_sts(q + 48, g3);
+                    m_sts(q + 64, h4);
+                    S = m_lds(q + 80);
+                    if (MED == MARCH_POLE) m_sts(q + 96, Pn);
+                }
+                if (MED == MARCH_MU)
+                    sh = make_float4(__fadd_rn(sh.x, S.x), __fadd_rn(sh.y, S.y), __fadd_rn(sh.z, S.z), __fadd_rn(sh.w, S.w));
+            }
             m_collide<MED>(h0, g1, h2, g3, h4, c, Pn, sh, r, ri, fs, n, sig);
+            if (EV && MED != MARCH_MU && leave) source(c, S, n);
             if (MED == MARCH_POLE) pole(mr, c, sig, Jn, Pn);
-            if (j) {
-                A0[j] = o.p0;
-                A1[j] = o.p1;
-                A3[j] = o.p3;
-                m_sts(g2a + 1024 * j, o.p2);
-                PP[j] = Po;
-                JJ[j] = Jo;
-            }
-            o = n;
-            Po = Pn;
-            Jo = Jn;
-        }
-        store(yl - (K - 1), o, Po, Jo);
-    };
-    // Any row: with events, walls, levels that have not started, fewer than K levels, rounded storage.
-    auto row_full = [&](int it) {
-        const unsigned s = smem + st * SB + lane * (PS / 32);
-        float4 g0, a1, g2, a3, g4, P = z4, J = z4;
-        stage(s, g0, a1, g2, a3, g4, P, J);
-        issue();
-        const unsigned scr = F32 ? s : sl + Cfg::O_X;  // the lane's event scratch
-        const int nact = min(kp, it / 2 + 1);          // levels with a row to compute
-        Quad5 o;
-        float4 Po = z4, Jo = z4;  // the pole's state after the previous level
-#pragma unroll
-        for (int j = 0; j < K; j++) {
-            if (j > nact) break;
-            Quad5 n;
-            float4 Pn = z4, Jn = z4;
-            const bool act = j < nact;
-            const int yu = yl - j;  // unwrapped
-            if (act) {
-                const unsigned mr = ring(j);
-                const float4 c = m_lds(mr);
-                const float4 h0 = j ? A0[j] : g0, h1 = j ? A1[j] : a1, h3 = j ? A3[j] : a3;
-                float4 h2 = j ? m_lds(g2a + 1024 * j) : g2, h4 = j ? o.p4 : g4;
-                Pn = j ? PP[j] : P;
-                Jn = j ? JJ[j] : J;
-                float4 g1 = make_float4(__shfl_up_sync(FULL, h1.w, 1), h1.x, h1.y, h1.z);
-                float4 g3 = make_float4(h3.y, h3.z, h3.w, __shfl_down_sync(FULL, h3.x, 1));
-                if (WL) {  // pulls across walls
-                    if (w.kind[0]) {
-                        if (X == 0) g1.x = sx * h3.x;
-                        const int k = G.nx - 1 - X;
-                        if ((unsigned)k < 4u) set(g3, k, sx * get(h1, k));
-                    }
-                    if (w.kind[1]) {
-                        // the plane-2 value kept for row 0 is plane 4 of the row itself (see below); for row
-                        // ny - 1, plane 2 of the row is the one computed by the previous iteration
-                        if (yu == 0) h2 = make_float4(sy * h2.x, sy * h2.y, sy * h2.z, sy * h2.w);
-                        if (yu == G.ny - 1) {
-                            if (j) h4 = m_lds(g2b + 1024 * j);
-                            h4 = make_float4(sy * h4.x, sy * h4.y, sy * h4.z, sy * h4.w);
-                        }
-                    }
-                }
-                float4 sh = z4;
-                if (MED == MARCH_MU) sh = mu_src(mr, g1, h2, g3, h4);
-                bool src = false;
-                if ((fb >> (K - 1 - j)) & 1) {
-                    m_sts(scr, h0);
-                    m_sts(scr + 512, g1);
-                    m_sts(scr + 1024, h2);
-                    m_sts(scr + 1536, g3);
-                    m_sts(scr + 2048, h4);
-                    events(wrapi(yu, G.ny), a.t + j, owned && yu >= y0 && yu < y1, scr, mr, Pn, sh);
-                    src = true;
-                }
-                float4 sig;
-                m_collide<MED>(h0, g1, h2, g3, h4, c, Pn, sh, r, ri, fs, n, sig);
-                if (MED == MARCH_POLE) pole(mr, c, sig, Jn, Pn);
-                if (MED != MARCH_MU && src) {  // the sources' terms, added last as collide2d adds them
-#pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        const float cl = get(c, k), S = get(sh, k);
-                        const float w0 = MED == MARCH_AN ? __fsub_rn(1.f, __fmul_rn(fs, cl))
-                                                         : __fsub_rn(1.f, 2.f * cl);
-                        const float Tm = __fmul_rn(-0.5f * cl, S), T0 = __fmul_rn(-w0, S);
-                        const float Tx = MED == MARCH_AN ? __fmul_rn(r, Tm) : Tm;
-                        const float Ty = MED == MARCH_AN ? __fmul_rn(ri, Tm) : Tm;
-                        set(n.p0, k, __fadd_rn(get(n.p0, k), T0));
-                        set(n.p1, k, __fadd_rn(get(n.p1, k), Tx));
-                        set(n.p2, k, __fadd_rn(get(n.p2, k), Ty));
-                        set(n.p3, k, __fadd_rn(get(n.p3, k), Tx));
-                        set(n.p4, k, __fadd_rn(get(n.p4, k), Ty));
-                    }
-                }
-                if (WL && (w.fx || w.fy)) {  // the absorbing layer
-                    const float fy = w.fy && (unsigned)yu < (unsigned)G.ny ? __ldg(w.fy + yu) : 1.f;
-                    float4 f = make_float4(fy, fy, fy, fy);
-                    if (w.fx && X >= 0 && X < G.nx) {  // the table is padded with 1 to the pitch
-                        const float4 fx = __ldg(reinterpret_cast<const float4 *>(w.fx + X));
-                        f = make_float4(__fmul_rn(fx.x, fy), __fmul_rn(fx.y, fy), __fmul_rn(fx.z, fy),
-                                        __fmul_rn(fx.w, fy));
-                    }
-                    float4 *v[5] = {&n.p0, &n.p1, &n.p2, &n.p3, &n.p4};
-#pragma unroll
-                    for (int p = 0; p < 5; p++)
-                        *v[p] = make_float4(__fmul_rn(v[p]->x, f.x), __fmul_rn(v[p]->y, f.y),
-                                            __fmul_rn(v[p]->z, f.z), __fmul_rn(v[p]->w, f.w));
-                }
-                // 16-bit storage: the state is rounded after every second step (K is even)
-                if (ST != LBEM_F32 && (j & 1) && j != K - 1) m_round<ST>(a.in, n);
-            }
+            if (WL) layer(yl - j, n);
+            // 16-bit storage: the state is rounded after every second step (and as it is stored)
+            if (ST != LBEM_F32 && (j & 1) && j != K - 1) m_round<ST>(a.in, n);
             if (j) {  // level j - 1's results become level j's inputs
                 A0[j] = o.p0;
                 A1[j] = o.p1;
                 A3[j] = o.p3;
                 m_sts(g2a + 1024 * j, o.p2);
                 // level j - 1 has just computed row 0: its plane 4 is what level j pulls back from the wall
-                if (WL && w.kind[1] && yu == -1) m_sts(g2b + 1024 * j, o.p4);
+                if (WL && w.kind[1] && yl - j == -1) m_sts(g2b + 1024 * j, o.p4);
                 PP[j] = Po;
                 JJ[j] = Jo;
             }
-            if (act) {
-                o = n;
-                Po = Pn;
-                Jo = Jn;
+            if (EV && leave && j < K - 1 && j == kp - 1) store(yl - j, n, Pn, Jn);
+            o = n;
+            Po = Pn;
+            Jo = Jn;
+        }
+        if (!EV || kp == K) store(yl - (K - 1), o, Po, Jo);
+        if (EV) {  // the receivers
+#pragma unroll 1
+            for (unsigned b = recs; b; b &= b - 1) {
+                const int l = __ffs(b) - 1;
+                const int4 v = m_lds_int4(smem + Cfg::O_EV + l * 16);
+                const long long tj = a.t + (yl - v.x);
+                if (!(v.y & 128) || (v.y & 31) != lane || tj >= a.evt.cap || yl - v.x >= kp) continue;
+                const unsigned q = smem + Cfg::O_Q + ((unsigned)v.y >> 8) * Cfg::QB + ((v.y >> 5) & 3) * 4;
+                const float q0 = m_lds1(q), q1 = m_lds1(q + 16), q2 = m_lds1(q + 32), q3 = m_lds1(q + 48),
+                            q4 = m_lds1(q + 64), cl = m_lds1(ring(yl - v.x) + ((v.y >> 5) & 3) * 4);
+                float f = field2d(v.w, cl, ((q0 + q1) + (q2 + q3)) + q4, q4 - q2, q1 - q3);
+                if (MED == MARCH_POLE && v.w == 2) f = __fsub_rn(f, m_lds1(q + 96));
+                if (MED == MARCH_AN && v.w == 3) f = __fmul_rn(f, r);
+                if (MED == MARCH_AN && v.w == 4) f = __fmul_rn(f, ri);
+                a.evt.traces[(long long)v.z * a.evt.cap + tj] = f;
             }
         }
-        store(yl - (kp - 1), o, Po, Jo);  // (all kp levels are busy by then)
+    };
+    // A row of a unit with many events: one level at a time, the levels' registers moving up by one at each, so that the
+    // code is a tenth of the unrolled row's.
+    auto row_many = [&]() {
+        const unsigned s = smem + st * SB + lane * (PS / 32);
+        float4 h0, h1, h2, h3, h4, Pn = z4, Jn = z4;
+        stage(s, h0, h1, h2, h3, h4, Pn, Jn);
+        issue();
+#pragma unroll 1
+        for (int j = 0; j < K; j++) {
+            Quad5 n;
+            const unsigned mr = ring(j), slot = 1024 * (j + 1);
+            const float4 c = m_lds(mr);
+            float4 g1 = make_float4(__shfl_up_sync(FULL, h1.w, 1), h1.x, h1.y, h1.z);
+            float4 g3 = make_float4(h3.y, h3.z, h3.w, __shfl_down_sync(FULL, h3.x, 1));
+            if (WL) wall_pulls(yl - j, h1, h3, g1, h2, g3, h4, j > 0, g2b + 1024 * j);
+            float4 sh = z4, sig;
+            bool src = false;
+            if (MED == MARCH_MU) sh = mu_src(mr, g1, h2, g3, h4);
+            src = events(yl - j, j, h0, g1, h2, g3, h4, c, Pn, sh);
+            m_collide<MED>(h0, g1, h2, g3, h4, c, Pn, sh, r, ri, fs, n, sig);
+            if (MED != MARCH_MU && src) source(c, sh, n);
+            if (MED == MARCH_POLE) pole(mr, c, sig, Jn, Pn);
+            if (WL) layer(yl - j, n);
+            if (ST != LBEM_F32 && (j & 1) && j != kp - 1) m_round<ST>(a.in, n);
+            if (j == kp - 1) store(yl - j, n, Pn, Jn);
+            if (j == K - 1) break;
+            // the next level's inputs, and this level's results in their place at the end of the row of registers
+            h0 = A0[1];
+            h1 = A1[1];
+            h3 = A3[1];
+            h4 = n.p4;
+            h2 = m_lds(g2a + slot);
+            m_sts(g2a + slot, n.p2);
+            if (WL && w.kind[1] && yl - j == 0) m_sts(g2b + slot, n.p4);
+            const float4 Pt = PP[1], Jt = JJ[1];
+#pragma unroll
+            for (int k = 1; k < K - 1; k++) {
+                A0[k] = A0[k + 1];
+                A1[k] = A1[k + 1];
+                A3[k] = A3[k + 1];
+                PP[k] = PP[k + 1];
+                JJ[k] = JJ[k + 1];
+            }
+            A0[K - 1] = n.p0;
+            A1[K - 1] = n.p1;
+            A3[K - 1] = n.p3;
+            PP[K - 1] = Pn;
+            JJ[K - 1] = Jn;
+            Pn = Pt;
+            Jn = Jt;
+        }
     };
     auto next_row = [&]() {
         const unsigned tmp = g2a;
@@ -598,36 +763,34 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
         st = st == D - 1 ? 0 : st + 1;
         rs = (rs + 1) & (NR - 1);
     };
-    // Rows by twos (an odd last one computes a row that nothing keeps): unrolled, so that half of the registers'
-    // moves go away, where both are plain; the other copy is out of the loop's way.
+    // Rows by twos (an odd last one computes a row that nothing keeps), so that half of the registers' moves go away.
 #pragma unroll 1
     for (int it = 0; it < nit; it += 2) {
-        if (hasev && (it & 15) == 0)  // the flags of the next 16 rows
-            fb |= (__ballot_sync(FULL, (a.evt.mask[wrapi(yl + (lane & 15), G.ny)] & smask) != 0) & 0xffffu)
-                  << (K - 1);
-        bool full = !F32 || kp < K || (fb & ((2u << K) - 1)) != 0;
-        if (WL) {
-            const int edge_y = max(w.nlayer, 1);
-            full |= xslow || (w.kind[1] && (yl - (K - 1) < edge_y || yl + 1 >= G.ny - edge_y));
-        }
-        if (__builtin_expect(!full, 1)) {
-#pragma unroll
-            for (int u = 0; u < 2; u++) {
-                asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
-                row_plain();
-                next_row();
-            }
-        } else {
+        if (many && (it & 15) == 0)  // the flags of the next 16 rows
+            fb |= (__ballot_sync(FULL, (a.evt.mask[wrapi(yl + (lane & 15), G.ny)] & smask) != 0) & 0xffffu) << (K - 1);
+        if (many) {
 #pragma unroll 1
             for (int u = 0; u < 2; u++) {
                 asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
-                row_full(it + u);
+                row_many();
                 next_row();
                 fb >>= 1;
             }
-            continue;
+        } else if (kp < K || (hasev && __any_sync(FULL, (unsigned)(yl + 1 - erow) <= (unsigned)K))) {
+#pragma unroll 1
+            for (int u = 0; u < 2; u++) {
+                asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
+                row(MarchTrue());
+                next_row();
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
+                row(MarchFalse());
+                next_row();
+            }
         }
-        fb >>= 2;
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
