@@ -169,7 +169,7 @@ lbem_status lbem_set_receivers(lbem_t *h, int n, const long long *site, const in
  * receivers sample the pre-collision fields.  One fused kernel launch per step,
  * or per two (three) steps where lbem_set_temporal_blocking enables it (two is
  * the default for 2D), or, for a call of at least 3 steps of a 2D grid that keeps
- * that default with no tile shape chosen, per 8 steps (see there), enqueued on the
+ * that default with no tile shape chosen, per 4 to 8 steps (see there), enqueued on the
  * stream (or replayed from a cached CUDA graph when enabled by lbem_set_graphs).
  * Requires a medium.  nsteps >= 0. */
 lbem_status lbem_step(lbem_t *h, int nsteps);
@@ -218,8 +218,8 @@ lbem_status lbem_get_boundaries(const lbem_t *h, int kind[3], int *layer, double
  * handle with walls or a mu array steps one step per launch with the general kernel (walls, layers and an
  * anisotropic medium included); without them it steps in pairs (lbem_set_temporal_blocking), bit-identical to
  * single steps.  The update J <- ((1 - gamma/2) J - wr2 P + wp2 E) / (1 + gamma/2) runs with three per-site
- * coefficients formed once here in FP64 (no division per step).  The handle holds a second P plane (every launch
- * writes P to the plane paired with its output
+ * coefficients formed once here in FP64 (no division per step).  The handle holds second J and P planes (every launch
+ * writes J and P to the planes paired with its output
  * population buffer); lbem_set_fields starts the pole at rest (D = E); lbem_save_state
  * appends J and P (lbem_info's state_bytes counts them).  Batches and the
  * adjoint take non-dispersive handles only.  Synchronises the stream. */
@@ -258,10 +258,13 @@ lbem_status lbem_set_watchdog(lbem_t *h, int every, double max_growth);
  * sites), walls and layers included; a dispersive pole without walls or a mu array with shape 0 at 4 per SM;
  * both bit-identical to their single steps.  With a pole and walls (or a pole with a mu array), and for
  * steps_per_pass = 3, every step of these media is a single step.
- * With steps_per_pass = 2 and tile_shape = -1 (the default), a call of lbem_step of at least 3 steps on an FP32 grid
- * of uniform mu without walls, a pole or a tensor runs 8 steps per launch by the marching kernel instead: a warp walks
- * a strip of columns down its rows with 8 time levels in flight (the last launch of a call takes the steps left), the
- * same bits again.  A tile shape >= 0 gives launches of two steps.
+ * With steps_per_pass = 2 and tile_shape = -1 (the default), a call of lbem_step of at least 3 steps runs several steps
+ * per launch by the marching kernel instead, wherever launches of two steps apply but for a pole in an anisotropic
+ * medium: a warp walks a strip of columns down its rows with 8 time levels in flight (6 with a heterogeneous mu or a
+ * pole, 4 with LBEM_I16B; the last launch of a call takes the steps left; walls and layers are applied on the way, with
+ * no pass after it).  The results are the same bits again: those of single steps for FP32 storage, of launches of two
+ * steps for 16-bit storage, whose state is rounded after every second step.  A tile shape >= 0 gives launches of two
+ * steps.
  * LBEM_ERR_ARG for values outside the current handle's set. */
 lbem_status lbem_set_temporal_blocking(lbem_t *h, int steps_per_pass, int tile_shape);
 

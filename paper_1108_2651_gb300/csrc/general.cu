@@ -42,9 +42,9 @@
 // the +-x pulls by warp shuffle (pull2d); pulls across a wall are then replaced
 // by the wall rule of walls.cu.  Per site: the B x grad ln mu source, sources
 // and receivers, the pole, the collision, the absorbing layer's factor.  The
-// pole's arrays are planes like c_L^2; J is read and written at the site only
-// (in place), P is read from the plane of the input's parity and written to
-// the other (a two-step launch reads P at sites of neighbouring tiles).
+// pole's arrays are planes like c_L^2; J and P are read from the planes of the
+// input's parity and written to the others (launches of several steps read them
+// at sites of neighbouring tiles or strips).
 #include <algorithm>
 
 #include "lbem_internal.cuh"
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(BLOCK, 4) step2d_gen(StepArgs a, Walls w, Gene
             set(Jn4, j, J);
             set(Pn4, j, P);
         }
-        *reinterpret_cast<float4 *>(q.J + o4) = Jn4;
+        *reinterpret_cast<float4 *>(q.Jn + o4) = Jn4;
         *reinterpret_cast<float4 *>(q.Pn + o4) = Pn4;
     }
     const float4 one4 = make_float4(1.f, 1.f, 1.f, 1.f);

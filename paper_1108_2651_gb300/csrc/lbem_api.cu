@@ -119,7 +119,8 @@ StepArgs step_args(const lbem_t *h, int cur_in) {
         a.med.pc = h->d_pc;
         a.med.pb = h->d_pb;
         a.med.pa = h->d_pa;
-        a.med.J = h->d_J;
+        a.med.J = h->pole_J(cur_in);
+        a.med.Jw = h->pole_J(cur_in ^ 1);
         a.med.Pr = h->pole_P(cur_in);
         a.med.Pw = h->pole_P(cur_in ^ 1);
     }
@@ -156,7 +157,8 @@ static cudaError_t launch_step(const lbem_t *h, const StepArgs &a, int variant) 
             q.pc = h->d_pc;
             q.pb = h->d_pb;
             q.pa = h->d_pa;
-            q.J = h->d_J;
+            q.J = a.med.J;
+            q.Jn = a.med.Jw;
             q.P = a.med.Pr;
             q.Pn = a.med.Pw;
         }
@@ -202,12 +204,12 @@ static int two_step_shape(const lbem_t *h) {
     if (!h->tb_shape_set && big) return h->has_mu ? 2 : 7 + rs2_nshapes() + 1;
     return h->tblock == 2 && h->tb_shape < tb2_nshapes(h->storage, h->has_mu) ? h->tb_shape : 0;
 }
-// Whether calls of at least MARCH_MIN_STEPS steps run by the marching kernel (march.cu), 8 steps a launch: where two
-// steps per launch are the default and no shape was chosen.  Two steps take one two-step launch as before.
+// Whether calls of at least MARCH_MIN_STEPS steps run by the marching kernel (march.cu), up to 8 steps a launch: where
+// two steps per launch are the default and no shape was chosen (but for a pole in an anisotropic medium).  Two steps
+// take one two-step launch as before.
 constexpr int MARCH_MIN_STEPS = 3;
 static bool march_ok(const lbem_t *h) {
-    return h->tblock == 2 && !h->tb_shape_set && h->dim == 2 && h->storage == LBEM_F32 && !h->general() && !h->has_mu &&
-           !h->walls();
+    return h->tblock == 2 && !h->tb_shape_set && multi_step_base(h) && !(h->disp && h->aniso);
 }
 static int steps_per_launch(const lbem_t *h) { return three_step_ok(h) ? 3 : two_step_ok(h) ? 2 : 1; }
 
@@ -260,7 +262,8 @@ static cudaError_t enqueue_steps(const lbem_t *h, int cur, long long t0, int nst
         StepArgs a = step_args(h, cur);
         a.t = t0;
         int launches = 0;
-        cudaError_t e = launch_march_2d(a, handle_walls(h), nsteps, h->stream, &launches);
+        cudaError_t e = launch_march_2d(a, handle_walls(h), h->storage, h->aniso, nsteps, h->stream,
+                                        &launches);
         if (e != cudaSuccess) return e;
         n = nsteps;
         cur ^= launches & 1;
@@ -489,7 +492,7 @@ void lbem_destroy(lbem_t *h) {
                     (void *)h->d_ev, (void *)h->d_evmask, (void *)h->d_amp, (void *)h->d_traces, (void *)h->d_partials,
                     (void *)h->d_diag, (void *)h->d_counter, (void *)h->d_stage, (void *)h->d_fx, (void *)h->d_fy,
                     (void *)h->d_fz,
-                    (void *)h->d_wp2, (void *)h->d_wr2, (void *)h->d_gam, (void *)h->d_J, (void *)h->d_P,
+                    (void *)h->d_wp2, (void *)h->d_wr2, (void *)h->d_gam, (void *)h->d_J, (void *)h->d_J2, (void *)h->d_P,
                     (void *)h->d_P2, (void *)h->d_pc, (void *)h->d_pb, (void *)h->d_pa})
         gfree(h, p);
     for (int k = 1; k <= 3; k++) gfree(h, h->d_tiles[k]);
@@ -633,7 +636,7 @@ lbem_status lbem_set_fields(lbem_t *h, const float *E, const float *B) {
     h->wd_last = -1.0;
     if (h->d_traces) LBEM_CUDA(cudaMemsetAsync(h->d_traces, 0, sizeof(float) * (size_t)h->nrec * h->cap, h->stream));
     if (h->disp) {  // the pole starts at rest: D = E
-        for (float *p : {h->d_J, h->d_P, h->d_P2})
+        for (float *p : {h->d_J, h->d_J2, h->d_P, h->d_P2})
             LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * (size_t)h->grid.plane, h->stream));
     }
     drop_graph(h);
@@ -857,7 +860,8 @@ lbem_status lbem_set_dispersion(lbem_t *h, const float *wp2, const float *wr2, c
     if (!h) return fail(LBEM_ERR_ARG, "null handle");
     if (!wp2) {  // back to a non-dispersive medium
         LBEM_CUDA(cudaStreamSynchronize(h->stream));
-        for (float **p : {&h->d_wp2, &h->d_wr2, &h->d_gam, &h->d_J, &h->d_P, &h->d_P2, &h->d_pc, &h->d_pb, &h->d_pa}) {
+        for (float **p : {&h->d_wp2, &h->d_wr2, &h->d_gam, &h->d_J, &h->d_J2, &h->d_P, &h->d_P2, &h->d_pc, &h->d_pb,
+                          &h->d_pa}) {
             gfree(h, *p);
             *p = nullptr;
         }
@@ -886,14 +890,15 @@ lbem_status lbem_set_dispersion(lbem_t *h, const float *wp2, const float *wr2, c
                                          " sites with a parameter not finite and >= 0, or wp^2 + wr^2 > 4 w0");
     const size_t pl = (size_t)h->grid.plane;  // stored as planes with the grid's pitch (padding zero)
     if (!h->d_wp2) {
-        for (float **p : {&h->d_wp2, &h->d_wr2, &h->d_gam, &h->d_J, &h->d_P, &h->d_P2, &h->d_pc, &h->d_pb, &h->d_pa})
+        for (float **p : {&h->d_wp2, &h->d_wr2, &h->d_gam, &h->d_J, &h->d_J2, &h->d_P, &h->d_P2, &h->d_pc, &h->d_pb,
+                          &h->d_pa})
             LBEM_CUDA(gmalloc(h, (void **)p, sizeof(float) * pl, "dispersive pole"));
     }
     const float *src[3] = {dp, dr, dg};
     float *dst[3] = {h->d_wp2, h->d_wr2, h->d_gam};
     for (int k = 0; k < 3; k++) LBEM_CUDA(launch_to_plane(h, src[k], dst[k], h->stream));
     LBEM_CUDA(launch_pole_coefficients(h, h->stream));
-    for (float *p : {h->d_J, h->d_P, h->d_P2}) LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * pl, h->stream));
+    for (float *p : {h->d_J, h->d_J2, h->d_P, h->d_P2}) LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * pl, h->stream));
     LBEM_CUDA(cudaStreamSynchronize(h->stream));
     h->disp = true;
     drop_graph(h);
@@ -989,7 +994,7 @@ lbem_status lbem_save_state(lbem_t *h, void *dst) {
     if (p.ex) LBEM_CUDA(cudaMemcpyAsync((char *)dst + db, p.ex, (size_t)h->npop * p.explane, cudaMemcpyDefault, h->stream));
     if (h->disp) {  // then the pole's J and P planes
         const size_t pb = sizeof(float) * (size_t)h->grid.plane;
-        LBEM_CUDA(cudaMemcpyAsync((char *)dst + db, h->d_J, pb, cudaMemcpyDefault, h->stream));
+        LBEM_CUDA(cudaMemcpyAsync((char *)dst + db, h->pole_J(h->cur), pb, cudaMemcpyDefault, h->stream));
         LBEM_CUDA(cudaMemcpyAsync((char *)dst + db + pb, h->pole_P(h->cur), pb, cudaMemcpyDefault, h->stream));
     }
     if (!is_device_ptr(dst)) LBEM_CUDA(cudaStreamSynchronize(h->stream));
@@ -1005,7 +1010,7 @@ lbem_status lbem_load_state(lbem_t *h, const void *src, long long t_at_save) {
         LBEM_CUDA(cudaMemcpyAsync(p.ex, (const char *)src + db, (size_t)h->npop * p.explane, cudaMemcpyDefault, h->stream));
     if (h->disp) {
         const size_t pb = sizeof(float) * (size_t)h->grid.plane;
-        LBEM_CUDA(cudaMemcpyAsync(h->d_J, (const char *)src + db, pb, cudaMemcpyDefault, h->stream));
+        LBEM_CUDA(cudaMemcpyAsync(h->pole_J(h->cur), (const char *)src + db, pb, cudaMemcpyDefault, h->stream));
         LBEM_CUDA(cudaMemcpyAsync(h->pole_P(h->cur), (const char *)src + db + pb, pb, cudaMemcpyDefault, h->stream));
     }
     if (!is_device_ptr(src)) LBEM_CUDA(cudaStreamSynchronize(h->stream));
@@ -1190,7 +1195,7 @@ lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best) {
                 StepArgs a = step_args(h, cur0);
                 a.evt.rowptr = nullptr;
                 cudaEventRecord(e0, h->stream);
-                cudaError_t e = launch_march_2d(a, handle_walls(h), trial_steps, h->stream, &n);
+                cudaError_t e = launch_march_2d(a, handle_walls(h), h->storage, h->aniso, trial_steps, h->stream, &n);
                 if (e != cudaSuccess) st = cuda_fail(e, "lbem_autotune");
                 cudaEventRecord(e1, h->stream);
             }

@@ -349,11 +349,11 @@ struct Medium {
     // anisotropic medium (general.cu): r = c_x / c_y = sqrt(mu_xx / mu_yy), mubar = sqrt(mu_xx mu_yy); 1, 1: isotropic
     float ar = 1.f, amu = 1.f;
     // one dispersive pole per site (null without; pitched planes): its parameters (wp2 non-null marks a pole), the
-    // per-site coefficients of its update (pole_update: pc, pb, pa), J (updated in place) and P, read from Pr
-    // (time t) and written to Pw (the plane of the output state's parity)
+    // per-site coefficients of its update (pole_update: pc, pb, pa), J and P, read from J and Pr (time t) and written
+    // to Jw and Pw (the planes of the output state's parity)
     const float *wp2 = nullptr, *wr2 = nullptr, *gam = nullptr, *Pr = nullptr;
-    const float *pc = nullptr, *pb = nullptr, *pa = nullptr;
-    float *J = nullptr, *Pw = nullptr, *Jw = nullptr;
+    const float *pc = nullptr, *pb = nullptr, *pa = nullptr, *J = nullptr;
+    float *Pw = nullptr, *Jw = nullptr;
 };
 
 // Walls and absorbing layers (walls.cu): per axis x, y 0 = periodic, 1 = PEC wall, 2 = PMC wall; layer
@@ -364,15 +364,15 @@ struct Walls {
     int nlayer = 0;  // width of the layer
 };
 // What the general single-step kernel (general.cu) adds to a step: one Drude-Lorentz pole per site (parameters
-// and state as planes with the grid's pitch, J at t - 1/2 (in place), P at t read from P and written to Pn; wp2
+// and state as planes with the grid's pitch, J at t - 1/2 and P at t read from J and P and written to Jn and Pn; wp2
 // null: no pole) and a uniform in-plane permeability tensor
 // (axis speeds c_x^2 = r cbar^2, c_y^2 = cbar^2 / r with cbar^2 the stored c_L^2; mubar = sqrt(mu_xx mu_yy)).
 struct General {
     const float *wp2 = nullptr, *wr2 = nullptr, *gam = nullptr;
     const float *pc = nullptr, *pb = nullptr, *pa = nullptr;  // pole_update's per-site coefficients
-    float *J = nullptr;        // updated in place
-    const float *P = nullptr;  // P at t
-    float *Pn = nullptr;       // P at t + 1 (the other plane: neighbouring tiles of a multi-step launch read P at t)
+    const float *J = nullptr, *P = nullptr;  // J at t - 1/2, P at t
+    // J at t + 1/2, P at t + 1 (the other planes: neighbouring tiles or strips of a multi-step launch read those at t)
+    float *Jn = nullptr, *Pn = nullptr;
     float r = 1.f, mubar = 1.f;
 };
 // Output rectangle of one edge tile: columns x0 .. x0+w-1, rows y0 .. y0+h-1.
@@ -527,11 +527,13 @@ struct lbem {
     cudaStream_t edge_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     // frequency-dispersive permittivity (lbem_set_dispersion): pole parameters and state, planes (pitch layout)
-    // P has two planes, paired with the population buffers: P at the time of buf[c] is pole_P(c), so a launch
+    // J and P have two planes each, paired with the population buffers: P at the time of buf[c] is pole_P(c), so a launch
     // reads P from the plane of its input's parity and writes the other one (every launch flips cur).
-    float *d_wp2 = nullptr, *d_wr2 = nullptr, *d_gam = nullptr, *d_J = nullptr, *d_P = nullptr, *d_P2 = nullptr;
+    float *d_wp2 = nullptr, *d_wr2 = nullptr, *d_gam = nullptr, *d_J = nullptr, *d_J2 = nullptr, *d_P = nullptr,
+          *d_P2 = nullptr;
     float *d_pc = nullptr, *d_pb = nullptr, *d_pa = nullptr;  // pole_update's coefficients (pole_coefficients)
     float *pole_P(int c) const { return c ? d_P2 : d_P; }
+    float *pole_J(int c) const { return c ? d_J2 : d_J; }
     bool disp = false;
     // anisotropic medium (lbem_set_medium_aniso): r = sqrt(mu_xx / mu_yy), mubar = sqrt(mu_xx mu_yy)
     bool aniso = false;
@@ -576,9 +578,17 @@ int tb2_nshapes(int storage, bool has_mu);
 // two steps per launch by register streaming (rstream.cu): FP32 storage, uniform mu
 int rs2_nshapes();
 cudaError_t launch_step_2d_rs2(const StepArgs &a, int shape, cudaStream_t s);
-// up to 8 steps per launch by marching strips down the rows (march.cu): enqueues the launches of nsteps steps from
-// a.in, alternating between the two buffers; *launches of them
-cudaError_t launch_march_2d(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches);
+// up to 8 steps per launch by marching strips down the rows (march.cu and, for the other media and storages,
+// march_media.cu, march16.cu): enqueues the launches of nsteps steps from a.in, alternating between the two buffers;
+// *launches of them.  launch_march_2d chooses by the medium: FP32 with an isotropic medium (uniform or heterogeneous mu)
+// or an anisotropic tensor, walls and layers included, or a pole without walls, mu or tensor; 16-bit storage with uniform
+// mu and nx % 4 == 0, without walls.
+cudaError_t launch_march_2d(const StepArgs &a, const Walls &w, int storage, bool aniso, int nsteps, cudaStream_t s,
+                            int *launches);
+cudaError_t launch_march_2d_an(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches);
+cudaError_t launch_march_2d_mu(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches);
+cudaError_t launch_march_2d_pole(const StepArgs &a, int nsteps, cudaStream_t s, int *launches);
+cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaStream_t s, int *launches);
 int ss2_nshapes();  // strip streaming (sstream.cu): two steps per launch, FP32, uniform mu
 cudaError_t launch_step_2d_ss2(const StepArgs &a, int shape, cudaStream_t s);
 cudaError_t launch_step_2d_ss2_an(const StepArgs &a, cudaStream_t s);  // anisotropic medium, no pole

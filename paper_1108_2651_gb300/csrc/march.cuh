@@ -15,6 +15,8 @@
 // Every site update is the single-step kernels' arithmetic in their order, so results are bit-identical to theirs
 // (16-bit storage: to two steps per launch, the state rounded to the storage after every second step).
 #pragma once
+#include <algorithm>
+
 #include "lbem_internal.cuh"
 
 namespace lbk {
@@ -48,10 +50,13 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
     return r;
 }
-// a - b and a + b of pairs one of which is a product: as fma(b, -1, a) and fma(b, 1, a), one rounding each, since the
-// compiler contracts a packed product with the packed sum that follows it.
+// a - b and a + b of pairs one of which may be a product: the compiler contracts a packed product with the packed sum that
+// follows it (also when that is written as a packed fma by 1), so the difference is fma(b, -1, a), one rounding, and the
+// sum two scalar ones.
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ float2 sum2(float2 a, float2 b) { return fma2(b, make_float2(1.f, 1.f), a); }
+__device__ __forceinline__ float2 sum2(float2 a, float2 b) {
+    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 __device__ __forceinline__ float4 quad(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
@@ -109,15 +114,26 @@ struct MarchArgs {
     StepArgs a;           // a.in: the state at a.t, a.out: where the state after `steps` steps goes
     Walls w;
     int steps;            // 1 .. K
-    int nstrips, nseg;    // units: strip s, segment g is block g * nstrips + s
+    int nstrips, nseg;    // units: strips of columns by segments of rows
+    // Walls: the first nl and last nr strips hold walled columns or layers; they have nsegx segments, and the first and
+    // last segments of a strip hold he (hex) rows (0: as the others)
+    int nl, nr, nsegx, he, hex;
 };
 
 // The unit's column and row ranges: whole chunks of 4 columns and rows, evenly.
 __host__ __device__ __forceinline__ int march_cut(int k, int n, int of) { return (int)((long long)k * of / n); }
+// The first row of segment k of n, of ny rows, the first and the last segment of he rows (0: as the others).
+__host__ __device__ __forceinline__ int march_row(int k, int n, int ny, int he) {
+    if (he == 0 || k == 0 || k == n) return k == n ? ny : march_cut(k, n, ny);
+    return he + march_cut(k - 1, n - 2, ny - 2 * he);
+}
 
 template <int ST, int MED, int K, int D>
 struct MarchCfg {
-    static constexpr int H = (K + 3) / 4 * 4;     // halo columns on either side
+    // Halo columns on either side.  A level spoils one more column; block-int16 rounding (after every second level, and
+    // as the last one is stored) spoils the rest of a group of four that holds a spoilt column, since they share an
+    // exponent: four columns per two levels.
+    static constexpr int H = ST == LBEM_I16B ? 2 * K : (K + 3) / 4 * 4;
     static constexpr int W = 128 - 2 * H;         // columns a strip can own
     static constexpr int PS = ST == LBEM_F32 ? 512 : 256;                  // bytes of a staged plane row
     static constexpr int SB = 5 * PS + (MED == MARCH_POLE ? 1024 : 0);     // bytes of a stage (POLE: P and J too)
@@ -154,16 +170,34 @@ __device__ __forceinline__ int m_encode(const PopBuf &b, float4 v, uint2 &r) {
         return 0;
     }
 }
+// Encode and decode 4 sites: what reading back the stored state gives.
+template <int ST>
+__device__ __forceinline__ float4 m_round4(const PopBuf &b, float4 v) {
+    if constexpr (ST == LBEM_I16B) {  // Codec::enc4e's steps without packing the mantissas
+        const float m = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+        const int e = ((__float_as_int(m) >> 23) & 0xff) - 127 + 1, ec = min(max(e, -99), 100);
+        const float s = pow2f(15 - ec), f = m < 0x1p-100f ? 0.f : pow2f(ec - 15);
+        auto one = [&](float x) {  // (a zero block: q * 0 + 0 = +0)
+            const float q = __fadd_rn(__fadd_rn(fminf(fmaxf(__fmul_rn(x, s), -32767.f), 32767.f), kMagic), -kMagic);
+            return __fmaf_rn(q, f, 0.f);
+        };
+        float4 r = make_float4(one(v.x), one(v.y), one(v.z), one(v.w));
+        if (!(m < 0x1p+100f)) r.x = r.y = r.z = r.w = __fmul_rn(32767.f, pow2f(112));
+        return r;
+    } else {
+        uint2 r;
+        const int e = m_encode<ST>(b, v, r);
+        return m_decode<ST>(b, r, e);
+    }
+}
 template <int ST>
 __device__ __forceinline__ void m_round(const PopBuf &b, Quad5 &o) {
     if constexpr (ST != LBEM_F32) {
-        float4 *v[5] = {&o.p0, &o.p1, &o.p2, &o.p3, &o.p4};
-#pragma unroll
-        for (int p = 0; p < 5; p++) {
-            uint2 r;
-            const int e = m_encode<ST>(b, *v[p], r);
-            *v[p] = m_decode<ST>(b, r, e);
-        }
+        o.p0 = m_round4<ST>(b, o.p0);
+        o.p1 = m_round4<ST>(b, o.p1);
+        o.p2 = m_round4<ST>(b, o.p2);
+        o.p3 = m_round4<ST>(b, o.p3);
+        o.p4 = m_round4<ST>(b, o.p4);
     }
 }
 
@@ -244,8 +278,8 @@ struct MarchFalse {
 
 // The march of one unit by one warp: kp steps from a.t.
 template <int ST, int MED, bool WL, int K, int D>
-__device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, int kp, int nstrips, int nseg, int strip,
-                                           int seg, unsigned smem) {
+__device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, int kp, int nstrips, int strip, int y0,
+                                           int y1, unsigned smem) {
     using Cfg = MarchCfg<ST, MED, K, D>;
     constexpr int H = Cfg::H, PS = Cfg::PS, SB = Cfg::SB, RB = Cfg::RB, NR = Cfg::NR;
     constexpr bool F32 = ST == LBEM_F32;
@@ -253,7 +287,6 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
     const int lane = threadIdx.x;
     const int xs = 4 * march_cut(strip, nstrips, G.nchunk);
     const int xe = strip == nstrips - 1 ? G.nx : 4 * march_cut(strip + 1, nstrips, G.nchunk);
-    const int y0 = march_cut(seg, nseg, G.ny), y1 = march_cut(seg + 1, nseg, G.ny);
     const int X = xs - H + 4 * lane;  // the lane's first column, unwrapped
     const int xw = wrapi(X, G.nx);
     // a lane whose columns are contiguous and aligned copies 16 (8) bytes per plane row; the others (at the wrap of a
@@ -578,8 +611,10 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
     };
     float4 fx = make_float4(1.f, 1.f, 1.f, 1.f);  // the columns' factors (the table is padded with 1 to the pitch)
     if (WL && w.fx && X >= 0 && X < G.nx) fx = __ldg(reinterpret_cast<const float4 *>(w.fx + X));
+    float fyl = 1.f;  // the rows' factors: lane l that of row yl - K + l, as of the last row with it % 16 = 0
+    int fy0 = 0;
     auto layer = [&](int yu, Quad5 &n) {
-        const float fy = w.fy && (unsigned)yu < (unsigned)G.ny ? __ldg(w.fy + yu) : 1.f;
+        const float fy = __shfl_sync(FULL, fyl, yu - fy0);
         const float4 f = make_float4(__fmul_rn(fx.x, fy), __fmul_rn(fx.y, fy), __fmul_rn(fx.z, fy), __fmul_rn(fx.w, fy));
         float4 *v[5] = {&n.p0, &n.p1, &n.p2, &n.p3, &n.p4};
 #pragma unroll
@@ -766,6 +801,11 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
     // Rows by twos (an odd last one computes a row that nothing keeps), so that half of the registers' moves go away.
 #pragma unroll 1
     for (int it = 0; it < nit; it += 2) {
+        if (WL && (it & 15) == 0) {
+            fy0 = yl - K;
+            const int y = fy0 + lane;
+            fyl = w.fy && (unsigned)y < (unsigned)G.ny ? __ldg(w.fy + y) : 1.f;
+        }
         if (many && (it & 15) == 0)  // the flags of the next 16 rows
             fb |= (__ballot_sync(FULL, (a.evt.mask[wrapi(yl + (lane & 15), G.ny)] & smask) != 0) & 0xffffu) << (K - 1);
         if (many) {
@@ -793,6 +833,107 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
         }
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+}
+
+template <int ST, int MED, bool WL, int K, int D>
+__global__ void __launch_bounds__(32, 8) march2d(const __grid_constant__ MarchArgs m) {
+    extern __shared__ __align__(1024) float march_smem[];
+    const unsigned smem = (unsigned)__cvta_generic_to_shared(march_smem);
+    const Grid &G = m.a.g;
+    if constexpr (WL) {
+        using Cfg = MarchCfg<ST, MED, K, D>;
+        const int nx = m.nl + m.nr, nbx = nx * m.nsegx;  // the walled strips' units first: they are the longer ones
+        int strip, y0, y1;
+        if (blockIdx.x < nbx) {
+            const int seg = blockIdx.x / nx, k = blockIdx.x - seg * nx;
+            strip = k < m.nl ? k : m.nstrips - nx + k;
+            y0 = march_row(seg, m.nsegx, G.ny, m.hex);
+            y1 = march_row(seg + 1, m.nsegx, G.ny, m.hex);
+        } else {
+            const int b = blockIdx.x - nbx, n = m.nstrips - nx, seg = b / n;
+            strip = m.nl + b - seg * n;
+            y0 = march_row(seg, m.nseg, G.ny, m.he);
+            y1 = march_row(seg + 1, m.nseg, G.ny, m.he);
+        }
+        // units away from walls and layers (their reach of K rows and columns included) are periodic ones
+        const int edge = max(m.w.nlayer, 1), X0 = 4 * march_cut(strip, m.nstrips, G.nchunk) - Cfg::H;
+        if ((m.w.kind[0] && (X0 < edge || X0 + 128 > G.nx - edge)) ||
+            (m.w.kind[1] && (y0 - K < edge || y1 + K > G.ny - edge)))
+            march_unit<ST, MED, true, K, D>(m.a, m.w, m.steps, m.nstrips, strip, y0, y1, smem);
+        else
+            march_unit<ST, MED, false, K, D>(m.a, m.w, m.steps, m.nstrips, strip, y0, y1, smem);
+    } else {
+        const int seg = blockIdx.x / m.nstrips, strip = blockIdx.x - seg * m.nstrips;
+        march_unit<ST, MED, false, K, D>(m.a, m.w, m.steps, m.nstrips, strip, march_cut(seg, m.nseg, G.ny),
+                                         march_cut(seg + 1, m.nseg, G.ny), smem);
+    }
+}
+
+// Launches of K steps, the last one of what is left.  One wave of units: as many segments as fill the GPU (a second
+// wave would leave it half empty), of at least two rows.  Each launch may start while the one before drains
+// (programmatic dependent launch; it waits for its input with griddepcontrol.wait): 128^2 8.2 us a launch against
+// 10.3 us, 1024^2 18 us against 20.5 us.
+template <int ST, int MED, bool WL, int K, int D>
+static cudaError_t launch_march(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches) {
+    using Cfg = MarchCfg<ST, MED, K, D>;
+    auto *k = march2d<ST, MED, WL, K, D>;
+    static int per_sm = 0, nsm = 0;
+    if (!per_sm) {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, 32, Cfg::smem);
+        if (e != cudaSuccess) return e;
+        per_sm = std::max(n, 1);
+    }
+    MarchArgs m;
+    m.a = a;
+    m.w = w;
+    m.nstrips = (a.g.nchunk + Cfg::W / 4 - 1) / (Cfg::W / 4);
+    const int cap = per_sm * nsm;
+    m.nl = m.nr = m.nsegx = m.he = m.hex = 0;
+    if (WL && w.kind[0]) {  // strips whose columns (with the halo) reach a wall or its layer
+        const int edge = std::max(w.nlayer, 1);
+        auto x0 = [&](int k) { return 4 * march_cut(k, m.nstrips, a.g.nchunk) - Cfg::H; };
+        while (m.nl < m.nstrips && x0(m.nl) < edge) m.nl++;
+        while (m.nl + m.nr < m.nstrips && x0(m.nstrips - 1 - m.nr) + 128 > a.g.nx - edge) m.nr++;
+    }
+    // a walled unit's row takes about twice a periodic one's: half the rows (segments twice as many)
+    m.nseg = std::max(1, std::min(cap / (m.nstrips + m.nl + m.nr), a.g.ny / 2));
+    m.nsegx = std::max(1, std::min(2 * m.nseg, a.g.ny / 2));
+    if (WL && w.kind[1] && m.nseg >= 4) {
+        const int reach = std::max(w.nlayer, 1) + K, he = std::max(reach, a.g.ny / m.nseg / 2 - (K - 1));
+        if (2 * he + (m.nseg - 2) * 2 <= a.g.ny) m.he = he;
+    }
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((m.nl + m.nr) * m.nsegx + (m.nstrips - m.nl - m.nr) * m.nseg));
+    cfg.blockDim = dim3(32);
+    cfg.dynamicSmemBytes = Cfg::smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    *launches = 0;
+    for (int t = 0; t < nsteps; t += K, ++*launches) {
+        m.steps = std::min(K, nsteps - t);
+        m.a.t = a.t + t;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k, m);
+        if (e != cudaSuccess) return e;
+        std::swap(m.a.in, m.a.out);
+        if (MED == MARCH_POLE) {
+            float *J = const_cast<float *>(m.a.med.J), *P = const_cast<float *>(m.a.med.Pr);
+            m.a.med.J = m.a.med.Jw;
+            m.a.med.Pr = m.a.med.Pw;
+            m.a.med.Jw = J;
+            m.a.med.Pw = P;
+        }
+    }
+    return cudaSuccess;
 }
 
 }  // namespace lbk

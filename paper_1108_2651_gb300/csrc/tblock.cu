@@ -340,10 +340,8 @@ __device__ __forceinline__ void tb_step_a(const StepArgs &a, const float *IN, co
             constexpr int JPL = TbGeom<TBY, false, true>::JS_PL;
             pp.P = lds4(PS + py * TW + c);
             pp.J = pp.wp = pp.wr = pp.gm = make_float4(0.f, 0.f, 0.f, 0.f);
-            // J is updated in place by the tile owning the site.  Lanes past nx (rows past ny) of a ragged last
-            // tile read J at wrapped sites of another tile, which may be updating them: their pole results only
-            // ever reach the row padding or are dropped, while the collisions they feed use P at t, which no
-            // launch writes in place.
+            // lanes past nx (rows past ny) of a ragged last tile work on wrapped sites: their pole results only ever
+            // reach the row padding or are dropped
             if (own) {
                 const float *js = JS + (py - 1) * TBX + 4 * lane;
                 pp.J = lds4(js);
@@ -427,8 +425,8 @@ __device__ __forceinline__ void tb_step_b(const StepArgs &a, const float *P, flo
         __stcs(o + 2 * pl4, o2);
         __stcs(o + 3 * pl4, o3);
         __stcs(o + 4 * pl4, o4);
-        if (POLE) {  // J in place (only this site reads it), P to the plane of the output's parity
-            *reinterpret_cast<float4 *>(a.med.J + off) = pp.J;
+        if (POLE) {  // J and P to the planes of the output's parity
+            *reinterpret_cast<float4 *>(a.med.Jw + off) = pp.J;
             *reinterpret_cast<float4 *>(a.med.Pw + off) = pp.P;
         }
     }

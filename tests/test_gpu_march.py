@@ -13,9 +13,9 @@ from paper_1108_2651_gb300 import lbem, workloads as W
 pytestmark = pytest.mark.gpu
 
 
-def _problem(shape, seed, nsteps):
-    eps, _ = W.random_medium(shape, seed)
-    p = W.Problem("march", 2, shape, eps, None, nsteps)
+def _problem(shape, seed, nsteps, mu=False):
+    eps, mu_r = W.random_medium(shape, seed, 1.2 if not mu else 1.0, mu=mu)
+    p = W.Problem("march", 2, shape, eps, mu_r, nsteps)
     p.E0, p.B0 = W.random_fields(shape, seed + 1, 0.3)
     ny, nx = shape
     n = ny * nx
@@ -29,14 +29,14 @@ def _problem(shape, seed, nsteps):
     return p
 
 
-def _run(p, calls, steps_per_pass=None, graphs=False):
+def _run(p, calls, steps_per_pass=None, graphs=False, storage="f32", shape=-1):
     import torch
 
     stream = torch.cuda.Stream() if graphs else None
-    s = lbem.Solver(p.shape, stream=stream.cuda_stream if stream else None)
+    s = lbem.Solver(p.shape, storage=storage, stream=stream.cuda_stream if stream else None)
     s.set_problem(p)
     if steps_per_pass:
-        lbem.lbem_set_temporal_blocking(s.h, steps_per_pass, -1)
+        lbem.lbem_set_temporal_blocking(s.h, steps_per_pass, shape)
     if graphs:
         lbem.lbem_set_graphs(s.h, True)
     for n in calls:
@@ -60,3 +60,33 @@ def test_march_is_bitwise_identical_to_single_steps(lbem, shape):
             got = _run(p, calls, graphs=graphs)
             for a, b in zip(got, ref):
                 np.testing.assert_array_equal(a, b, err_msg=f"{shape}, calls {calls}, graphs {graphs}")
+
+
+@pytest.mark.parametrize("shape", [(1, 4), (7, 116), (33, 260), (300, 452)])
+@pytest.mark.parametrize("medium", ["mu", "aniso", "pole", "walls", "walls_mu", "walls_aniso"])
+def test_march_media_are_bitwise_identical_to_single_steps(lbem, shape, medium):
+    p = _problem(shape, 800 + shape[1], 29, mu=medium.endswith("mu"))
+    rng = np.random.default_rng(5)
+    if medium.endswith("aniso"):
+        p.aniso = (2.0, 1.0)
+    if medium == "pole":
+        p.wp2 = rng.uniform(0.0, 0.5, shape)
+        p.wr2 = rng.uniform(0.0, 0.1, shape)
+        p.gamma = rng.uniform(0.0, 0.2, shape)
+    if medium.startswith("walls"):
+        p.bc, p.layer, p.gamma_max = (lbem.BC_PEC, lbem.BC_PMC, 0), min(5, min(shape) // 2), 0.3
+    ref = _run(p, [29], steps_per_pass=1)
+    for calls, graphs in (([29], False), ([6, 8, 15], True), ([3, 4, 5, 17], False)):
+        for a, b in zip(_run(p, calls, graphs=graphs), ref):
+            np.testing.assert_array_equal(a, b, err_msg=f"{medium} {shape}, calls {calls}")
+
+
+@pytest.mark.parametrize("shape", [(1, 4), (7, 116), (33, 260), (300, 1028)])
+@pytest.mark.parametrize("storage", ["f16", "bf16", "i16b"])
+def test_march_16bit_equals_launches_of_two_steps(lbem, shape, storage):
+    """(300, 1028): strips' edges long enough that a block exponent taken from a spoilt halo column shows.)"""
+    p = _problem(shape, 900 + shape[1], 30)
+    for calls in ([30], [8, 22], [4, 6, 10, 10], [3, 27]):
+        ref = _run(p, calls, steps_per_pass=2, shape=0, storage=storage)
+        for a, b in zip(_run(p, calls, storage=storage), ref):
+            np.testing.assert_array_equal(a, b, err_msg=f"{storage} {shape}, calls {calls}")
