@@ -416,6 +416,9 @@ struct lbem_batch {
     size_t units_cap = 0;
     int nunits = 0;
     int *d_sched = nullptr;
+    // the marching kernel's units (march_batch.cu; the members' sizes never change)
+    lbk::BatchMarchUnit *d_march = nullptr;
+    int nmarch = 0;
     // the two-step kernels' packed states with halos: two population buffers and c_L^2, [rows][W] per plane, member m
     // from packed row r0[m] (d_r0, n + 1 entries)
     float *d_pack = nullptr;  // 11 planes: buffer 0 (5), buffer 1 (5), c_L^2 (1)
@@ -448,11 +451,12 @@ using namespace lbk;
 // Variants: R = 1, 2, 4 rows per warp; 0 one site per thread; -1 persistent register pipeline; -5, -6 R = 1
 // capped for 5 / 6 blocks per SM; -7, -8 linear over each member's padded plane (uncapped / 5 blocks per SM);
 // 100 + k: two steps per launch through shared-memory tiles, tile shape k (launch_batch_tb2); 200 + k: two steps per
-// launch by strip streaming, shape k (launch_batch_ss2).
-static const int kRowsB[] = {1, 2, 4, 0, -1, -5, -6, -7, -8, 100, 101, 102, 103, 104, 200, 201};
+// launch by strip streaming, shape k (launch_batch_ss2); 300: up to 8 steps per launch by marching (launch_batch_march).
+static const int kRowsB[] = {1, 2, 4, 0, -1, -5, -6, -7, -8, 100, 101, 102, 103, 104, 200, 201, 300};
 static const int kBatchVariants = (int)(sizeof(kRowsB) / sizeof(kRowsB[0]));
 static const int kLinVariant = 7;  // the single-step kernel that takes the odd step of a two-step variant
-static bool two_step(int variant) { return kRowsB[variant] >= 100; }
+static bool march_variant(int variant) { return kRowsB[variant] >= 300; }
+static bool two_step(int variant) { return kRowsB[variant] >= 100 && !march_variant(variant); }
 static bool strip_variant(int variant) { return kRowsB[variant] >= 200; }
 
 static void drop_batch_graph(lbem_batch_t *b) {
@@ -596,6 +600,7 @@ static lbem_status upload_unit_tables(lbem_batch_t *b, int shape) {
     if (ul.size() > (size_t)(1 << 30)) return fail(LBEM_ERR_ARG, "lbem_batch: too many units");
     if (b->units_cap < ul.size()) {
         cudaFree(b->d_units);
+    cudaFree(b->d_march);
         b->d_units = nullptr;
         b->units_cap = 0;
         if (cudaMalloc((void **)&b->d_units, sizeof(BatchUnit) * ul.size()) != cudaSuccess) {
@@ -611,7 +616,35 @@ static lbem_status upload_unit_tables(lbem_batch_t *b, int shape) {
     return LBEM_OK;
 }
 
+// The marching kernel's unit table, and every member's step arguments for both buffer parities.
+static lbem_status upload_march_tables(lbem_batch_t *b) {
+    if (!b->d_march) {
+        std::vector<Grid> grids(b->n);
+        for (int k = 0; k < b->n; k++) grids[k] = b->members[k]->grid;
+        const std::vector<BatchMarchUnit> u = batch_march_units(b->n, grids.data());
+        if (cudaMalloc((void **)&b->d_march, sizeof(BatchMarchUnit) * u.size()) != cudaSuccess) {
+            cudaGetLastError();
+            b->d_march = nullptr;
+            return fail(LBEM_ERR_NOMEM, "lbem_batch: no room for the unit table");
+        }
+        b->nmarch = (int)u.size();
+        LBEM_CUDA(cudaMemcpyAsync(b->d_march, u.data(), sizeof(BatchMarchUnit) * u.size(), cudaMemcpyHostToDevice,
+                                  b->stream));
+        LBEM_CUDA(cudaStreamSynchronize(b->stream));
+    }
+    std::vector<StepArgs> args(2 * (size_t)b->n);
+    for (int k = 0; k < b->n; k++) {
+        args[2 * k] = step_args(b->members[k], b->members[k]->cur);
+        args[2 * k + 1] = step_args(b->members[k], b->members[k]->cur ^ 1);
+    }
+    LBEM_CUDA(cudaMemcpyAsync(b->d_args, args.data(), sizeof(StepArgs) * args.size(), cudaMemcpyHostToDevice,
+                              b->stream));
+    LBEM_CUDA(cudaStreamSynchronize(b->stream));  // host vectors go out of scope
+    return LBEM_OK;
+}
+
 static lbem_status upload_tables(lbem_batch_t *b, int variant) {
+    if (march_variant(variant)) return upload_march_tables(b);
     if (two_step(variant)) {  // the pair kernel's tiles, and the linear single-step kernel's table for an odd step
         lbem_status st = strip_variant(variant) ? upload_unit_tables(b, kRowsB[variant] - 200)
                                                 : upload_tile_tables(b, batch_tb2_rows(kRowsB[variant] - 100));
@@ -696,9 +729,20 @@ static cudaError_t launch_batch(lbem_batch_t *b, int variant, int offset) {
 }
 
 // Enqueue nsteps steps of `variant` from the members' current state (t0 in device memory): one launch per step, or
-// for a two-step variant one launch per pair of steps, after a single step first when nsteps is odd.  Returns the
+// for a two-step variant one launch per pair of steps, after a single step first when nsteps is odd, or one per 8
+// steps, the last one of what is left (marching).  Returns the
 // number of launches (each one flips the members' buffers) in *nlaunch.
 static cudaError_t enqueue_batch(lbem_batch_t *b, int variant, int nsteps, int *nlaunch) {
+    if (march_variant(variant)) {
+        int n = 0;
+        for (int t = 0; t < nsteps; t += MARCH_BATCH_STEPS, n++) {
+            cudaError_t e = launch_batch_march(b->d_args, b->d_march, b->nmarch, b->d_t0, t,
+                                               std::min(MARCH_BATCH_STEPS, nsteps - t), n & 1, b->stream);
+            if (e != cudaSuccess) return e;
+        }
+        *nlaunch = n;
+        return cudaSuccess;
+    }
     if (!two_step(variant)) {
         for (int k = 0; k < nsteps; k++) {
             cudaError_t e = launch_batch(b, variant, k);
@@ -819,9 +863,11 @@ lbem_status lbem_batch_step(lbem_batch_t *b, int nsteps) {
         int nl = 0;
         LBEM_CUDA(enqueue_batch(b, b->variant, nsteps, &nl));
     }
-    // each single-step launch flips the members' buffers; the two-step variants unpack the pairs' result into the
+    // each single-step or marching launch flips the members' buffers; the two-step variants unpack the pairs' result into the
     // buffer they packed from, so only their odd first step flips
-    const int flips = two_step(b->variant) ? (nsteps & 1) : nsteps;
+    const int flips = march_variant(b->variant) ? (nsteps + MARCH_BATCH_STEPS - 1) / MARCH_BATCH_STEPS
+                      : two_step(b->variant)    ? (nsteps & 1)
+                                                : nsteps;
     for (lbem_t *h : b->members) {
         h->cur ^= (flips & 1);
         h->t += nsteps;

@@ -339,14 +339,15 @@ static lbem_status rebuild_events(lbem_t *h) {
     gfree(h, h->d_ev);
     h->d_ev = nullptr;
     h->nev = (int)sorted.size();
-    if (h->nev) {
-        std::vector<unsigned long long> mask(h->grid.nrows, 0);
-        for (size_t i = 0; i < order.size(); i++) mask[rows[order[i]]] |= 1ull << (sorted[i].x / event_bucket(nx));
-        if (!h->d_evmask)
-            LBEM_CUDA(gmalloc(h, (void **)&h->d_evmask, sizeof(unsigned long long) * h->grid.nrows, "event columns"));
-        LBEM_CUDA(cudaMemcpy(h->d_evmask, mask.data(), sizeof(mask[0]) * mask.size(), cudaMemcpyHostToDevice));
+    // the row pointers and, from the next multiple of 8 bytes, the rows' column masks: one array, one copy
+    const size_t nrp = (size_t)(h->grid.nrows + 2) / 2 * 2;
+    if (h->dim == 2) rowptr.resize(nrp + 2 * (size_t)h->grid.nrows, 0);
+    for (size_t i = 0; i < order.size() && h->dim == 2; i++) {
+        const int b = sorted[i].x / event_bucket(nx);
+        rowptr[nrp + 2 * rows[order[i]] + (b >> 5)] |= (int)(1u << (b & 31));
     }
-    if (!h->d_rowptr) LBEM_CUDA(gmalloc(h, (void **)&h->d_rowptr, sizeof(int) * (h->grid.nrows + 1), "event rows"));
+    if (!h->d_rowptr) LBEM_CUDA(gmalloc(h, (void **)&h->d_rowptr, sizeof(int) * rowptr.size(), "event rows"));
+    h->d_evmask = reinterpret_cast<unsigned long long *>(h->d_rowptr + nrp);
     LBEM_CUDA(cudaMemcpy(h->d_rowptr, rowptr.data(), sizeof(int) * rowptr.size(), cudaMemcpyHostToDevice));
     if (h->nev) {
         LBEM_CUDA(gmalloc(h, (void **)&h->d_ev, sizeof(Event) * sorted.size(), "events"));
@@ -489,7 +490,7 @@ void lbem_destroy(lbem_t *h) {
     drop_graph(h);
     adjoint_free(h);
     for (void *p : {(void *)h->pool, (void *)h->cL2, (void *)h->mu, (void *)h->dlnmu, (void *)h->d_rowptr,
-                    (void *)h->d_ev, (void *)h->d_evmask, (void *)h->d_amp, (void *)h->d_traces, (void *)h->d_partials,
+                    (void *)h->d_ev, (void *)h->d_amp, (void *)h->d_traces, (void *)h->d_partials,
                     (void *)h->d_diag, (void *)h->d_counter, (void *)h->d_stage, (void *)h->d_fx, (void *)h->d_fy,
                     (void *)h->d_fz,
                     (void *)h->d_wp2, (void *)h->d_wr2, (void *)h->d_gam, (void *)h->d_J, (void *)h->d_J2, (void *)h->d_P,

@@ -486,7 +486,7 @@ struct lbem {
     // events
     int *d_rowptr = nullptr;
     lbk::Event *d_ev = nullptr;
-    unsigned long long *d_evmask = nullptr;  // Events::mask
+    unsigned long long *d_evmask = nullptr;  // Events::mask (in d_rowptr's array)
     float *d_amp = nullptr;
     float *d_traces = nullptr;
     int nsrc = 0, nrec = 0, nt = 0, cap = 0, nev = 0;
@@ -632,6 +632,14 @@ struct __align__(16) BatchUnit {
     const int *rowptr;
     const Event *ev;
 };
+// One unit of the batch's marching kernel (march_batch.cu): member m, its strip and rows y0 .. y1-1.
+struct __align__(16) BatchMarchUnit {
+    int m, strip, y0, y1;
+};
+constexpr int MARCH_BATCH_STEPS = 8;                          // steps per launch
+std::vector<BatchMarchUnit> batch_march_units(int n, const Grid *grids);  // tall units first
+cudaError_t launch_batch_march(const StepArgs *args, const BatchMarchUnit *units, int nunits, const long long *t0p,
+                               int toff, int steps, int par, cudaStream_t s);
 int batch_ss2_nshapes();
 int batch_ss2_rows(int shape);    // chunk rows (TBY) of a shape
 int batch_ss2_chunks(int shape);  // chunks of a full unit
