@@ -269,11 +269,12 @@ __device__ __forceinline__ void m_collide(float4 g0, float4 g1, float4 g2, float
     o.p4 = quad(o4a, o4b);
 }
 
-struct MarchTrue {
-    static constexpr bool value = true;
+// The copies of a row's code: without events; with events, or of a launch of fewer than K steps.
+struct MarchPlain {
+    static constexpr bool ev = false;
 };
-struct MarchFalse {
-    static constexpr bool value = false;
+struct MarchAny {
+    static constexpr bool ev = true;
 };
 
 // The march of one unit by one warp: kp steps from a.t.
@@ -638,12 +639,13 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
             set(n.p4, k, __fadd_rn(get(n.p4, k), Ty));
         }
     };
-    // One row, every level one row further.  EV: a row with events or of a launch of fewer than K steps; its straight
-    // line only hands the quads of the lanes concerned to their places in shared memory and adds the sources' terms
-    // (S^ = 0 adds -0 and changes nothing), and the records are gone through once, before and after: with their code at
-    // every level the row was 20 KB that the instruction cache did not hold, 3 us a row against 0.5 us of a plain one.
-    auto row = [&](auto evc) {
-        constexpr bool EV = decltype(evc)::value;
+    // One row, every level one row further.  EV: a row with events; its straight line only hands the quads of the lanes
+    // concerned to their places in shared memory, and (SRC: with sources, or in a launch of fewer than K steps) adds the
+    // sources' terms (S^ = 0 adds -0 and changes nothing); the records are gone through once, before and after.  With
+    // their code at every level the row was 20 KB that the instruction cache did not hold, 3 us against 0.5 us of a
+    // plain one.
+    auto row = [&](auto mode) {
+        constexpr bool EV = decltype(mode)::ev, SRC = EV;
         const unsigned s = smem + st * SB + lane * (PS / 32);
         float4 g0, a1, g2, a3, g4, P = z4, J = z4;
         stage(s, g0, a1, g2, a3, g4, P, J);
@@ -651,7 +653,7 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
         unsigned levels = 0, recs = 0;  // EV: the levels to leave the line at, the records of the row's levels
         unsigned long long place = 0;   // the lane's place per level (6 bits, 32: none)
         if (EV) {
-            if (kp < K) levels = 1u << (kp - 1);
+            if (SRC && kp < K) levels = 1u << (kp - 1);
             recs = __ballot_sync(FULL, (unsigned)(yl - erow) < (unsigned)K);
 #pragma unroll 1
             for (unsigned b = recs; b; b &= b - 1) {
@@ -662,7 +664,7 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
                 if ((v.y & 31) == lane) {
                     const unsigned q = (unsigned)v.y >> 8;
                     place |= (unsigned long long)(32 | q) << (6 * j);
-                    if (!(v.y & 128))
+                    if (SRC && !(v.y & 128))
                         m_sts1(smem + Cfg::O_Q + q * Cfg::QB + 80 + ((v.y >> 5) & 3) * 4,
                                __fsub_rn(0.f, m_lds1(smem + Cfg::O_AMP + (l * K + j) * 4)));
                 }
@@ -692,14 +694,14 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
                     m_sts(q + 32, h2);
                     m_sts(q + 48, g3);
                     m_sts(q + 64, h4);
-                    S = m_lds(q + 80);
+                    if (SRC) S = m_lds(q + 80);
                     if (MED == MARCH_POLE) m_sts(q + 96, Pn);
                 }
-                if (MED == MARCH_MU)
+                if (SRC && MED == MARCH_MU)
                     sh = make_float4(__fadd_rn(sh.x, S.x), __fadd_rn(sh.y, S.y), __fadd_rn(sh.z, S.z), __fadd_rn(sh.w, S.w));
             }
             m_collide<MED>(h0, g1, h2, g3, h4, c, Pn, sh, r, ri, fs, n, sig);
-            if (EV && MED != MARCH_MU && leave) source(c, S, n);
+            if (SRC && MED != MARCH_MU && leave) source(c, S, n);
             if (MED == MARCH_POLE) pole(mr, c, sig, Jn, Pn);
             if (WL) layer(yl - j, n);
             // 16-bit storage: the state is rounded after every second step (and as it is stored)
@@ -714,12 +716,12 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
                 PP[j] = Po;
                 JJ[j] = Jo;
             }
-            if (EV && leave && j < K - 1 && j == kp - 1) store(yl - j, n, Pn, Jn);
+            if (SRC && leave && j < K - 1 && j == kp - 1) store(yl - j, n, Pn, Jn);
             o = n;
             Po = Pn;
             Jo = Jn;
         }
-        if (!EV || kp == K) store(yl - (K - 1), o, Po, Jo);
+        if (!SRC || kp == K) store(yl - (K - 1), o, Po, Jo);
         if (EV) {  // the receivers
 #pragma unroll 1
             for (unsigned b = recs; b; b &= b - 1) {
@@ -798,37 +800,61 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
         st = st == D - 1 ? 0 : st + 1;
         rs = (rs + 1) & (NR - 1);
     };
-    // Rows by twos (an odd last one computes a row that nothing keeps), so that half of the registers' moves go away.
-#pragma unroll 1
-    for (int it = 0; it < nit; it += 2) {
+    auto row_head = [&](int it) {
         if (WL && (it & 15) == 0) {
             fy0 = yl - K;
             const int y = fy0 + lane;
             fyl = w.fy && (unsigned)y < (unsigned)G.ny ? __ldg(w.fy + y) : 1.f;
         }
-        if (many && (it & 15) == 0)  // the flags of the next 16 rows
-            fb |= (__ballot_sync(FULL, (a.evt.mask[wrapi(yl + (lane & 15), G.ny)] & smask) != 0) & 0xffffu) << (K - 1);
-        if (many) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
+    };
+    // The rows, in loops that hold one copy of the code each (a loop with a second copy in it costs a plain row 150 to 280
+    // cycles for the jump across, taken or not).
+    int it = 0;
+    if (many) {
 #pragma unroll 1
-            for (int u = 0; u < 2; u++) {
-                asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
-                row_many();
-                next_row();
-                fb >>= 1;
-            }
-        } else if (kp < K || (hasev && __any_sync(FULL, (unsigned)(yl + 1 - erow) <= (unsigned)K))) {
+        for (; it < nit; it++) {
+            if ((it & 15) == 0)  // the flags of the next 16 rows
+                fb |= (__ballot_sync(FULL, (a.evt.mask[wrapi(yl + (lane & 15), G.ny)] & smask) != 0) & 0xffffu)
+                      << (K - 1);
+            row_head(it);
+            row_many();
+            next_row();
+            fb >>= 1;
+        }
+    }
 #pragma unroll 1
-            for (int u = 0; u < 2; u++) {
-                asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
-                row(MarchTrue());
+    while (it < nit) {
+        // the lane's record is on one of the levels' rows from iteration `from` to `from` + K - 1
+        const int from = erow - (y0 - (kp - 1));
+        const unsigned near = __ballot_sync(FULL, (unsigned)(it - from) < (unsigned)K);
+        if (kp < K || near) {
+            do {
+                row_head(it);
+                row(MarchAny());
                 next_row();
-            }
+                it++;
+            } while (it < nit && (kp < K || __any_sync(FULL, (unsigned)(it - from) < (unsigned)K)));
         } else {
-#pragma unroll
-            for (int u = 0; u < 2; u++) {
-                asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
-                row(MarchFalse());
+            // plain rows up to the next record, by twos, so that half of the registers' moves go away (an odd last one
+            // of the unit computes a row that nothing keeps; before a record one is left to the other copy)
+            int end = __reduce_min_sync(FULL, from > it ? from : 0x7ffffff0);
+            end = end >= nit ? nit : it + ((end - it) & ~1);
+            if (end == it) {
+                row_head(it);
+                row(MarchAny());
                 next_row();
+                it++;
+            }
+            constexpr int U = WL ? 1 : 2;  // (the longer row with walls singly, to keep its code short)
+#pragma unroll 1
+            for (; it < end; it += U) {
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    row_head(it + u);
+                    row(MarchPlain());
+                    next_row();
+                }
             }
         }
     }
@@ -901,11 +927,12 @@ static cudaError_t launch_march(const StepArgs &a, const Walls &w, int nsteps, c
         while (m.nl < m.nstrips && x0(m.nl) < edge) m.nl++;
         while (m.nl + m.nr < m.nstrips && x0(m.nstrips - 1 - m.nr) + 128 > a.g.nx - edge) m.nr++;
     }
-    // a walled unit's row takes about twice a periodic one's: half the rows (segments twice as many)
-    m.nseg = std::max(1, std::min(cap / (m.nstrips + m.nl + m.nr), a.g.ny / 2));
-    m.nsegx = std::max(1, std::min(2 * m.nseg, a.g.ny / 2));
+    // a walled unit's row takes up to three times a periodic one's: a third of the rows (4096^2 with a 32-site layer, 200
+    // steps: 5.2 ms, with half of the rows 6.1, with two thirds 7.1)
+    m.nseg = std::max(1, std::min(cap / (m.nstrips + 2 * (m.nl + m.nr)), a.g.ny / 2));
+    m.nsegx = std::max(1, std::min(3 * m.nseg, a.g.ny / 2));
     if (WL && w.kind[1] && m.nseg >= 4) {
-        const int reach = std::max(w.nlayer, 1) + K, he = std::max(reach, a.g.ny / m.nseg / 2 - (K - 1));
+        const int reach = std::max(w.nlayer, 1) + K, he = std::max(reach, a.g.ny / m.nseg / 3 - (K - 1));
         if (2 * he + (m.nseg - 2) * 2 <= a.g.ny) m.he = he;
     }
     cudaLaunchAttribute at[1];
