@@ -17,7 +17,7 @@
 //            h'_{0 gamma} = 2 w0 sigma_gamma - h_{0 gamma} + T_0,  w0 = 1 - 3 c_L^2
 //   Eq. 3 :  S = c_eff^2 (B x grad ln mu - mu j) = (c_L^2/2) S^,
 //            T_{i gamma} = -(w_i/c_L^2) S_gamma:  T_m = -(c_L^2/4) S^, T_0 = -(w0/2) S^.
-#include "lbem_internal.cuh"
+#include "site3d.cuh"
 
 namespace lbk {
 
@@ -62,70 +62,6 @@ __device__ __forceinline__ void pull3d(const PopBuf &in, const Grid &G, int row,
     }
 }
 
-struct Mom3 {
-    float sx, sy, sz, bx, by, bz;
-};
-
-__device__ __forceinline__ Mom3 moments3(const float h[21]) {
-    Mom3 m;
-    m.sx = ((h[0] + h[3]) + (h[6] + h[9])) + ((h[12] + h[15]) + h[18]);
-    m.sy = ((h[1] + h[4]) + (h[7] + h[10])) + ((h[13] + h[16]) + h[19]);
-    m.sz = ((h[2] + h[5]) + (h[8] + h[11])) + ((h[14] + h[17]) + h[20]);
-    // R_{gamma kappa} = h[(1+kappa)*3 + gamma] - h[(4+kappa)*3 + gamma]
-    m.bx = (h[10] - h[19]) - (h[8] - h[17]);   // R_yz - R_zy
-    m.by = (h[5] - h[14]) - (h[9] - h[18]);    // R_zx - R_xz
-    m.bz = (h[6] - h[15]) - (h[4] - h[13]);    // R_xy - R_yx
-    return m;
-}
-
-__device__ __forceinline__ float field3d(int comp, float cl, const Mom3 &m) {
-    switch (comp) {
-        case 0: return -cl * m.sx;
-        case 1: return -cl * m.sy;
-        case 2: return -cl * m.sz;
-        case 3: return m.bx;
-        case 4: return m.by;
-        default: return m.bz;
-    }
-}
-
-// In-place collision of one site: h[p] <- h'[p].
-__device__ __forceinline__ void collide3d(float h[21], float cl, float shx, float shy, float shz) {
-    const Mom3 m = moments3(h);
-    const float w0 = 1.f - 3.f * cl;
-    const float lx = cl * m.sx, ly = cl * m.sy, lz = cl * m.sz;
-    const float tmx = -0.25f * cl * shx, tmy = -0.25f * cl * shy, tmz = -0.25f * cl * shz;
-    const float hbx = 0.5f * m.bx, hby = 0.5f * m.by, hbz = 0.5f * m.bz;
-    // rest
-    h[0] = (2.f * w0 * m.sx - h[0]) - 0.5f * w0 * shx;
-    h[1] = (2.f * w0 * m.sy - h[1]) - 0.5f * w0 * shy;
-    h[2] = (2.f * w0 * m.sz - h[2]) - 0.5f * w0 * shz;
-    // +x: c x B = (0, -Bz, By)
-    h[3] = (lx - h[3]) + tmx;
-    h[4] = ((ly - hbz) - h[4]) + tmy;
-    h[5] = ((lz + hby) - h[5]) + tmz;
-    // +y: c x B = (Bz, 0, -Bx)
-    h[6] = ((lx + hbz) - h[6]) + tmx;
-    h[7] = (ly - h[7]) + tmy;
-    h[8] = ((lz - hbx) - h[8]) + tmz;
-    // +z: c x B = (-By, Bx, 0)
-    h[9] = ((lx - hby) - h[9]) + tmx;
-    h[10] = ((ly + hbx) - h[10]) + tmy;
-    h[11] = (lz - h[11]) + tmz;
-    // -x
-    h[12] = (lx - h[12]) + tmx;
-    h[13] = ((ly + hbz) - h[13]) + tmy;
-    h[14] = ((lz - hby) - h[14]) + tmz;
-    // -y
-    h[15] = ((lx - hbz) - h[15]) + tmx;
-    h[16] = (ly - h[16]) + tmy;
-    h[17] = ((lz + hbx) - h[17]) + tmz;
-    // -z
-    h[18] = ((lx + hby) - h[18]) + tmx;
-    h[19] = ((ly - hbx) - h[19]) + tmy;
-    h[20] = (lz - h[20]) + tmz;
-}
-
 template <bool MU>
 __global__ void __launch_bounds__(BLOCK) step3d(StepArgs a) {
     using C = Codec<LBEM_F32>;
@@ -152,10 +88,11 @@ __global__ void __launch_bounds__(BLOCK) step3d(StepArgs a) {
             float h[21];
 #pragma unroll
             for (int p = 0; p < 21; p++) h[p] = get(v[p], j);
-            const Mom3 m = moments3(h);
-            set(shx, j, m.by * get(dz, j) - m.bz * get(dy, j));
-            set(shy, j, m.bz * get(dx, j) - m.bx * get(dz, j));
-            set(shz, j, m.bx * get(dy, j) - m.by * get(dx, j));
+            float sx, sy, sz;
+            mu_source3(moments3(h), get(dx, j), get(dy, j), get(dz, j), sx, sy, sz);
+            set(shx, j, sx);
+            set(shy, j, sy);
+            set(shz, j, sz);
         }
     }
     if (a.evt.rowptr) {
@@ -167,7 +104,7 @@ __global__ void __launch_bounds__(BLOCK) step3d(StepArgs a) {
             if (ev.kind == 0) {
                 if (a.t < a.evt.nt) {
                     float jj = __ldg(a.evt.amp + (long long)ev.index * a.evt.nt + a.t);
-                    if (MU) jj *= __ldg(a.med.mu + (long long)row * G.pitch + ev.x);
+                    if (MU) jj = __fmul_rn(jj, __ldg(a.med.mu + (long long)row * G.pitch + ev.x));
                     if (ev.comp == 0) set(shx, j, get(shx, j) - jj);
                     else if (ev.comp == 1) set(shy, j, get(shy, j) - jj);
                     else set(shz, j, get(shz, j) - jj);
@@ -185,7 +122,8 @@ __global__ void __launch_bounds__(BLOCK) step3d(StepArgs a) {
         float h[21];
 #pragma unroll
         for (int p = 0; p < 21; p++) h[p] = get(v[p], j);
-        collide3d(h, get(cl, j), get(shx, j), get(shy, j), get(shz, j));
+        collide3d_free(h, get(cl, j));
+        if (MU || a.evt.rowptr) source3d(h, get(cl, j), get(shx, j), get(shy, j), get(shz, j));
 #pragma unroll
         for (int p = 0; p < 21; p++) set(v[p], j, h[p]);
     }
@@ -195,20 +133,13 @@ __global__ void __launch_bounds__(BLOCK) step3d(StepArgs a) {
     }
 }
 
-// Walls (walls.cu, in 3D): a population h_{i gamma} pulled across a wall normal to axis a is the site's own
-// h_{opp(i) gamma} times wall_sign3(kind, gamma, a): the geometric mirror of the tensor component it carries
-// (+1 when gamma == a, -1 otherwise) times +1 for PEC and -1 for PMC.
-__device__ __forceinline__ float wall_sign3(int kind, int gm, int ax) {
-    return (kind == 1 ? 1.f : -1.f) * (gm == ax ? 1.f : -1.f);
-}
-
 // One site per thread: a warp covers 32 consecutive sites of a row; the +-x
 // pulls are plain (unaligned, coalesced) loads whose overlap L1/L2 absorbs.
 // Far fewer registers than the 4-sites-per-lane kernel, so more warps per SM.
 // With WL, pulls across walls follow wall_sign3 and the absorbing layer's
 // factor fx(x) fy(y) fz(z) scales the result.
 template <bool MU, bool WL = false>
-__global__ void __launch_bounds__(BLOCK, WL ? 5 : 1) step3d_site(StepArgs a, Walls w) {
+__global__ void __launch_bounds__(BLOCK, 5) step3d_site(StepArgs a, Walls w) {
     const Grid &G = a.g;
     const int tpr = G.pitch;  // threads per row (pitch is a multiple of 32)
     const long long tid = (long long)blockIdx.x * BLOCK + threadIdx.x;
@@ -253,20 +184,19 @@ __global__ void __launch_bounds__(BLOCK, WL ? 5 : 1) step3d_site(StepArgs a, Wal
     if (MU) {
         const float dx = __ldg(a.med.dlnmu + o), dy = __ldg(a.med.dlnmu + G.plane + o),
                     dz = __ldg(a.med.dlnmu + 2 * G.plane + o);
-        const Mom3 m = moments3(h);
-        shx = m.by * dz - m.bz * dy;
-        shy = m.bz * dx - m.bx * dz;
-        shz = m.bx * dy - m.by * dx;
+        mu_source3(moments3(h), dx, dy, dz, shx, shy, shz);
     }
+    bool src = MU;
     if (a.evt.rowptr) {
         const int e0 = __ldg(a.evt.rowptr + row), e1 = __ldg(a.evt.rowptr + row + 1);
         for (int e = e0; e < e1; e++) {
             const Event ev = a.evt.ev[e];
             if (ev.x != x) continue;
             if (ev.kind == 0) {
+                src = true;
                 if (a.t < a.evt.nt) {
                     float jj = __ldg(a.evt.amp + (long long)ev.index * a.evt.nt + a.t);
-                    if (MU) jj *= __ldg(a.med.mu + o);
+                    if (MU) jj = __fmul_rn(jj, __ldg(a.med.mu + o));
                     if (ev.comp == 0) shx -= jj;
                     else if (ev.comp == 1) shy -= jj;
                     else shz -= jj;
@@ -276,7 +206,8 @@ __global__ void __launch_bounds__(BLOCK, WL ? 5 : 1) step3d_site(StepArgs a, Wal
             }
         }
     }
-    collide3d(h, cl, shx, shy, shz);
+    collide3d_free(h, cl);
+    if (src) source3d(h, cl, shx, shy, shz);  // (S^ = 0 would add -0)
     float *out = static_cast<float *>(a.out.data);
     if (WL && (w.fx || w.fy || w.fz)) {
         const float f = __fmul_rn(__fmul_rn(w.fx ? w.fx[x] : 1.f, w.fy ? w.fy[y] : 1.f), w.fz ? w.fz[z] : 1.f);

@@ -211,6 +211,12 @@ constexpr int MARCH_MIN_STEPS = 3;
 static bool march_ok(const lbem_t *h) {
     return h->tblock == 2 && !h->tb_shape_set && multi_step_base(h) && !(h->disp && h->aniso);
 }
+// 3D: triples of steps by the marching kernel (march3d.cu) where several steps per launch are the default, with uniform
+// mu and the one-site-per-thread launch shapes; offsets in a plane must fit 32 bits.
+static bool march3_ok(const lbem_t *h) {
+    return h->tblock == 2 && h->dim == 3 && h->variant >= 1 && !h->has_mu && h->grid.plane < (1LL << 31) &&
+           march_3d_pays(h->grid, h->bc[0] || h->bc[1] || h->bc[2]);
+}
 static int steps_per_launch(const lbem_t *h) { return three_step_ok(h) ? 3 : two_step_ok(h) ? 2 : 1; }
 
 // Enqueue nsteps steps starting from buffer `cur` at time t0: triples (pairs) of steps with the three-step
@@ -291,6 +297,17 @@ static cudaError_t enqueue_steps(const lbem_t *h, int cur, long long t0, int nst
             }
             if (e != cudaSuccess) return e;
             cur ^= 1;
+        }
+    }
+    if (march3_ok(h)) {
+        const int K = MARCH3_STEPS, launches = (nsteps - n) / K;
+        if (launches > 0) {
+            StepArgs a = step_args(h, cur);
+            a.t = t0 + n;
+            cudaError_t e = launch_march_3d(a, handle_walls(h), launches, h->stream);
+            if (e != cudaSuccess) return e;
+            n += K * launches;
+            cur ^= launches & 1;
         }
     }
     for (; n < nsteps; n++) {

@@ -589,6 +589,11 @@ cudaError_t launch_march_2d_an(const StepArgs &a, const Walls &w, int nsteps, cu
 cudaError_t launch_march_2d_mu(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches);
 cudaError_t launch_march_2d_pole(const StepArgs &a, int nsteps, cudaStream_t s, int *launches);
 cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaStream_t s, int *launches);
+// 3D, MARCH3_STEPS steps per launch, uniform mu, walls and layers included (march3d.cu): nlaunch launches from a.in,
+// alternating between the two buffers
+constexpr int MARCH3_STEPS = 3;
+bool march_3d_pays(const Grid &g, bool walls);  // whether it takes less time than single steps on this grid
+cudaError_t launch_march_3d(const StepArgs &a, const Walls &w, int nlaunch, cudaStream_t s);
 int ss2_nshapes();  // strip streaming (sstream.cu): two steps per launch, FP32, uniform mu
 cudaError_t launch_step_2d_ss2(const StepArgs &a, int shape, cudaStream_t s);
 cudaError_t launch_step_2d_ss2_an(const StepArgs &a, cudaStream_t s);  // anisotropic medium, no pole

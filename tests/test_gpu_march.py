@@ -90,3 +90,31 @@ def test_march_16bit_equals_launches_of_two_steps(lbem, shape, storage):
         ref = _run(p, calls, steps_per_pass=2, shape=0, storage=storage)
         for a, b in zip(_run(p, calls, storage=storage), ref):
             np.testing.assert_array_equal(a, b, err_msg=f"{storage} {shape}, calls {calls}")
+
+
+# grids that the rule on sizes gives to the 3D kernel (28 x 16 columns a tile, segments of the planes): one tile, a tile
+# that is a column or a row too wide, one plane a segment, an odd remainder of everything, several waves of blocks
+@pytest.mark.parametrize("walls", [False, True])
+@pytest.mark.parametrize("shape", [(220, 16, 28), (64, 64, 85), (90, 81, 84), (3, 250, 460), (75, 61, 90),
+                                   (131, 119, 131)])
+def test_march_3d_is_bitwise_identical_to_single_steps(lbem, shape, walls):
+    nsteps = 14
+    eps, _ = W.random_medium(shape, 5, 1.0)
+    p = W.Problem("march3", 3, shape, eps, None, nsteps)
+    p.E0, p.B0 = W.random_fields(shape, 6, 0.3)
+    nz, ny, nx = shape
+    n = nz * ny * nx
+    rng = np.random.default_rng(7)
+    corners = [0, nx - 1, (ny - 1) * nx, n - 1, min(nx - 1, 28), (nz // 2 * ny + min(ny - 1, 16)) * nx]
+    p.src_site = np.unique(np.concatenate([corners, rng.integers(0, n, 4)])).astype(np.int64)
+    p.src_comp = rng.integers(0, 3, p.src_site.size).astype(np.int32)
+    p.src_amp = rng.standard_normal((p.src_site.size, nsteps))
+    p.rec_site = np.concatenate([corners, rng.integers(0, n, 24)]).astype(np.int64)
+    p.rec_comp = np.resize(np.arange(6, dtype=np.int32), p.rec_site.size)
+    if walls:
+        p.bc, p.layer, p.gamma_max = (1, 2, 1), min(3, min(shape) // 2), 0.2
+    ref = _run(p, [nsteps], steps_per_pass=1)
+    for calls in ([nsteps], [3, 4, 5, 2]):
+        for graphs in (False, True):
+            for a, b in zip(ref, _run(p, calls, graphs=graphs)):
+                np.testing.assert_array_equal(a, b)
