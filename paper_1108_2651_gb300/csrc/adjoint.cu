@@ -22,10 +22,20 @@
 // B_y = g_1 - g_3; 3D: B = sum_i g_i x c_i).  Finally
 //   dL/d eps_r = dL/dc_L^2 * dc_L^2/d eps_r = -dL/dc_L^2 * c_L^2 / eps_r.
 //
-// Checkpointing: lbem_forward_record keeps the state every K steps; the
-// backward pass recomputes one segment of at most K states at a time (kept
-// in device memory) and runs the adjoint kernel backwards through it.  The
-// gradient is accumulated over time steps in FP64; each step's contribution at
+// Of a state g^t the adjoint needs sigma only: 3 words a site in 3D against the
+// state's 21.  In 3D the forward kernels write it as they step (the sums are
+// those of the collision), and lambda is stored by opposite directions, so that
+// its transposed streaming is the forward step's pull and the kernel of several
+// steps per launch (march3d.cu) serves both.  lbem_forward_record keeps every
+// step's sigma where that takes no more memory than states every K steps and a
+// segment of K states would (3 nsteps <= 21 (nsteps / K + K)); the backward pass
+// is then one sweep.  Else, and in 2D (a state is 5 words, sigma 1), it
+// keeps the state every K steps, and the backward pass recomputes one segment
+// of at most K steps at a time: its sigmas in 3D, its states in 2D.  40 steps of
+// 96^3 with K = 10 recorded and gone back: 5.23 ms with states kept and
+// recomputed, buffers allocated each time and single steps; 2.7 ms with sigmas
+// and the last run's buffers; 2.3 ms with three steps per launch (18.5 us a step
+// forward, of L2 bandwidth as the steps themselves).  The gradient is accumulated over time steps in FP64; each step's contribution at
 // a site is formed in FP32, like the rest of the arithmetic (GB300's FP64 rate
 // is a small fraction of its FP32 rate, and the per-site FP64 products had made
 // the adjoint step compute-bound).
@@ -34,28 +44,49 @@
 #include <algorithm>
 #include <vector>
 
-#include "lbem_internal.cuh"
+#include "site3d.cuh"
 
 namespace lbk {
 
+// A run's buffers; the next run of the handle takes them over as far as they are large enough.
 struct AdjointState {
     int nsteps = 0, every = 0, ncp = 0;
     long long t0 = 0;
-    size_t state_floats = 0;
+    size_t state_floats = 0, sig_floats = 0;
+    bool all = false;       // 3D: seg holds every step's sigma, and there are no checkpoints
     float *cps = nullptr;   // [ncp][state]
-    float *seg = nullptr;   // [every][state]
+    float *seg = nullptr;   // 2D: [every][state]; 3D: sigma of every step, or of a segment's: [..][3][plane]
+    float *work = nullptr;  // 3D with checkpoints: [2][state], the states recomputed
     float *lam = nullptr;   // [2][state]
     double *gcl = nullptr;  // [plane]
     float *cot = nullptr;   // [nrec][nsteps]
     float *gout = nullptr;  // [nsite] staging for host outputs
     double *gcl_out = nullptr;
+    size_t cps_cap = 0, seg_cap = 0, work_cap = 0, lam_cap = 0, gcl_cap = 0, cot_cap = 0;  // elements
 };
+
+// Makes p hold at least need elements (its contents are lost when it has to grow).
+template <class T>
+static bool ensure(T *&p, size_t &cap, size_t need) {
+    if (cap >= need) return true;
+    cudaFree(p);
+    p = nullptr;
+    cap = 0;
+    if (cudaMalloc((void **)&p, need * sizeof(T)) != cudaSuccess) {
+        cudaGetLastError();
+        p = nullptr;
+        return false;
+    }
+    cap = need;
+    return true;
+}
 
 void adjoint_free(lbem_t *h) {
     if (!h || !h->adj) return;
     AdjointState *a = h->adj;
     cudaFree(a->cps);
     cudaFree(a->seg);
+    cudaFree(a->work);
     cudaFree(a->lam);
     cudaFree(a->gcl);
     cudaFree(a->cot);
@@ -188,144 +219,11 @@ __global__ void __launch_bounds__(BLOCK) adjoint2d(AdjArgs a) {
 }
 
 // ------------------------------------------------------------------ 3D
-__global__ void __launch_bounds__(BLOCK) adjoint3d(AdjArgs a) {
-    const Grid &G = a.g;
-    const int lane = threadIdx.x & 31;
-    const long long wg = ((long long)blockIdx.x * BLOCK + threadIdx.x) >> 5;
-    const int wpr = G.nchunk_pad >> 5;
-    const int row = (int)(wg / wpr);
-    const int c = (int)(wg - (long long)row * wpr) * 32 + lane;
-    if (row >= G.nrows) return;
-    const bool active = c < G.nchunk;
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int z = row / G.ny, y = row - z * G.ny;
-    const int rym = z * G.ny + (y == 0 ? G.ny - 1 : y - 1), ryp = z * G.ny + (y == G.ny - 1 ? 0 : y + 1);
-    const int rzm = (z == 0 ? G.nz - 1 : z - 1) * G.ny + y, rzp = (z == G.nz - 1 ? 0 : z + 1) * G.ny + y;
-    const float *L = a.lam_in;
-    const float *S = static_cast<const float *>(a.state.data);
-    float4 m[21];
-    float4 sg[3];
-#pragma unroll
-    for (int gm = 0; gm < 3; gm++) {
-        // mu_{i gamma}(y) = lambda_{i gamma}(y + c_i)
-        m[0 + gm] = active ? f4(L, G.plane, 0 + gm, row, G.pitch, c) : z4;
-        m[3 + gm] = xshift(L, G.plane, 3 + gm, row, G, c, lane, +1, active);
-        m[6 + gm] = active ? f4(L, G.plane, 6 + gm, ryp, G.pitch, c) : z4;
-        m[9 + gm] = active ? f4(L, G.plane, 9 + gm, rzp, G.pitch, c) : z4;
-        m[12 + gm] = xshift(L, G.plane, 12 + gm, row, G, c, lane, -1, active);
-        m[15 + gm] = active ? f4(L, G.plane, 15 + gm, rym, G.pitch, c) : z4;
-        m[18 + gm] = active ? f4(L, G.plane, 18 + gm, rzm, G.pitch, c) : z4;
-        // sigma_gamma of g^t(y), g_i(y) = P_i(y - c_i)
-        float4 acc = active ? f4(S, G.plane, 0 + gm, row, G.pitch, c) : z4;
-        const float4 s1 = xshift(S, G.plane, 3 + gm, row, G, c, lane, -1, active);
-        const float4 s4 = xshift(S, G.plane, 12 + gm, row, G, c, lane, +1, active);
-        const float4 s2 = active ? f4(S, G.plane, 6 + gm, rym, G.pitch, c) : z4;
-        const float4 s3 = active ? f4(S, G.plane, 9 + gm, rzm, G.pitch, c) : z4;
-        const float4 s5 = active ? f4(S, G.plane, 15 + gm, ryp, G.pitch, c) : z4;
-        const float4 s6 = active ? f4(S, G.plane, 18 + gm, rzp, G.pitch, c) : z4;
-        for (int j = 0; j < 4; j++)
-            set(acc, j, ((get(acc, j) + get(s1, j)) + (get(s2, j) + get(s3, j))) + ((get(s4, j) + get(s5, j)) + get(s6, j)));
-        sg[gm] = acc;
-    }
-    if (!active) return;
-    const float4 cl = f4(a.cL2, 0, 0, row, G.pitch, c);
-    float4 jv[3] = {z4, z4, z4};
-    float dg[4] = {0.f, 0.f, 0.f, 0.f};  // this step's contribution, FP32; accumulated over steps in FP64
-    // receivers add to lambda after M^T; collect them first per site
-    float4 recE[3] = {z4, z4, z4}, recB[3] = {z4, z4, z4};
-    if (a.evt.rowptr) {
-        const int e0 = __ldg(a.evt.rowptr + row), e1 = __ldg(a.evt.rowptr + row + 1);
-        for (int e = e0; e < e1; e++) {
-            const Event ev = a.evt.ev[e];
-            if ((ev.x >> 2) != c) continue;
-            const int j = ev.x & 3;
-            if (ev.kind == 0) {
-                if (a.t < a.evt.nt) set(jv[ev.comp], j, get(jv[ev.comp], j) + __ldg(a.evt.amp + (long long)ev.index * a.evt.nt + a.t));
-            } else {
-                const long long n = a.t - a.t0;
-                if (n < 0 || n >= a.nsteps || a.t >= a.evt.cap) continue;
-                const float r = __ldg(a.cot + (long long)ev.index * a.nsteps + n);
-                if (ev.comp < 3) set(recE[ev.comp], j, get(recE[ev.comp], j) + r);
-                else set(recB[ev.comp - 3], j, get(recB[ev.comp - 3], j) + r);
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-        float h[21];
-#pragma unroll
-        for (int p = 0; p < 21; p++) h[p] = get(m[p], j);
-        const float q = get(cl, j), w0 = 1.f - 3.f * q;
-        float mv[3], nu[3];
-        for (int gm = 0; gm < 3; gm++) {
-            mv[gm] = ((h[3 + gm] + h[6 + gm]) + (h[9 + gm] + h[12 + gm])) + (h[15 + gm] + h[18 + gm]);
-            nu[gm] = w0 * h[gm] + 0.5f * q * mv[gm];
-        }
-        // V = sum_i mu_i x c_i, the same contraction that reads B from h
-        const float vx = (h[10] - h[19]) - (h[8] - h[17]);
-        const float vy = (h[5] - h[14]) - (h[9] - h[18]);
-        const float vz = (h[6] - h[15]) - (h[4] - h[13]);
-        const float hx = 0.5f * vx, hy = 0.5f * vy, hz = 0.5f * vz;
-        const float Lx = 2.f * nu[0], Ly = 2.f * nu[1], Lz = 2.f * nu[2];
-        float o[21];
-        o[0] = Lx - h[0];
-        o[1] = Ly - h[1];
-        o[2] = Lz - h[2];
-        o[3] = Lx - h[3];             // +x: c x V = (0, -Vz, Vy)
-        o[4] = (Ly - hz) - h[4];
-        o[5] = (Lz + hy) - h[5];
-        o[6] = (Lx + hz) - h[6];      // +y: (Vz, 0, -Vx)
-        o[7] = Ly - h[7];
-        o[8] = (Lz - hx) - h[8];
-        o[9] = (Lx - hy) - h[9];      // +z: (-Vy, Vx, 0)
-        o[10] = (Ly + hx) - h[10];
-        o[11] = Lz - h[11];
-        o[12] = Lx - h[12];           // -x
-        o[13] = (Ly + hz) - h[13];
-        o[14] = (Lz - hy) - h[14];
-        o[15] = (Lx - hz) - h[15];    // -y
-        o[16] = Ly - h[16];
-        o[17] = (Lz + hx) - h[17];
-        o[18] = (Lx + hy) - h[18];    // -z
-        o[19] = (Ly - hx) - h[19];
-        o[20] = Lz - h[20];
-        float d = 0.f;
-        for (int gm = 0; gm < 3; gm++) {
-            const float s = get(sg[gm], j);
-            d += s * mv[gm] - 6.f * (s * h[gm]);
-            d += get(jv[gm], j) * (0.25f * mv[gm] - 1.5f * h[gm]);
-            // E_gamma = -c_L^2 sigma_gamma receivers
-            const float rE = get(recE[gm], j);
-            if (rE != 0.f) {
-                for (int i = 0; i < 7; i++) o[3 * i + gm] -= q * rE;
-                d -= s * rE;
-            }
-        }
-        // B receivers: B_nu = sum_i (g_i x c_i)_nu = eps_{gamma kappa nu} c_{i kappa} g_{i gamma}
-        const float bx = get(recB[0], j), by = get(recB[1], j), bz = get(recB[2], j);
-        if (bx != 0.f || by != 0.f || bz != 0.f) {
-            // d B_x/d h: +h[10](+z,y) -h[19](-z,y) -h[8](+y,z) +h[17](-y,z)
-            o[10] += bx; o[19] -= bx; o[8] -= bx; o[17] += bx;
-            o[5] += by; o[14] -= by; o[9] -= by; o[18] += by;
-            o[6] += bz; o[15] -= bz; o[4] -= bz; o[13] += bz;
-        }
-#pragma unroll
-        for (int p = 0; p < 21; p++) set(m[p], j, o[p]);
-        dg[j] = d;
-    }
-    for (int j = 0; j < 4; j++) {
-        const int x = 4 * c + j;
-        if (x < G.nx) a.gcl[(long long)row * G.pitch + x] += (double)dg[j];
-    }
-    PopBuf ob{a.lam_out, nullptr, G.plane, 0, G.pitch, 0};
-#pragma unroll
-    for (int p = 0; p < 21; p++) Codec<LBEM_F32>::store4(ob, p, row, c, m[p]);
-}
-
-// One site per thread (48-64 registers instead of 170): the same update as adjoint3d.  The FP64
-// gradient accumulator is loaded with the other operands, at the top, so its latency overlaps theirs.
+// One site per thread; the same update as the kernel of several steps per launch.  lambda is stored by opposite
+// directions, so mu is pulled as the forward step pulls.  The FP64 gradient accumulator is loaded with the other operands,
+// at the top, so its latency overlaps theirs.  MINB = 5 caps the registers (handle variant 2).
 template <int MINB>
-__global__ void __launch_bounds__(BLOCK, MINB) adjoint3d_site(AdjArgs a) {
+__global__ void __launch_bounds__(BLOCK, MINB) adjoint3d_site(AdjArgs a, const float *sig) {
     const Grid &G = a.g;
     const long long tid = (long long)blockIdx.x * BLOCK + threadIdx.x;
     const int row = (int)(tid / G.pitch);
@@ -335,108 +233,33 @@ __global__ void __launch_bounds__(BLOCK, MINB) adjoint3d_site(AdjArgs a) {
     const int rym = z * G.ny + (y == 0 ? G.ny - 1 : y - 1), ryp = z * G.ny + (y == G.ny - 1 ? 0 : y + 1);
     const int rzm = (z == 0 ? G.nz - 1 : z - 1) * G.ny + y, rzp = (z == G.nz - 1 ? 0 : z + 1) * G.ny + y;
     const int xm = x == 0 ? G.nx - 1 : x - 1, xp = x == G.nx - 1 ? 0 : x + 1;
-    const float *L = a.lam_in;
-    const float *S = static_cast<const float *>(a.state.data);
-    auto at = [&](const float *b, int p, int r, int xx) { return __ldg(b + p * G.plane + (long long)r * G.pitch + xx); };
+    auto at = [&](int p, int r, int xx) { return __ldg(a.lam_in + p * G.plane + (long long)r * G.pitch + xx); };
     const long long o = (long long)row * G.pitch + x;
     const double gacc = a.gcl[o];
-    float h[21], sg[3];
+    float v[21], sg[3];
 #pragma unroll
-    for (int gm = 0; gm < 3; gm++) {
-        // mu_{i gamma}(y) = lambda_{i gamma}(y + c_i)
-        h[0 + gm] = at(L, 0 + gm, row, x);
-        h[3 + gm] = at(L, 3 + gm, row, xp);
-        h[6 + gm] = at(L, 6 + gm, ryp, x);
-        h[9 + gm] = at(L, 9 + gm, rzp, x);
-        h[12 + gm] = at(L, 12 + gm, row, xm);
-        h[15 + gm] = at(L, 15 + gm, rym, x);
-        h[18 + gm] = at(L, 18 + gm, rzm, x);
-        // sigma_gamma of g^t(y), g_i(y) = P_i(y - c_i)
-        sg[gm] = ((at(S, 0 + gm, row, x) + at(S, 3 + gm, row, xm)) + (at(S, 6 + gm, rym, x) + at(S, 9 + gm, rzm, x))) +
-                 ((at(S, 12 + gm, row, xp) + at(S, 15 + gm, ryp, x)) + at(S, 18 + gm, rzp, x));
+    for (int g = 0; g < 3; g++) {
+        v[0 + g] = at(0 + g, row, x);
+        v[3 + g] = at(3 + g, row, xm);
+        v[6 + g] = at(6 + g, rym, x);
+        v[9 + g] = at(9 + g, rzm, x);
+        v[12 + g] = at(12 + g, row, xp);
+        v[15 + g] = at(15 + g, ryp, x);
+        v[18 + g] = at(18 + g, rzp, x);
+        sg[g] = __ldg(sig + g * G.plane + o);
     }
-    const float q = __ldg(a.cL2 + o), w0 = 1.f - 3.f * q;
-    float jv[3] = {0.f, 0.f, 0.f}, rE[3] = {0.f, 0.f, 0.f}, rB[3] = {0.f, 0.f, 0.f};
+    const float q = __ldg(a.cL2 + o);
+    AdjEvents3 ev = {};
     if (a.evt.rowptr) {
         const int e0 = __ldg(a.evt.rowptr + row), e1 = __ldg(a.evt.rowptr + row + 1);
         for (int e = e0; e < e1; e++) {
-            const Event ev = a.evt.ev[e];
-            if (ev.x != x) continue;
-            if (ev.kind == 0) {
-                if (a.t < a.evt.nt) {
-                    const float jj = __ldg(a.evt.amp + (long long)ev.index * a.evt.nt + a.t);
-                    if (ev.comp == 0) jv[0] += jj;
-                    else if (ev.comp == 1) jv[1] += jj;
-                    else jv[2] += jj;
-                }
-            } else {
-                const long long n = a.t - a.t0;
-                if (n < 0 || n >= a.nsteps || a.t >= a.evt.cap) continue;
-                const float r = __ldg(a.cot + (long long)ev.index * a.nsteps + n);
-                switch (ev.comp) {
-                    case 0: rE[0] += r; break;
-                    case 1: rE[1] += r; break;
-                    case 2: rE[2] += r; break;
-                    case 3: rB[0] += r; break;
-                    case 4: rB[1] += r; break;
-                    default: rB[2] += r; break;
-                }
-            }
+            const Event k = a.evt.ev[e];
+            if (k.x == x) adjoint3_event(ev, k, a.evt, a.cot, a.nsteps, a.t, a.t0);
         }
     }
-    float mv[3], nu[3];
+    a.gcl[o] = gacc + (double)adjoint3_site(v, sg, q, ev);
 #pragma unroll
-    for (int gm = 0; gm < 3; gm++) {
-        mv[gm] = ((h[3 + gm] + h[6 + gm]) + (h[9 + gm] + h[12 + gm])) + (h[15 + gm] + h[18 + gm]);
-        nu[gm] = w0 * h[gm] + 0.5f * q * mv[gm];
-    }
-    const float vx = (h[10] - h[19]) - (h[8] - h[17]);
-    const float vy = (h[5] - h[14]) - (h[9] - h[18]);
-    const float vz = (h[6] - h[15]) - (h[4] - h[13]);
-    const float hx = 0.5f * vx, hy = 0.5f * vy, hz = 0.5f * vz;
-    const float Lx = 2.f * nu[0], Ly = 2.f * nu[1], Lz = 2.f * nu[2];
-    float d = 0.f;  // this step's contribution, FP32; accumulated over steps in FP64
-#pragma unroll
-    for (int gm = 0; gm < 3; gm++) {
-        d += sg[gm] * mv[gm] - 6.f * (sg[gm] * h[gm]);
-        d += jv[gm] * (0.25f * mv[gm] - 1.5f * h[gm]);
-    }
-    float out[21];
-    out[0] = Lx - h[0];
-    out[1] = Ly - h[1];
-    out[2] = Lz - h[2];
-    out[3] = Lx - h[3];
-    out[4] = (Ly - hz) - h[4];
-    out[5] = (Lz + hy) - h[5];
-    out[6] = (Lx + hz) - h[6];
-    out[7] = Ly - h[7];
-    out[8] = (Lz - hx) - h[8];
-    out[9] = (Lx - hy) - h[9];
-    out[10] = (Ly + hx) - h[10];
-    out[11] = Lz - h[11];
-    out[12] = Lx - h[12];
-    out[13] = (Ly + hz) - h[13];
-    out[14] = (Lz - hy) - h[14];
-    out[15] = (Lx - hz) - h[15];
-    out[16] = Ly - h[16];
-    out[17] = (Lz + hx) - h[17];
-    out[18] = (Lx + hy) - h[18];
-    out[19] = (Ly - hx) - h[19];
-    out[20] = Lz - h[20];
-#pragma unroll
-    for (int gm = 0; gm < 3; gm++)
-        if (rE[gm] != 0.f) {
-            for (int i = 0; i < 7; i++) out[3 * i + gm] -= q * rE[gm];
-            d -= sg[gm] * rE[gm];
-        }
-    if (rB[0] != 0.f || rB[1] != 0.f || rB[2] != 0.f) {
-        out[10] += rB[0]; out[19] -= rB[0]; out[8] -= rB[0]; out[17] += rB[0];
-        out[5] += rB[1]; out[14] -= rB[1]; out[9] -= rB[1]; out[18] += rB[1];
-        out[6] += rB[2]; out[15] -= rB[2]; out[4] -= rB[2]; out[13] += rB[2];
-    }
-    a.gcl[o] = gacc + (double)d;
-#pragma unroll
-    for (int p = 0; p < 21; p++) __stcs(a.lam_out + p * G.plane + o, out[p]);
+    for (int p = 0; p < 21; p++) __stcs(a.lam_out + p * G.plane + o, v[p]);
 }
 
 // dL/d eps_r = -dL/dc_L^2 * c_L^2 / eps_r with eps_r = (D-1) c_ref^2 / c_L^2 (mu = 1), dense output.
@@ -454,23 +277,67 @@ __global__ void adjoint_finish(Grid G, const double *gcl, const float *cL2, int 
 }
 
 static cudaError_t launch_adjoint(const lbem_t *h, const AdjArgs &a) {
-    if (h->dim == 3 && h->variant >= 1) {  // the one-site-per-thread shapes, as the forward kernel
-        const long long threads = (long long)a.g.nrows * a.g.pitch;
-        const unsigned blocks = (unsigned)((threads + BLOCK - 1) / BLOCK);
-        if (h->variant == 2) adjoint3d_site<5><<<blocks, BLOCK, 0, h->stream>>>(a);  // registers capped
-        else adjoint3d_site<1><<<blocks, BLOCK, 0, h->stream>>>(a);
-        return cudaGetLastError();
-    }
     const long long warps = (long long)a.g.nrows * (a.g.nchunk_pad / 32);
-    const unsigned blocks = (unsigned)((warps * 32 + BLOCK - 1) / BLOCK);
-    if (h->dim == 2) adjoint2d<<<blocks, BLOCK, 0, h->stream>>>(a);
-    else adjoint3d<<<blocks, BLOCK, 0, h->stream>>>(a);
+    adjoint2d<<<(unsigned)((warps * 32 + BLOCK - 1) / BLOCK), BLOCK, 0, h->stream>>>(a);
     return cudaGetLastError();
 }
 
-static cudaError_t launch_fwd(const lbem_t *h, const StepArgs &a) {
-    if (h->dim == 2) return launch_step_2d(a, h->storage, false, h->variant, h->stream);
-    return launch_step_3d(a, false, h->variant, h->stream);
+// 3D: n steps from a.in at a.t, alternating between a.in and a.out, their sigmas to sig (unless null); *launches of them.
+static cudaError_t forward_3d(const lbem_t *h, StepArgs a, int n, float *sig, int *launches) {
+    const int groups = march3_ok(h, true) ? n / MARCH3_STEPS : 0, done = groups * MARCH3_STEPS;
+    if (groups) {
+        Adj3 r;
+        r.sig = sig;
+        const cudaError_t e = sig ? launch_march_3d_adj(a, r, true, groups, h->stream)
+                                  : launch_march_3d(a, Walls(), groups, h->stream);
+        if (e != cudaSuccess) return e;
+        if (groups & 1) std::swap(a.in, a.out);
+        a.t += done;
+    }
+    for (int k = done; k < n; k++) {
+        const cudaError_t e = launch_step_3d(a, false, h->variant, h->stream, nullptr,
+                                             sig ? sig + (size_t)k * 3 * a.g.plane : nullptr);
+        if (e != cudaSuccess) return e;
+        std::swap(a.in, a.out);
+        a.t++;
+    }
+    *launches = groups + n - done;
+    return cudaSuccess;
+}
+
+// 3D: n adjoint steps back from a.t, lambda from a.in, alternating with a.out; adj.sig: the sigma of step a.t.
+static cudaError_t adjoint_sigma(const lbem_t *h, StepArgs a, Adj3 adj, int n, int *launches) {
+    const int groups = march3_ok(h, true) ? n / MARCH3_STEPS : 0, done = groups * MARCH3_STEPS;
+    if (groups) {
+        const cudaError_t e = launch_march_3d_adj(a, adj, false, groups, h->stream);
+        if (e != cudaSuccess) return e;
+        if (groups & 1) std::swap(a.in, a.out);
+        a.t -= done;
+        adj.sig -= (long long)done * 3 * a.g.plane;
+    }
+    for (int k = done; k < n; k++) {
+        AdjArgs q;
+        q.g = a.g;
+        q.lam_in = static_cast<const float *>(a.in.data);
+        q.lam_out = static_cast<float *>(a.out.data);
+        q.cL2 = a.med.cL2;
+        q.gcl = adj.gcl;
+        q.evt = a.evt;
+        q.cot = adj.cot;
+        q.nsteps = adj.nsteps;
+        q.t = a.t;
+        q.t0 = adj.t0;
+        const unsigned blocks = (unsigned)(((long long)a.g.nrows * a.g.pitch + BLOCK - 1) / BLOCK);
+        if (h->variant == 2) adjoint3d_site<5><<<blocks, BLOCK, 0, h->stream>>>(q, adj.sig);
+        else adjoint3d_site<1><<<blocks, BLOCK, 0, h->stream>>>(q, adj.sig);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        std::swap(a.in, a.out);
+        a.t--;
+        adj.sig -= 3 * a.g.plane;
+    }
+    *launches = groups + n - done;
+    return cudaSuccess;
 }
 
 bool is_device_ptr(const void *p);
@@ -491,28 +358,51 @@ lbem_status lbem_forward_record(lbem_t *h, int nsteps, int every) {
     if (h->walls()) return fail(LBEM_ERR_STATE, "lbem_forward_record: the adjoint supports periodic boundaries only");
     if (h->disp || h->aniso)
         return fail(LBEM_ERR_STATE, "lbem_forward_record: the adjoint supports non-dispersive isotropic media only");
-    adjoint_free(h);
-    AdjointState *A = new AdjointState();
-    h->adj = A;
+    const size_t state = (size_t)h->npop * h->grid.plane, sig = 3 * (size_t)h->grid.plane;
+    every = std::min(every, nsteps);
+    const int ncp = (nsteps + every - 1) / every;
+    bool all = h->dim == 3 && sig * nsteps <= state * (ncp + every);
+    if (h->adj) {  // the last run's buffers serve again if they are of this run's size (up to twice that)
+        const size_t cap = all ? h->adj->seg_cap : h->adj->cps_cap, need = all ? sig * nsteps : state * ncp;
+        if (h->adj->all != all || cap < need || cap > 2 * need) adjoint_free(h);
+    }
+    if (!h->adj) h->adj = new AdjointState();
+    AdjointState *A = h->adj;
+    all = all && ensure(A->seg, A->seg_cap, sig * nsteps);
     A->nsteps = nsteps;
-    A->every = std::min(every, nsteps);
-    A->ncp = (nsteps + A->every - 1) / A->every;
+    A->every = every;
+    A->ncp = ncp;
     A->t0 = h->t;
-    A->state_floats = (size_t)h->npop * h->grid.plane;
-    const size_t sb = A->state_floats * sizeof(float);
-    if (cudaMalloc((void **)&A->cps, sb * A->ncp) != cudaSuccess) {
-        cudaGetLastError();
+    A->state_floats = state;
+    A->sig_floats = sig;
+    A->all = all;
+    if (!A->all && !ensure(A->cps, A->cps_cap, A->state_floats * A->ncp)) {
         adjoint_free(h);
         return fail(LBEM_ERR_NOMEM, "lbem_forward_record: no room for the checkpoints");
     }
+    if (A->all) {
+        int launches = 0;
+        LBEM_CUDA(forward_3d(h, step_args(h, h->cur), nsteps, A->seg, &launches));
+        h->cur ^= launches & 1;
+        h->t += nsteps;
+        return LBEM_OK;
+    }
+    const size_t sb = A->state_floats * sizeof(float);
     for (int n = 0; n < nsteps; n++) {
         if (n % A->every == 0)
             LBEM_CUDA(cudaMemcpyAsync(A->cps + (size_t)(n / A->every) * A->state_floats, h->buf[h->cur].data, sb,
                                       cudaMemcpyDeviceToDevice, h->stream));
         StepArgs a = step_args(h, h->cur);
-        LBEM_CUDA(launch_fwd(h, a));
-        h->cur ^= 1;
-        h->t++;
+        int steps = 1, launches = 1;
+        if (h->dim == 3) {
+            steps = std::min(A->every, nsteps - n);
+            LBEM_CUDA(forward_3d(h, a, steps, nullptr, &launches));
+            n += steps - 1;
+        } else {
+            LBEM_CUDA(launch_step_2d(a, h->storage, false, h->variant, h->stream));
+        }
+        h->cur ^= launches & 1;
+        h->t += steps;
     }
     return LBEM_OK;
 }
@@ -525,28 +415,51 @@ lbem_status lbem_adjoint(lbem_t *h, const float *trace_cot, float *grad_eps, dou
         return fail(LBEM_ERR_STATE, "lbem_adjoint: receiver capacity shorter than the recorded run");
     const size_t sb = A->state_floats * sizeof(float);
     const Grid &G = h->grid;
-    if (!A->seg) {
-        cudaError_t e = cudaMalloc((void **)&A->seg, sb * A->every);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&A->lam, 2 * sb);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&A->gcl, sizeof(double) * G.plane);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(LBEM_ERR_NOMEM, "lbem_adjoint: no room for the segment and adjoint buffers");
-        }
-    }
+    const bool d3 = h->dim == 3;
+    const size_t seg = A->all ? A->sig_floats * A->nsteps : (d3 ? A->sig_floats : A->state_floats) * A->every;
+    if (!ensure(A->lam, A->lam_cap, 2 * A->state_floats) || !ensure(A->gcl, A->gcl_cap, (size_t)G.plane) ||
+        !ensure(A->seg, A->seg_cap, seg) || (d3 && !A->all && !ensure(A->work, A->work_cap, 2 * A->state_floats)))
+        return fail(LBEM_ERR_NOMEM, "lbem_adjoint: no room for the segment and adjoint buffers");
     const size_t ncot = (size_t)h->nrec * A->nsteps;
-    cudaFree(A->cot);
-    A->cot = nullptr;
     if (ncot) {
         if (!trace_cot) return fail(LBEM_ERR_ARG, "lbem_adjoint: trace_cot is NULL but receivers are set");
-        LBEM_CUDA(cudaMalloc((void **)&A->cot, ncot * sizeof(float)));
+        if (!ensure(A->cot, A->cot_cap, ncot)) return fail(LBEM_ERR_CUDA, "lbem_adjoint: no room for the cotangents");
         LBEM_CUDA(cudaMemcpyAsync(A->cot, trace_cot, ncot * sizeof(float), cudaMemcpyDefault, h->stream));
     }
-    LBEM_CUDA(cudaMemsetAsync(A->lam, 0, 2 * sb, h->stream));
+    LBEM_CUDA(cudaMemsetAsync(A->lam, 0, sb, h->stream));  // lambda of the end
     LBEM_CUDA(cudaMemsetAsync(A->gcl, 0, sizeof(double) * G.plane, h->stream));
     int lc = 0;  // lam[lc] holds lambda^{t+1}
     StepArgs base = step_args(h, 0);
-    for (int k = A->ncp - 1; k >= 0; k--) {
+    if (d3) {
+        const int nseg = A->all ? 1 : A->ncp;
+        for (int k = nseg - 1; k >= 0; k--) {
+            const int n0 = k * A->every, len = A->all ? A->nsteps : std::min(A->every, A->nsteps - n0);
+            int launches = 0;
+            if (!A->all) {  // recompute the segment's sigmas (sources on, no trace writes)
+                StepArgs a = base;
+                LBEM_CUDA(cudaMemcpyAsync(A->work, A->cps + (size_t)k * A->state_floats, sb, cudaMemcpyDeviceToDevice,
+                                          h->stream));
+                a.in.data = A->work;
+                a.out.data = A->work + A->state_floats;
+                a.evt.cap = 0;
+                a.t = A->t0 + n0;
+                LBEM_CUDA(forward_3d(h, a, len, A->seg, &launches));
+            }
+            StepArgs a = base;
+            a.in.data = A->lam + (size_t)lc * A->state_floats;
+            a.out.data = A->lam + (size_t)(lc ^ 1) * A->state_floats;
+            a.t = A->t0 + n0 + len - 1;
+            Adj3 q;
+            q.sig = A->seg + (size_t)(len - 1) * A->sig_floats;
+            q.gcl = A->gcl;
+            q.cot = A->cot;
+            q.nsteps = A->nsteps;
+            q.t0 = A->t0;
+            LBEM_CUDA(adjoint_sigma(h, a, q, len, &launches));
+            lc ^= launches & 1;
+        }
+    }
+    for (int k = d3 ? -1 : A->ncp - 1; k >= 0; k--) {
         const int n0 = k * A->every;
         const int len = std::min(A->every, A->nsteps - n0);
         LBEM_CUDA(cudaMemcpyAsync(A->seg, A->cps + (size_t)k * A->state_floats, sb, cudaMemcpyDeviceToDevice, h->stream));
@@ -556,7 +469,7 @@ lbem_status lbem_adjoint(lbem_t *h, const float *trace_cot, float *grad_eps, dou
             a.out.data = A->seg + (size_t)j * A->state_floats;
             a.evt.cap = 0;
             a.t = A->t0 + n0 + j - 1;
-            LBEM_CUDA(launch_fwd(h, a));
+            LBEM_CUDA(launch_step_2d(a, h->storage, false, h->variant, h->stream));
         }
         for (int j = len - 1; j >= 0; j--) {
             AdjArgs a;

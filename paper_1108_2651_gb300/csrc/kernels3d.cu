@@ -138,8 +138,9 @@ __global__ void __launch_bounds__(BLOCK) step3d(StepArgs a) {
 // Far fewer registers than the 4-sites-per-lane kernel, so more warps per SM.
 // With WL, pulls across walls follow wall_sign3 and the absorbing layer's
 // factor fx(x) fy(y) fz(z) scales the result.
-template <bool MU, bool WL = false>
-__global__ void __launch_bounds__(BLOCK, 5) step3d_site(StepArgs a, Walls w) {
+// With SIG, sigma of the state that the step starts from goes to sig[3][plane] (the adjoint's record).
+template <bool MU, bool WL = false, bool SIG = false>
+__global__ void __launch_bounds__(BLOCK, 5) step3d_site(StepArgs a, Walls w, float *sig) {
     const Grid &G = a.g;
     const int tpr = G.pitch;  // threads per row (pitch is a multiple of 32)
     const long long tid = (long long)blockIdx.x * BLOCK + threadIdx.x;
@@ -206,6 +207,12 @@ __global__ void __launch_bounds__(BLOCK, 5) step3d_site(StepArgs a, Walls w) {
             }
         }
     }
+    if (SIG) {
+        const Mom3 m = moments3(h);
+        sig[o] = m.sx;
+        sig[G.plane + o] = m.sy;
+        sig[2 * G.plane + o] = m.sz;
+    }
     collide3d_free(h, cl);
     if (src) source3d(h, cl, shx, shy, shz);  // (S^ = 0 would add -0)
     float *out = static_cast<float *>(a.out.data);
@@ -222,18 +229,20 @@ __global__ void __launch_bounds__(BLOCK, 5) step3d_site(StepArgs a, Walls w) {
 // registers capped for 5 resident blocks per SM
 int nvariants_3d() { return 3; }
 
-cudaError_t launch_step_3d(const StepArgs &a, bool has_mu, int variant, cudaStream_t s, const Walls *w) {
+cudaError_t launch_step_3d(const StepArgs &a, bool has_mu, int variant, cudaStream_t s, const Walls *w, float *sig) {
     const bool walls = w && (w->kind[0] || w->kind[1] || w->kind[2]);
-    if (variant >= 1 || walls) {  // walls: the one-site-per-thread kernel, which applies them
+    if (variant >= 1 || walls || sig) {  // walls, sigma: the one-site-per-thread kernel
         const long long threads = (long long)a.g.nrows * a.g.pitch;
         const unsigned blocks = (unsigned)((threads + BLOCK - 1) / BLOCK);
         const Walls wv = walls ? *w : Walls();
-        if (walls) {
-            if (has_mu) step3d_site<true, true><<<blocks, BLOCK, 0, s>>>(a, wv);
-            else step3d_site<false, true><<<blocks, BLOCK, 0, s>>>(a, wv);
+        if (sig) {  // (the adjoint's medium: uniform mu, no walls)
+            step3d_site<false, false, true><<<blocks, BLOCK, 0, s>>>(a, wv, sig);
+        } else if (walls) {
+            if (has_mu) step3d_site<true, true><<<blocks, BLOCK, 0, s>>>(a, wv, nullptr);
+            else step3d_site<false, true><<<blocks, BLOCK, 0, s>>>(a, wv, nullptr);
         } else {
-            if (has_mu) step3d_site<true><<<blocks, BLOCK, 0, s>>>(a, wv);
-            else step3d_site<false><<<blocks, BLOCK, 0, s>>>(a, wv);
+            if (has_mu) step3d_site<true><<<blocks, BLOCK, 0, s>>>(a, wv, nullptr);
+            else step3d_site<false><<<blocks, BLOCK, 0, s>>>(a, wv, nullptr);
         }
         return cudaGetLastError();
     }

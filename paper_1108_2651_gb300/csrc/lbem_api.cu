@@ -213,9 +213,9 @@ static bool march_ok(const lbem_t *h) {
 }
 // 3D: triples of steps by the marching kernel (march3d.cu) where several steps per launch are the default, with uniform
 // mu and the one-site-per-thread launch shapes; offsets in a plane must fit 32 bits.
-static bool march3_ok(const lbem_t *h) {
+bool march3_ok(const lbem_t *h, bool adjoint) {
     return h->tblock == 2 && h->dim == 3 && h->variant >= 1 && !h->has_mu && h->grid.plane < (1LL << 31) &&
-           march_3d_pays(h->grid, h->bc[0] || h->bc[1] || h->bc[2]);
+           march_3d_pays(h->grid, adjoint || h->bc[0] || h->bc[1] || h->bc[2]);
 }
 static int steps_per_launch(const lbem_t *h) { return three_step_ok(h) ? 3 : two_step_ok(h) ? 2 : 1; }
 

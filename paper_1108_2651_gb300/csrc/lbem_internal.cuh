@@ -592,8 +592,21 @@ cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaS
 // 3D, MARCH3_STEPS steps per launch, uniform mu, walls and layers included (march3d.cu): nlaunch launches from a.in,
 // alternating between the two buffers
 constexpr int MARCH3_STEPS = 3;
-bool march_3d_pays(const Grid &g, bool walls);  // whether it takes less time than single steps on this grid
+// whether it takes less time than single steps on this grid (more: with walls, with sigma written, and for the adjoint)
+bool march_3d_pays(const Grid &g, bool more);
 cudaError_t launch_march_3d(const StepArgs &a, const Walls &w, int nlaunch, cudaStream_t s);
+bool march3_ok(const lbem_t *h, bool adjoint = false);  // whether (adjoint) steps of this handle go to it
+// what the 3D adjoint records and accumulates (adjoint.cu)
+struct Adj3 {
+    float *sig = nullptr;       // sigma of the state a step starts from, [3][plane]; the next step's follows
+    double *gcl = nullptr;      // dL/dc_L^2, [plane]
+    const float *cot = nullptr; // receivers' cotangents [nrec][nsteps]
+    int nsteps = 0;
+    long long t0 = 0;
+};
+// nlaunch launches of MARCH3_STEPS steps each from a.in at a.t: forward ones that write sigma (record), or adjoint ones
+// back from a.t, whose lambda (by opposite directions) alternates between a.in and a.out and whose first sigma is adj.sig
+cudaError_t launch_march_3d_adj(const StepArgs &a, const Adj3 &adj, bool record, int nlaunch, cudaStream_t s);
 int ss2_nshapes();  // strip streaming (sstream.cu): two steps per launch, FP32, uniform mu
 cudaError_t launch_step_2d_ss2(const StepArgs &a, int shape, cudaStream_t s);
 cudaError_t launch_step_2d_ss2_an(const StepArgs &a, cudaStream_t s);  // anisotropic medium, no pole
@@ -655,7 +668,8 @@ cudaError_t launch_fields_2d(const lbem_t *h, float *E, float *B, cudaStream_t s
 cudaError_t launch_diag_2d(const lbem_t *h, double *partials, int nblocks, cudaStream_t s);
 // 3D (kernels3d.cu)
 int nvariants_3d();
-cudaError_t launch_step_3d(const StepArgs &a, bool has_mu, int variant, cudaStream_t s, const Walls *w = nullptr);
+cudaError_t launch_step_3d(const StepArgs &a, bool has_mu, int variant, cudaStream_t s, const Walls *w = nullptr,
+                           float *sig = nullptr);
 cudaError_t launch_init_3d(const lbem_t *h, const float *E, const float *B, cudaStream_t s);
 cudaError_t launch_fields_3d(const lbem_t *h, float *E, float *B, cudaStream_t s);
 cudaError_t launch_diag_3d(const lbem_t *h, double *partials, int nblocks, cudaStream_t s);

@@ -25,9 +25,14 @@
 
 namespace lbk {
 
+// What the kernel does: steps; steps that also write each level's sigma (the adjoint's record); adjoint steps, which go
+// back in time (level j at a.t - j) on lambda stored by opposite directions.
+enum { M3_STEP, M3_RECORD, M3_ADJOINT };
+
 struct March3Args {
     StepArgs a;
     Walls w;
+    Adj3 adj;
     int ntx, nty, nseg;
 };
 
@@ -36,7 +41,7 @@ constexpr int M3_PLANES = 512;  // the most planes a block marches
 __host__ __device__ __forceinline__ int cut3(int k, int n, int of) { return (int)((long long)k * of / n); }
 
 // TY rows of columns by NW warps: a thread holds NR = TY / NW columns (rows ty, ty + NW, ..).
-template <int K, int NW, int NR, bool WL>
+template <int K, int NW, int NR, bool WL, int MODE>
 __global__ void __launch_bounds__(32 * NW, 1) march3d(const __grid_constant__ March3Args m) {
     constexpr int TY = NW * NR;
     static_assert(TY <= 32, "a plane's mask of rows with events is one word");
@@ -76,6 +81,9 @@ __global__ void __launch_bounds__(32 * NW, 1) march3d(const __grid_constant__ Ma
     constexpr unsigned SP = 32 * TY * 4;
     const unsigned stage = (unsigned)__cvta_generic_to_shared(sm3 + 2 * (K - 1) * 6 * TY * 32) + (wid * 32 + lane) * 4;
     const int zend = z1 - 1 + (K - 1);
+    // adjoint: then each level's sigma (3 words a level) and the gradient (FP64) at the sites that the block owns
+    const unsigned stg = stage + (22 + 3 * K) * SP + (wid * 32 + lane) * 4;
+    auto own = [&](int r, int z) { return X >= xs && X < xe && Y[r] >= ys && Y[r] < ye && z >= z0 && z < z1; };
     // copies of column r at plane zl (wrapped zw) into its stage
     auto load = [&](int r, int zl, int zw) {
         if (zl <= zend) {
@@ -110,17 +118,53 @@ __global__ void __launch_bounds__(32 * NW, 1) march3d(const __grid_constant__ Ma
                 ld(18 + g, a6);
             }
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d + 21 * SP), "l"(a.med.cL2 + o) : "memory");
+            if (MODE == M3_ADJOINT) {
+                if (own(r, zl))
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(stg + r * NW * 256), "l"(m.adj.gcl + o)
+                                 : "memory");
+#pragma unroll
+                for (int j = 0; j < K; j++)
+                    if (own(r, zl - j)) {  // (a plane of the grid, not a wrapped one)
+                        const float *sg = m.adj.sig - j * 3 * G.plane + (unsigned)(zl - j) * zstride + col;
+#pragma unroll
+                        for (int g = 0; g < 3; g++)
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d + (22 + 3 * j + g) * SP),
+                                         "l"(sg + g * G.plane)
+                                         : "memory");
+                    }
+            }
         }
         asm volatile("cp.async.commit_group;\n" ::);
     };
     // one level's update at the thread's site of column r, plane z (unwrapped): receivers, collision, sources, layer
-    auto update = [&](float h[21], float cl, int r, int z, long long t, unsigned rows, float fz) {
+    auto update = [&](float h[21], float cl, int r, int z, int j, unsigned rows, float fz, const float sg[3], double &grad) {
+        if constexpr (MODE == M3_ADJOINT) {
+            AdjEvents3 ev = {};
+            if (rows >> (wid + NW * r) & 1) {
+                const long long ro = (long long)wrapi(z, G.nz) * G.ny + yw[r];
+                const int e0 = __ldg(a.evt.rowptr + ro), e1 = __ldg(a.evt.rowptr + ro + 1);
+                for (int e = e0; e < e1; e++) {
+                    const Event q = a.evt.ev[e];
+                    if (q.x == xw) adjoint3_event(ev, q, a.evt, m.adj.cot, m.adj.nsteps, a.t - j, m.adj.t0);
+                }
+            }
+            grad += (double)adjoint3_site(h, sg, cl, ev);
+            return;
+        }
+        const long long t = a.t + j;
+        if (MODE == M3_RECORD && own(r, z)) {
+            const Mom3 mo = moments3(h);
+            float *q = m.adj.sig + j * 3 * G.plane + (unsigned)z * zstride + yw[r] * G.pitch + xw;
+            __stcs(q, mo.sx);
+            __stcs(q + G.plane, mo.sy);
+            __stcs(q + 2 * G.plane, mo.sz);
+        }
         float shx = 0.f, shy = 0.f, shz = 0.f;
         bool src = false;
         if (rows >> (wid + NW * r) & 1) {  // (a warp is one row)
             const long long ro = (long long)wrapi(z, G.nz) * G.ny + yw[r];
             const int e0 = __ldg(a.evt.rowptr + ro), e1 = __ldg(a.evt.rowptr + ro + 1);
-            const bool rec = X >= xs && X < xe && Y[r] >= ys && Y[r] < ye && z >= z0 && z < z1;
+            const bool rec = own(r, z);
             for (int e = e0; e < e1; e++) {
                 const Event ev = a.evt.ev[e];
                 if (ev.x != xw) continue;
@@ -152,6 +196,7 @@ __global__ void __launch_bounds__(32 * NW, 1) march3d(const __grid_constant__ Ma
     // one before, (walls) -z of that plane; the medium and the event rows of the levels' planes
     float R[NR][K][3], PX[NR][K][3], MX[NR][K][3], PZ0[NR][K][3], PZ1[NR][K][3], MZ[NR][K][3], C[NR][K], F[K];
     unsigned EV[K];
+    double GR[NR][K];  // the gradient with the levels' contributions so far
 #pragma unroll
     for (int r = 0; r < NR; r++)
 #pragma unroll
@@ -160,6 +205,7 @@ __global__ void __launch_bounds__(32 * NW, 1) march3d(const __grid_constant__ Ma
             for (int g = 0; g < 3; g++)
                 R[r][j][g] = PX[r][j][g] = MX[r][j][g] = PZ0[r][j][g] = PZ1[r][j][g] = MZ[r][j][g] = 0.f;
             C[r][j] = 0.f;
+            GR[r][j] = 0.;
         }
     // the next launch's blocks may take their places; this one's inputs are those of the launch before
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -238,10 +284,17 @@ __global__ void __launch_bounds__(32 * NW, 1) march3d(const __grid_constant__ Ma
 #pragma unroll
             for (int j = K - 1; j > 0; j--) {
                 C[r][j] = C[r][j - 1];
+                GR[r][j] = GR[r][j - 1];
             }
             C[r][0] = rd(21);
+            float sg[K][3] = {};
+            if (MODE == M3_ADJOINT) {
+#pragma unroll
+                for (int q = 0; q < 3 * K; q++) sg[q / 3][q % 3] = rd(22 + q);
+                asm volatile("ld.shared.f64 %0, [%1];" : "=d"(GR[r][0]) : "r"(stg + r * NW * 256));
+            }
             load(r, z + 1, zn);
-            update(v, C[r][0], r, z, a.t, EV[0], F[0]);
+            update(v, C[r][0], r, z, 0, EV[0], F[0], sg[0], GR[r][0]);
 #pragma unroll
             for (int j = 1; j < K; j++) {
                 float h[21];
@@ -290,15 +343,16 @@ __global__ void __launch_bounds__(32 * NW, 1) march3d(const __grid_constant__ Ma
                     cur[(g * TY + row) * 32] = v[6 + g];
                     cur[((3 + g) * TY + row) * 32] = v[15 + g];
                 }
-                update(h, C[r][j], r, zj, a.t + j, EV[j], F[j]);
+                update(h, C[r][j], r, zj, j, EV[j], F[j], sg[j], GR[r][j]);
 #pragma unroll
                 for (int p = 0; p < 21; p++) v[p] = h[p];
             }
             const int zo = z - (K - 1);
             if (zo >= z0 && X >= xs && X < xe && Y[r] >= ys && Y[r] < ye) {
-                float *q = out + (unsigned)zo * zstride + yw[r] * G.pitch + xw;
+                const unsigned o = (unsigned)zo * zstride + yw[r] * G.pitch + xw;
 #pragma unroll
-                for (int p = 0; p < 21; p++) __stcs(q + p * G.plane, v[p]);
+                for (int p = 0; p < 21; p++) __stcs(out + p * G.plane + o, v[p]);
+                if (MODE == M3_ADJOINT) m.adj.gcl[o] = GR[r][K - 1];
             }
         }
         zw = zn;
@@ -327,10 +381,10 @@ static long long plan3(const Grid &g, int wave, int *ntx, int *nty, int *nseg) {
 }
 
 // Each launch may start while the one before drains (it waits for its input with griddepcontrol.wait).
-template <int K, int NW, int NR, bool WL>
-static cudaError_t launch_march3(const StepArgs &a, const Walls &w, int nlaunch, cudaStream_t s) {
-    constexpr int TY = NW * NR, smem = (2 * (K - 1) * 6 + 22) * TY * 32 * 4;
-    auto *k = march3d<K, NW, NR, WL>;
+template <int K, int NW, int NR, bool WL, int MODE>
+static cudaError_t launch_march3(const StepArgs &a, const Walls &w, const Adj3 &adj, int nlaunch, cudaStream_t s) {
+    constexpr int TY = NW * NR, smem = (2 * (K - 1) * 6 + 22 + (MODE == M3_ADJOINT ? 3 * K + 2 : 0)) * TY * 32 * 4;
+    auto *k = march3d<K, NW, NR, WL, MODE>;
     static int per_sm = 0, nsm = 0;
     if (!per_sm) {
         int dev = 0, n = 0;
@@ -344,6 +398,7 @@ static cudaError_t launch_march3(const StepArgs &a, const Walls &w, int nlaunch,
     March3Args m;
     m.a = a;
     m.w = w;
+    m.adj = adj;
     plan3<K, TY>(a.g, per_sm * nsm, &m.ntx, &m.nty, &m.nseg);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -356,9 +411,11 @@ static cudaError_t launch_march3(const StepArgs &a, const Walls &w, int nlaunch,
     cfg.attrs = at;
     cfg.numAttrs = 1;
     for (int l = 0; l < nlaunch; l++) {
-        m.a.t = a.t + (long long)K * l;
         const cudaError_t e = cudaLaunchKernelEx(&cfg, k, m);
         if (e != cudaSuccess) return e;
+        constexpr int dt = MODE == M3_ADJOINT ? -K : K;
+        m.a.t += dt;
+        if (MODE != M3_STEP) m.adj.sig += dt * 3 * a.g.plane;
         std::swap(m.a.in, m.a.out);
     }
     return cudaSuccess;
@@ -369,15 +426,22 @@ constexpr int M3_WARPS = 10, M3_COLS = 2;
 cudaError_t launch_march_3d(const StepArgs &a, const Walls &w, int nlaunch, cudaStream_t s) {
     constexpr int K = MARCH3_STEPS;
     const bool walls = w.kind[0] || w.kind[1] || w.kind[2];
-    return walls ? launch_march3<K, M3_WARPS, M3_COLS, true>(a, w, nlaunch, s)
-                 : launch_march3<K, M3_WARPS, M3_COLS, false>(a, w, nlaunch, s);
+    return walls ? launch_march3<K, M3_WARPS, M3_COLS, true, M3_STEP>(a, w, Adj3(), nlaunch, s)
+                 : launch_march3<K, M3_WARPS, M3_COLS, false, M3_STEP>(a, w, Adj3(), nlaunch, s);
+}
+
+cudaError_t launch_march_3d_adj(const StepArgs &a, const Adj3 &adj, bool record, int nlaunch, cudaStream_t s) {
+    constexpr int K = MARCH3_STEPS;
+    return record ? launch_march3<K, M3_WARPS, M3_COLS, false, M3_RECORD>(a, Walls(), adj, nlaunch, s)
+                  : launch_march3<K, M3_WARPS, M3_COLS, false, M3_ADJOINT>(a, Walls(), adj, nlaunch, s);
 }
 
 // Whether K steps of the marching kernel take less time than K single ones.  Marching takes 2.5 us a plane of a wave of
-// blocks (3.4 with walls), a single step 3.5 us and 25.4 ns (28.7) per thousand sites, measured on cubes of 24 to 192:
-// 64^3 8.2 us a step either way, 48^3 5.1 against 6.2 us; with walls 64^3 11.4 against 10.3 us, 80^3 14.3 against 20.5 us.
+// blocks (3.4 with more to do: walls, sigma, the adjoint), a single step 3.5 us and 25.4 ns (28.7) per thousand sites,
+// measured on cubes of 24 to 192: 64^3 8.2 us a step either way, 48^3 5.1 against 6.2 us; with walls 64^3 11.4 against
+// 10.3 us, 80^3 14.3 against 20.5 us; 40 steps recorded and gone back 64^3 1.20 against 1.07 ms, 80^3 1.49 against 1.84 ms.
 // A grid a little wider than a tile, say 30 x 24 x 96, pays for two tiles.
-bool march_3d_pays(const Grid &g, bool walls) {
+bool march_3d_pays(const Grid &g, bool more) {
     constexpr int K = MARCH3_STEPS;
     int nsm = 0, dev = 0, ntx, nty, nseg;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -385,7 +449,7 @@ bool march_3d_pays(const Grid &g, bool walls) {
         return false;
     const double planes = (double)plan3<K, M3_WARPS * M3_COLS>(g, nsm, &ntx, &nty, &nseg);
     const double sites = (double)g.nx * g.ny * g.nz;
-    return planes * (walls ? 3.4 : 2.5) <= K * (3.5 + sites * (walls ? 28.7e-6 : 25.4e-6));
+    return planes * (more ? 3.4 : 2.5) <= K * (3.5 + sites * (more ? 28.7e-6 : 25.4e-6));
 }
 
 }  // namespace lbk

@@ -101,4 +101,88 @@ __device__ __forceinline__ float wall_sign3(int kind, int gm, int ax) {
     return (kind == 1 ? 1.f : -1.f) * (gm == ax ? 1.f : -1.f);
 }
 
+// The direction opposite to i (of planes 3 i + gamma), as a plane.
+__host__ __device__ constexpr int opp3(int p) { return p < 3 ? p : p < 12 ? p + 9 : p - 9; }
+
+// What a site's events add to its adjoint update: the point current, and the receivers' cotangents by component.
+struct AdjEvents3 {
+    float j[3], rE[3], rB[3];
+};
+
+// One site of the adjoint step (adjoint.cu states it): v[opp3(p)] = mu_p, the populations of lambda^{t+1} pulled as the
+// forward step pulls (lambda is stored by opposite directions), becomes lambda^t in the same order; returns the step's
+// contribution to dL/dc_L^2.  sg: sigma of g^t, q: c_L^2.
+__device__ __forceinline__ float adjoint3_site(float v[21], const float sg[3], float q, const AdjEvents3 &ev) {
+    float h[21];
+#pragma unroll
+    for (int p = 0; p < 21; p++) h[p] = v[opp3(p)];
+    const float w0 = __fmaf_rn(-3.f, q, 1.f), hq = 0.5f * q;
+    float mv[3], L[3];
+    float d = 0.f;
+#pragma unroll
+    for (int g = 0; g < 3; g++) {
+        mv[g] = ((h[3 + g] + h[6 + g]) + (h[9 + g] + h[12 + g])) + (h[15 + g] + h[18 + g]);
+        L[g] = 2.f * __fmaf_rn(w0, h[g], __fmul_rn(hq, mv[g]));
+        d = __fadd_rn(d, __fmaf_rn(sg[g], mv[g], -__fmul_rn(6.f, __fmul_rn(sg[g], h[g]))));
+        d = __fmaf_rn(ev.j[g], __fmaf_rn(0.25f, mv[g], -__fmul_rn(1.5f, h[g])), d);
+    }
+    // V = sum_i mu_i x c_i, the same contraction that reads B from h (V/2 is exact)
+    const float vx = (h[10] - h[19]) - (h[8] - h[17]);
+    const float vy = (h[5] - h[14]) - (h[9] - h[18]);
+    const float vz = (h[6] - h[15]) - (h[4] - h[13]);
+    const float xpy = __fmaf_rn(0.5f, vy, L[0]), xmy = __fmaf_rn(-0.5f, vy, L[0]);
+    const float xpz = __fmaf_rn(0.5f, vz, L[0]), xmz = __fmaf_rn(-0.5f, vz, L[0]);
+    const float ypx = __fmaf_rn(0.5f, vx, L[1]), ymx = __fmaf_rn(-0.5f, vx, L[1]);
+    const float ypz = __fmaf_rn(0.5f, vz, L[1]), ymz = __fmaf_rn(-0.5f, vz, L[1]);
+    const float zpx = __fmaf_rn(0.5f, vx, L[2]), zmx = __fmaf_rn(-0.5f, vx, L[2]);
+    const float zpy = __fmaf_rn(0.5f, vy, L[2]), zmy = __fmaf_rn(-0.5f, vy, L[2]);
+    float o[21] = {L[0], L[1], L[2],      // rest
+                   L[0], ymz, zpy,        // +x: c x V = (0, -Vz, Vy)
+                   xpz, L[1], zmx,        // +y: (Vz, 0, -Vx)
+                   xmy, ypx, L[2],        // +z: (-Vy, Vx, 0)
+                   L[0], ypz, zmy,        // -x
+                   xmz, L[1], zpx,        // -y
+                   xpy, ymx, L[2]};       // -z
+#pragma unroll
+    for (int p = 0; p < 21; p++) o[p] = __fsub_rn(o[p], h[p]);
+    // receivers: E_gamma = -c_L^2 sigma_gamma;  B_nu = eps_{gamma kappa nu} sum_i c_{i kappa} g_{i gamma}
+#pragma unroll
+    for (int g = 0; g < 3; g++)
+        if (ev.rE[g] != 0.f) {
+#pragma unroll
+            for (int i = 0; i < 7; i++) o[3 * i + g] = __fmaf_rn(-q, ev.rE[g], o[3 * i + g]);
+            d = __fmaf_rn(-sg[g], ev.rE[g], d);
+        }
+    if (ev.rB[0] != 0.f || ev.rB[1] != 0.f || ev.rB[2] != 0.f) {
+        o[10] += ev.rB[0]; o[19] -= ev.rB[0]; o[8] -= ev.rB[0]; o[17] += ev.rB[0];
+        o[5] += ev.rB[1]; o[14] -= ev.rB[1]; o[9] -= ev.rB[1]; o[18] += ev.rB[1];
+        o[6] += ev.rB[2]; o[15] -= ev.rB[2]; o[4] -= ev.rB[2]; o[13] += ev.rB[2];
+    }
+#pragma unroll
+    for (int p = 0; p < 21; p++) v[opp3(p)] = o[p];
+    return d;
+}
+
+// Adds event e of site time t to ev (cot: the receivers' cotangents [nrec][nsteps] of the steps from t0).
+__device__ __forceinline__ void adjoint3_event(AdjEvents3 &ev, const Event &e, const Events &E, const float *cot,
+                                               int nsteps, long long t, long long t0) {
+    if (e.kind == 0) {
+        if (t < E.nt) {
+            const float jj = __ldg(E.amp + (long long)e.index * E.nt + t);
+#pragma unroll
+            for (int g = 0; g < 3; g++)
+                if (e.comp == g) ev.j[g] += jj;
+        }
+    } else {
+        const long long n = t - t0;
+        if (n < 0 || n >= nsteps || t >= E.cap) return;
+        const float r = __ldg(cot + (long long)e.index * nsteps + n);
+#pragma unroll
+        for (int g = 0; g < 3; g++) {
+            if (e.comp == g) ev.rE[g] += r;
+            if (e.comp == 3 + g) ev.rB[g] += r;
+        }
+    }
+}
+
 }  // namespace lbk

@@ -118,3 +118,43 @@ def test_march_3d_is_bitwise_identical_to_single_steps(lbem, shape, walls):
         for graphs in (False, True):
             for a, b in zip(ref, _run(p, calls, graphs=graphs)):
                 np.testing.assert_array_equal(a, b)
+
+
+# the 3D adjoint: sigma of every step or of checkpointed segments, three steps per launch or one; the last shape is too
+# small for three
+@pytest.mark.parametrize("shape", [(90, 81, 84), (75, 61, 90), (9, 20, 37)])
+def test_march_3d_adjoint_is_bitwise_identical_to_single_steps(lbem, shape):
+    import torch
+
+    from paper_1108_2651_gb300.autograd import receiver_traces
+
+    n = int(np.prod(shape))
+    eps0 = torch.from_numpy(W.random_medium(shape, 5, 1.0)[0].astype(np.float32)).cuda()
+
+    def run(nsteps, every, steps_per_pass, repeat=1):
+        rng = np.random.default_rng(8)
+        p = W.Problem("march3", 3, shape, None, None, nsteps)
+        p.src_site = np.unique(np.concatenate([[0, n - 1], rng.integers(0, n, 4)])).astype(np.int64)
+        p.src_comp = np.resize(np.arange(3, dtype=np.int32), p.src_site.size)
+        p.src_amp = rng.standard_normal((p.src_site.size, nsteps))
+        p.rec_site = np.concatenate([p.src_site, rng.integers(0, n, 24)]).astype(np.int64)
+        p.rec_comp = np.resize(np.arange(6, dtype=np.int32), p.rec_site.size)
+        cot = torch.from_numpy(rng.standard_normal((p.rec_site.size, nsteps)).astype(np.float32)).cuda()
+        s = lbem.Solver(shape)
+        lbem.lbem_set_temporal_blocking(s.h, steps_per_pass, -1)
+        for _ in range(repeat):  # a second run takes over the first one's buffers
+            eps = eps0.clone().requires_grad_(True)
+            tr = receiver_traces(eps, s, p, checkpoint_every=every)
+            tr.backward(cot)
+        torch.cuda.synchronize()
+        lbem.lbem_check_guards(s.h)
+        s.close()
+        return tr.detach().cpu().numpy(), eps.grad.cpu().numpy()
+
+    for nsteps, everys in ((14, (14, 4, 1)), (241, (241, 16))):  # 241 steps, a state kept every 16
+        ref = run(nsteps, nsteps, 1)
+        assert np.abs(ref[1]).max() > 0
+        for every in everys:
+            for spp, repeat in ((1, 1), (2, 2)):
+                for a, b in zip(ref, run(nsteps, every, spp, repeat)):
+                    np.testing.assert_array_equal(a, b)
