@@ -225,9 +225,8 @@ __global__ void __launch_bounds__(BLOCK) adjoint2d(AdjArgs a) {
 template <int MINB>
 __global__ void __launch_bounds__(BLOCK, MINB) adjoint3d_site(AdjArgs a, const float *sig) {
     const Grid &G = a.g;
-    const long long tid = (long long)blockIdx.x * BLOCK + threadIdx.x;
-    const int row = (int)(tid / G.pitch);
-    const int x = (int)(tid - (long long)row * G.pitch);
+    int row, x;
+    site_of(G, row, x);
     if (row >= G.nrows || x >= G.nx) return;
     const int z = row / G.ny, y = row - z * G.ny;
     const int rym = z * G.ny + (y == 0 ? G.ny - 1 : y - 1), ryp = z * G.ny + (y == G.ny - 1 ? 0 : y + 1);

@@ -652,7 +652,8 @@ lbem_status lbem_set_fields(lbem_t *h, const float *E, const float *B) {
     LBEM_CUDA(e);
     h->t = 0;
     h->wd_last = -1.0;
-    if (h->d_traces) LBEM_CUDA(cudaMemsetAsync(h->d_traces, 0, sizeof(float) * (size_t)h->nrec * h->cap, h->stream));
+    if (h->d_traces && h->storage != LBEM_F32)  // (the FP32 kernels clear them)
+        LBEM_CUDA(cudaMemsetAsync(h->d_traces, 0, sizeof(float) * (size_t)h->nrec * h->cap, h->stream));
     if (h->disp) {  // the pole starts at rest: D = E
         for (float *p : {h->d_J, h->d_J2, h->d_P, h->d_P2})
             LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * (size_t)h->grid.plane, h->stream));

@@ -395,6 +395,14 @@ struct __align__(16) StepArgs {
 };
 
 // Periodic index, cheap when v is already in range (the common case).
+// One site per thread, a warp 32 consecutive ones of a row (pitch is a multiple of 32): the thread's row and x, by one
+// 32-bit division.  (Dividing the thread's 64-bit index by the pitch takes longer than the rest of a light kernel.)
+__device__ __forceinline__ void site_of(const Grid &G, int &row, int &x) {
+    const unsigned w = blockIdx.x * (BLOCK / 32) + (threadIdx.x >> 5), wpr = (unsigned)G.pitch >> 5;
+    row = (int)(w / wpr);
+    x = (int)(w - row * wpr) * 32 + (threadIdx.x & 31);
+}
+
 __device__ __forceinline__ int wrapi(int v, int n) {
     if ((unsigned)v < (unsigned)n) return v;
     v %= n;
@@ -663,6 +671,8 @@ int batch_ss2_rows(int shape);    // chunk rows (TBY) of a shape
 int batch_ss2_chunks(int shape);  // chunks of a full unit
 cudaError_t launch_batch_ss2(const StepArgs *args, const BatchUnit *units, int nunits, int *sched, const long long *t0p,
                              int toff, int par, const BatchPacked &pk, long long rows, int shape, cudaStream_t s);
+// The initial state from dense fields (null: zero); the FP32 kernels also clear the receivers' traces (ntr floats; 16-bit
+// storage leaves them to the caller).
 cudaError_t launch_init_2d(const lbem_t *h, const float *E, const float *B, cudaStream_t s);
 cudaError_t launch_fields_2d(const lbem_t *h, float *E, float *B, cudaStream_t s);
 cudaError_t launch_diag_2d(const lbem_t *h, double *partials, int nblocks, cudaStream_t s);
