@@ -5,15 +5,16 @@ s seeded smoothed random field, sigma = 20 cells, seed 2), Ricker point
 current at the centre (~20 cells per local wavelength), 64 receivers, 5000
 time steps, FP32 storage.  One benchmark step is one full pass of the hot
 path over that input: medium upload, initial state, 5000 fused
-stream-collide steps with the source and receivers (2500 launches of the
-two-step kernel, the library's default for this case), field extraction,
+stream-collide steps with the source and receivers (625 launches of the
+marching kernel, 8 steps each, the library's default), field extraction,
 receiver traces and the FP64 diagnostics.  The distributions (2 x 336 MB)
 are larger than L2, so no flush is needed between steps.
 
 Metric: Mlups (10^6 lattice-site updates per second) = sites x 5000 / time.
-The stream-collide kernels are bound by HBM bandwidth: 44 algorithmic bytes
-per site per launch (5 populations read + 5 written in FP32, plus c_L^2),
-whether a launch advances one step or two.
+A launch moves 44 algorithmic bytes per site (5 populations read + 5 written
+in FP32, plus c_L^2), whether it advances one step or eight: single steps and
+pairs are bound by HBM bandwidth, the marching kernel by the issue of its
+arithmetic.
 
 --impl reference times the FP64 CPU oracle (test infrastructure) on a
 bounded sample of the same workload.  With torchrun (N > 1) the path shards:
@@ -44,8 +45,10 @@ BYTES_PER_SITE = {"f32": 44, "f16": 24, "bf16": 24, "i16b": 26.5}
 # the kernel that was captured.
 NCU_TRAFFIC = {("het2d_4096", "f32", "tb2-0"): 433.764864e6 + 300.201472e6,
                ("het2d_4096", "f32", "tb2-10"): 412.030720e6 + 284.538624e6,
+               ("het2d_4096", "f32", "march"): 449.122560e6 + 290.532864e6,
                ("het2d_4096", "f16", "tb2-0"): 238.282240e6 + 128.542464e6,
                ("het2d_4096", "i16b", "tb2-0"): 264.385536e6 + 150.971648e6,
+               ("het3d_192", "f32", "march"): 698.538240e6 + 551.214336e6,
                # dram__bytes.sum.per_second x gpu__time_duration.sum (6.657849 TB/s x 174.752 us), step2d_gen
                ("het2d_drude_4096", "f32", "disp"): 6.657849e12 * 174.752e-6,
                ("het2d_aniso_4096", "f32", "tb2an"): 431.234560e6 + 297.513216e6,
@@ -54,8 +57,31 @@ PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 
 
 def BATCH_SPL(variant):
-    """Steps per launch of a batch launch shape (lbem_batch_set_variant: 9, 10, 11 advance two steps)."""
-    return 2 if variant >= 9 else 1
+    """Steps per launch of a batch launch shape (lbem_batch_set_variant: 9 to 15 advance two steps, 16 eight)."""
+    return 8 if variant == 16 else 2 if variant >= 9 else 1
+
+
+def batch_kernel(variant):
+    return ("march2d_batch" if variant == 16 else "step2d_batch_ss2" if variant >= 14 else
+            "step2d_batch_tb2" if variant >= 9 else "step2d_batch")
+
+
+def steps_per_launch(p, storage, spp, tile_shape_set=False):
+    """Steps that one launch of lbem_step advances: with the two-step default and no tile shape chosen, those of the
+    marching kernel for the workload's medium and storage; else the steps per pass that were set."""
+    if p.D == 3:
+        return 3 if spp == 2 and p.mu_r is None else 1
+    pole, tensor = p.wp2 is not None, getattr(p, "aniso", None) is not None
+    if spp != 2 or tile_shape_set or (pole and (tensor or p.mu_r is not None or any(p.bc))):
+        return spp
+    if storage == "i16b":
+        return 4
+    return 6 if pole or p.mu_r is not None else 8
+
+
+def step_launches(p, nsteps, spl):
+    """Launches of nsteps steps, spl each (2D: a last one of what is left over; 3D: single steps)."""
+    return nsteps // spl + (nsteps % spl if p.D == 3 or spl <= 3 else (nsteps % spl > 0))
 
 
 def measured_peak_gbs():
@@ -166,7 +192,7 @@ def run_batch_main(args, lbem, torch, stream, peak, peak_kind):
     for s in ss:
         s.close()
     spl = BATCH_SPL(v)
-    launches = nsteps // spl + nsteps % spl
+    launches = step_launches(probs[0], nsteps, spl)
     per = ms / launches
     gbs = 44 * sites / (per * 1e-3) / 1e9
     value = sites * nsteps / (ms * 1e-3) / 1e6
@@ -175,8 +201,7 @@ def run_batch_main(args, lbem, torch, stream, peak, peak_kind):
                       "vs_baseline": None, "dtype": "f32", "data": "synthetic",
                       "config": {"workload": "batch256", "media": len(probs), "sites": sites, "lb_steps": nsteps},
                       "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
-                                   "traffic": None, "kernel": ("step2d_batch_ss2" if v >= 14 else "step2d_batch_tb2" if spl == 2
-                                                                 else "step2d_batch") + f" (variant {v})", "steps_per_launch": spl,
+                                   "traffic": None, "kernel": f"{batch_kernel(v)} (variant {v})", "steps_per_launch": spl,
                                    "ms_per_launch": per, "peak_kind": peak_kind},
                       "gpu_launches": args.steps * launches, "clocks": clk.summary()}), flush=True)
 
@@ -217,8 +242,9 @@ def run_adjoint_main(args, lbem, torch, stream, peak, peak_kind):
     ms = start.elapsed_time(stop) / args.steps
     bwd = float(np.mean([a.elapsed_time(b) for a, b in evs]))
     s.close()
-    # backward bytes: recompute of nsteps - every forward steps (172 B/site) + nsteps adjoint steps (272 B/site)
-    bb = ((nsteps - 10) * 172 + nsteps * 272) * n3
+    # backward bytes: adjoint steps, three per launch (224 B/site: lambda 84 read and 84 written, c_L^2 4, FP64
+    # gradient 16, sigma 3 x 12); every step's sigma is kept, so nothing is recomputed
+    bb = nsteps * 224 / 3 * n3
     gbs = bb / (bwd * 1e-3) / 1e9
     print(json.dumps({"metric": "Mlups", "value": n3 * nsteps / (ms * 1e-3) / 1e6, "unit": "Mlups", "n_gpus": 1,
                       "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
@@ -227,17 +253,20 @@ def run_adjoint_main(args, lbem, torch, stream, peak, peak_kind):
                                  "checkpoint_every": 10, "note": "value counts forward site-steps per second of "
                                  "forward record + backward pass"},
                       "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
-                                   "traffic": None, "kernel": "backward pass (recompute + adjoint3d_site)",
+                                   "traffic": None, "kernel": "backward pass (march3d, adjoint steps, 3 per launch)",
                                    "ms_backward": bwd, "peak_kind": peak_kind},
                       "gpu_launches": None, "clocks": clk.summary()}), flush=True)
 
 
 def _time_run(lbem, torch, s, p, nsteps, stream, passes=1):
-    """Device time (ms) of `passes` full runs of nsteps steps on solver s (launch shape autotuned), after one
-    untimed run; returns (ms, variant, steps per launch)."""
+    """Device time (ms) of `passes` full runs of nsteps steps on solver s (single-step launch shape autotuned; the
+    default path of several steps per launch where it was not switched off), after one untimed run; returns (ms,
+    variant, steps per pass)."""
     s.set_problem(p)
     v = lbem.lbem_autotune(s.h, 50)
-    spp = lbem.lbem_get_temporal_blocking(s.h)[0]
+    spp = 2 if p.D == 3 else lbem.lbem_get_temporal_blocking(s.h)[0]  # (3D reports 1)
+    if spp == 2:
+        lbem.lbem_set_temporal_blocking(s.h, 2, -1)
     lbem.lbem_step(s.h, nsteps)
     ev = []
     for _ in range(passes):
@@ -261,11 +290,12 @@ def other_forms(lbem, torch, p, peak, stream):
         s = lbem.Solver(p.shape, storage=st, stream=stream.cuda_stream)
         ms, v, spp = _time_run(lbem, torch, s, p, p.nsteps, stream)
         s.close()
-        per = ms / (p.nsteps // spp + p.nsteps % spp)  # per launch of `spp` steps
+        spl = steps_per_launch(p, st, spp)
+        per = ms / step_launches(p, p.nsteps, spl)  # per launch of `spl` steps
         gbs = BYTES_PER_SITE[st] * n / (per * 1e-3) / 1e9
         out[st] = {"mlups": n * p.nsteps / (ms * 1e-3) / 1e6, "ms_per_launch": per, "achieved_gbs": gbs,
-                   "frac": gbs / peak, "bytes_per_site_per_launch": BYTES_PER_SITE[st], "steps_per_launch": spp,
-                   "variant": v}
+                   "frac": gbs / peak, "bytes_per_site_per_launch": BYTES_PER_SITE[st], "steps_per_launch": spl,
+                   "steps_per_pass": spp, "variant": v}
     # single-step launches (same workload, FP32): the fastest single-step kernel, 44 B/site per step
     s = lbem.Solver(p.shape, stream=stream.cuda_stream)
     lbem.lbem_set_temporal_blocking(s.h, 1, -1)
@@ -302,10 +332,12 @@ def other_forms(lbem, torch, p, peak, stream):
         if best1 is None or ms1 < best1[0]:
             best1 = (ms1, v1, spp1)
     ms, v, spp = best1
-    per = ms / (p1.nsteps // spp + p1.nsteps % spp)
+    spl1 = steps_per_launch(p1, "f32", spp)
+    per = ms / step_launches(p1, p1.nsteps, spl1)
     gbs = 44 * n1 / (per * 1e-3) / 1e9
     out["f32_1024"] = {"mlups": n1 * p1.nsteps / (ms * 1e-3) / 1e6, "ms_per_launch": per, "effective_gbs": gbs,
-                       "frac": gbs / peak, "bytes_per_site_per_launch": 44, "steps_per_launch": spp, "variant": v,
+                       "frac": gbs / peak, "bytes_per_site_per_launch": 44, "steps_per_launch": spl1,
+                       "steps_per_pass": spp, "variant": v,
                        "l2_resident": True, "graphs": True, "lb_steps": p1.nsteps}
     probs = W.batch_2d(256, nsteps=2000)
     ss = []
@@ -332,12 +364,12 @@ def other_forms(lbem, torch, p, peak, stream):
     for s in ss:
         s.close()
     spl = BATCH_SPL(v)
-    per = ms / (2000 // spl)
+    per = ms / step_launches(probs[0], 2000, spl)
     gbs = 44 * sites / (per * 1e-3) / 1e9
     out["batch256"] = {"mlups": sites * 2000 / (ms * 1e-3) / 1e6, "ms_per_launch": per, "achieved_gbs": gbs,
                        "frac": gbs / peak, "sites": sites, "media": len(probs), "lb_steps": 2000, "variant": v,
                        "graph": True, "steps_per_launch": spl,
-                       "kernel": "step2d_batch_ss2" if v >= 14 else "step2d_batch_tb2" if spl == 2 else "step2d_batch"}
+                       "kernel": batch_kernel(v)}
     # heterogeneous permeability (B x grad ln mu source at every site), 2000 steps: 52 B/site per launch (the
     # grad ln mu planes add 8 to the 44), two steps per launch by default, then single-step launches
     pm = W.heterogeneous_2d_mu(p.shape[0], seed=2, nsteps=2000)
@@ -346,30 +378,30 @@ def other_forms(lbem, torch, p, peak, stream):
         if spp_set == 1:
             lbem.lbem_set_temporal_blocking(s.h, 1, -1)
         ms, v, spp = _time_run(lbem, torch, s, pm, 2000, stream)
-        shape_mu = lbem.lbem_get_temporal_blocking(s.h)[1]
         s.close()
-        per = ms / (2000 // spp)
+        spl = steps_per_launch(pm, "f32", spp)
+        per = ms / step_launches(pm, 2000, spl)
         gbs = 52 * n / (per * 1e-3) / 1e9
-        kern = ("step2d_ss2<MU>" if shape_mu == 2 else f"step2d_tb2<MU> (tile shape {shape_mu})") if spp == 2 \
-            else f"step2d<f32, MU> (variant {v})"
+        kern = "march2d<MU>" if spp == 2 else f"step2d<f32, MU> (variant {v})"
         out[key] = {"mlups": n * 2000 / (ms * 1e-3) / 1e6, "ms_per_launch": per, "achieved_gbs": gbs,
-                    "frac": gbs / peak, "bytes_per_site_per_launch": 52, "steps_per_launch": spp, "variant": v,
-                    "lb_steps": 2000, "kernel": kern}
-    # the same medium in a PEC box with a 32-site absorbing layer, 2000 steps: the stream-collide launches plus
-    # the edge kernel after each (44 algorithmic B/site per launch; the edge recompute counts as overhead)
+                    "frac": gbs / peak, "bytes_per_site_per_launch": 52, "steps_per_launch": spl, "steps_per_pass": spp,
+                    "variant": v, "lb_steps": 2000, "kernel": kern}
+    # the same medium in a PEC box with a 32-site absorbing layer, 2000 steps (walls and layer applied in the
+    # marching kernel; 44 algorithmic B/site per launch)
     pw = W.heterogeneous_2d_walls(p.shape[0], seed=2, nsteps=2000)
     s = lbem.Solver(pw.shape, stream=stream.cuda_stream)
     ms, v, spp = _time_run(lbem, torch, s, pw, 2000, stream)
     s.close()
-    per = ms / (2000 // spp)
+    spl = steps_per_launch(pw, "f32", spp)
+    per = ms / step_launches(pw, 2000, spl)
     gbs = 44 * n / (per * 1e-3) / 1e9
     out["f32_walls_absorbing"] = {"mlups": n * 2000 / (ms * 1e-3) / 1e6, "ms_per_launch": per, "achieved_gbs": gbs,
-                                  "frac": gbs / peak, "bytes_per_site_per_launch": 44, "steps_per_launch": spp,
-                                  "variant": v, "lb_steps": 2000, "bc": list(pw.bc), "layer": pw.layer,
+                                  "frac": gbs / peak, "bytes_per_site_per_launch": 44, "steps_per_launch": spl,
+                                  "steps_per_pass": spp, "variant": v, "lb_steps": 2000, "bc": list(pw.bc), "layer": pw.layer,
                                   "gamma_max": pw.gamma_max}
     # the same medium with a lossy Drude cylinder (one dispersive pole per site), 2000 steps: 44 B/site plus the
-    # pole's J and P read and written (16) and its three parameters read (12) = 72 B/site per launch; two steps
-    # per launch by default (the tile kernel carrying the pole), then single-step launches of the general kernel
+    # pole's J and P read and written (16) and its three parameters read (12) = 72 B/site per launch; the
+    # marching kernel carrying the pole by default, then single-step launches of the general kernel
     pd = W.heterogeneous_2d_drude(p.shape[0], seed=2, nsteps=2000)
     for key, spp_set in (("f32_drude_dispersive", 2), ("f32_drude_single_step", 1)):
         s = lbem.Solver(pd.shape, stream=stream.cuda_stream)
@@ -377,47 +409,48 @@ def other_forms(lbem, torch, p, peak, stream):
             lbem.lbem_set_temporal_blocking(s.h, 1, -1)
         ms, v, spp = _time_run(lbem, torch, s, pd, 2000, stream)
         s.close()
-        per = ms / (2000 // spp)
+        spl = steps_per_launch(pd, "f32", spp)
+        per = ms / step_launches(pd, 2000, spl)
         gbs = 72 * n / (per * 1e-3) / 1e9
         out[key] = {"mlups": n * 2000 / (ms * 1e-3) / 1e6, "ms_per_launch": per, "achieved_gbs": gbs,
-                    "frac": gbs / peak, "bytes_per_site_per_launch": 72, "steps_per_launch": spp, "lb_steps": 2000,
-                    "kernel": "step2d_tb2<POLE>" if spp == 2 else "step2d_gen"}
+                    "frac": gbs / peak, "bytes_per_site_per_launch": 72, "steps_per_launch": spl, "steps_per_pass": spp,
+                    "lb_steps": 2000, "kernel": "march2d<POLE>" if spp == 2 else "step2d_gen"}
     # the same medium made uniaxial, mu = diag(2, 1) (per-axis lattice weights), 2000 steps: 44 B/site per
-    # launch, two steps per launch by default (the strip or the tile kernel with per-axis weights, as autotuned),
-    # then single-step launches of the general kernel
+    # launch, the marching kernel with per-axis weights by default, then single-step launches of the general kernel
     pa = W.heterogeneous_2d_aniso(p.shape[0], seed=2, nsteps=2000)
     for key, spp_set in (("f32_anisotropic", 2), ("f32_anisotropic_single_step", 1)):
         s = lbem.Solver(pa.shape, stream=stream.cuda_stream)
         if spp_set == 1:
             lbem.lbem_set_temporal_blocking(s.h, 1, -1)
         ms, v, spp = _time_run(lbem, torch, s, pa, 2000, stream)
-        shape_an = lbem.lbem_get_temporal_blocking(s.h)[1]
         s.close()
-        per = ms / (2000 // spp)
+        spl = steps_per_launch(pa, "f32", spp)
+        per = ms / step_launches(pa, 2000, spl)
         gbs = 44 * n / (per * 1e-3) / 1e9
-        kern = ("step2d_ss2<AN>" if shape_an == 1 else "step2d_tb2<AN>") if spp == 2 else "step2d_gen"
+        kern = "march2d<AN>" if spp == 2 else "step2d_gen"
         out[key] = {"mlups": n * 2000 / (ms * 1e-3) / 1e6, "ms_per_launch": per, "achieved_gbs": gbs,
-                    "frac": gbs / peak, "bytes_per_site_per_launch": 44, "steps_per_launch": spp, "lb_steps": 2000,
-                    "kernel": kern, "mu_tensor": list(pa.aniso)}
-    # 192^3 in a PEC box with a 16-site absorbing layer (walls applied by the one-site-per-thread 3D kernel),
-    # 500 steps: 172 B/site
+                    "frac": gbs / peak, "bytes_per_site_per_launch": 44, "steps_per_launch": spl, "steps_per_pass": spp,
+                    "lb_steps": 2000, "kernel": kern, "mu_tensor": list(pa.aniso)}
+    # 192^3 in a PEC box with a 16-site absorbing layer (walls applied in the 3D marching kernel),
+    # 500 steps: 172 B/site per launch
     qb = W.heterogeneous_3d(192, nsteps=500)
     qb.bc, qb.layer, qb.gamma_max = (1, 1, 1), 16, 0.2
     s = lbem.Solver(qb.shape, stream=stream.cuda_stream)
-    ms, v, _ = _time_run(lbem, torch, s, qb, 500, stream)
+    ms, v, spp = _time_run(lbem, torch, s, qb, 500, stream)
     s.close()
     n3 = int(np.prod(qb.shape))
-    per = ms / 500
+    spl = steps_per_launch(qb, "f32", spp)
+    per = ms / step_launches(qb, 500, spl)
     gbs = 172 * n3 / (per * 1e-3) / 1e9
     out["het3d_192_box"] = {"mlups": n3 * 500 / (ms * 1e-3) / 1e6, "ms_per_launch": per, "achieved_gbs": gbs,
-                            "frac": gbs / peak, "bytes_per_site": 172, "variant": v, "lb_steps": 500,
-                            "steps_per_launch": 1,
+                            "frac": gbs / peak, "bytes_per_site_per_launch": 172, "variant": v, "lb_steps": 500,
+                            "steps_per_launch": spl, "steps_per_pass": spp,
                             "bc": list(qb.bc), "layer": qb.layer}
     q = W.heterogeneous_3d(192, nsteps=1000)
     s = lbem.Solver(q.shape, stream=stream.cuda_stream)
-    ms, v, _ = _time_run(lbem, torch, s, q, 1000, stream)
-    # adjoint: forward with a checkpoint every 100 steps, then the reverse-time pass (segment recompute +
-    # adjoint kernel, FP64 gradient accumulation), cotangent = the traces themselves; the faster of the
+    ms, v, spp = _time_run(lbem, torch, s, q, 1000, stream)
+    # adjoint: forward with a checkpoint every 100 steps, then the reverse-time pass (segment recompute writing
+    # sigma + adjoint steps, three steps per launch, FP64 gradient accumulation), cotangent = the traces themselves; the faster of the
     # two one-site-per-thread adjoint shapes (3D variants 1 and 2) on a short trial
     trial = {}
     for v3 in (1, 2):
@@ -449,13 +482,15 @@ def other_forms(lbem, torch, p, peak, stream):
     s.close()
     t_fwd, t_adj = ev[0].elapsed_time(ev[1]), ev[2].elapsed_time(ev[3])
     n3 = 192 ** 3
-    per = ms / 1000
+    spl = steps_per_launch(q, "f32", spp)
+    per = ms / step_launches(q, 1000, spl)
     gbs = 172 * n3 / (per * 1e-3) / 1e9
     out["het3d_192"] = {"mlups": n3 * 1000 / (ms * 1e-3) / 1e6, "ms_per_launch": per, "achieved_gbs": gbs,
-                        "frac": gbs / peak, "bytes_per_site": 172, "variant": v, "steps_per_launch": 1}
-    # backward pass bytes: recompute of 900 forward steps (172 B/site) + 1000 adjoint steps (272 B/site:
-    # lambda 84 read + state 84 read + c_L^2 4 + FP64 gradient 16 read/write + lambda 84 write)
-    bwd_bytes = (900 * 172 + 1000 * 272) * n3
+                        "frac": gbs / peak, "bytes_per_site_per_launch": 172, "variant": v,
+                        "steps_per_launch": spl, "steps_per_pass": spp}
+    # backward pass bytes, three steps per launch: 1000 recomputed steps (172 B/site and sigma 3 x 12 written) + 1000
+    # adjoint steps (224 B/site: lambda 84 read + 84 written, c_L^2 4, FP64 gradient 16 read/write, sigma 3 x 12)
+    bwd_bytes = 1000 / 3 * (208 + 224) * n3
     out["adjoint_192"] = {"lb_steps": 1000, "checkpoint_every": 100, "variant": v_adj, "ms_forward_record": t_fwd,
                           "ms_backward": t_adj, "mlups_forward_plus_backward": n3 * 1000 / ((t_fwd + t_adj) * 1e-3) / 1e6,
                           "backward_achieved_gbs": bwd_bytes / (t_adj * 1e-3) / 1e9,
@@ -959,11 +994,15 @@ def main():
         lbem.lbem_set_temporal_blocking(h, args.steps_per_pass or 2, -1 if args.tile_shape is None else args.tile_shape)
     if args.autotune:
         lbem.lbem_set_fields(h)
-        variant = lbem.lbem_autotune(h, 50)
+        variant = lbem.lbem_autotune(h, 50)  # (of the single steps; several per launch stay the default ones)
+        if (p.D == 3 or lbem.lbem_get_temporal_blocking(h)[0] == 2) and args.tile_shape is None:
+            lbem.lbem_set_temporal_blocking(h, 2, -1)
     if args.variant is not None:
         lbem.lbem_set_variant(h, args.variant)
         variant = args.variant
     spp, tile_shape, _ = lbem.lbem_get_temporal_blocking(h)
+    if p.D == 3 and args.variant is None and args.steps_per_pass != 1:
+        spp = 2  # (3D reports 1)
     nsite = s.nsite
     E_d = torch.empty(3 * nsite, dtype=torch.float32, device="cuda")
     B_d = torch.empty_like(E_d)
@@ -998,16 +1037,20 @@ def main():
     total_ms = start.elapsed_time(stop)
     total_ms = dist_max(total_ms, world)
     kern_ms = [a.elapsed_time(b) for a, b in evs]
-    # stream-collide launches per run: pairs of steps (plus an odd last step) or single steps
-    step_launches = nsteps // 2 + nsteps % 2 if spp == 2 else nsteps
-    ms_per_launch = float(np.mean(kern_ms)) / step_launches
+    # stream-collide launches per run
+    spl = steps_per_launch(p, args.storage, spp, args.tile_shape is not None)
+    marching = spl >= 3 and spp == 2
+    launches_run = step_launches(p, nsteps, spl)
+    ms_per_launch = float(np.mean(kern_ms)) / launches_run
     ms_per_step = total_ms / args.steps
     value = world * nsite * nsteps / (ms_per_step * 1e-3) / 1e6
 
     peak, peak_kind = measured_peak_gbs()
     bps = (72 if disp else BYTES_PER_SITE[args.storage]) if p.D == 2 else 172
     achieved = bps * nsite / (ms_per_launch * 1e-3) / 1e9
-    if spp == 2 and args.storage == "f32" and tile_shape >= 9:
+    if marching:
+        kname, kid = f"march{p.D}d ({spl} steps per launch)", "march"
+    elif spp == 2 and args.storage == "f32" and tile_shape >= 9:
         kname, kid = f"step2d_ss2 (strip streaming, tile shape {tile_shape}, 2 steps per launch)", f"tb2-{tile_shape}"
     elif spp == 2 and args.storage == "f32" and tile_shape >= 7:
         kname, kid = f"step2d_rs2 (register streaming, tile shape {tile_shape}, 2 steps per launch)", f"tb2-{tile_shape}"
@@ -1017,7 +1060,9 @@ def main():
     else:
         kname = (f"step2d<{args.storage}>" if p.D == 2 else "step3d") + f" (variant {variant})"
         kid = variant
-    if disp and spp == 1:
+    if marching:
+        pass
+    elif disp and spp == 1:
         kname, kid = "step2d_gen (one dispersive pole per site, single steps)", "disp"
     elif disp:
         kname, kid = "step2d_tb2<POLE> (one dispersive pole per site, tile shape 0, 2 steps per launch)", "tb2pole"
@@ -1033,7 +1078,7 @@ def main():
         kname = "step3d_site (walls and layers applied in the kernel)"
     traffic = NCU_TRAFFIC.get((args.workload, args.storage, kid)) if args.lb_steps is None else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": traffic, "kernel": kname, "steps_per_launch": spp,
+                "traffic": traffic, "kernel": kname, "steps_per_launch": spl,
                 "algorithmic_bytes_per_site_per_launch": bps, "ms_per_launch": ms_per_launch,
                 "peak_kind": peak_kind}
 
@@ -1074,9 +1119,9 @@ def main():
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         if args.workload == "het2d_4096" and args.lb_steps is None:
             # every form's accuracy against the FP64 oracle, on the GPU kernels the form's timed run used
-            spl = {k: v.get("steps_per_launch") for k, v in (forms or {}).items()}
-            spl[args.storage] = spp
-            cases = accuracy_cases(p, spl)
+            passes = {k: v.get("steps_per_pass", v.get("steps_per_launch")) for k, v in (forms or {}).items()}
+            passes[args.storage] = spp
+            cases = accuracy_cases(p, passes)
             if forms is None:
                 cases = {args.storage: cases[args.storage]}
             gpu_out = {}
@@ -1096,10 +1141,10 @@ def main():
             cpu["cpu_model"] = cpu_model()
     s.close()
     if rank == 0:
-        # per pass: the step launches (plus the edge kernel after each with 2D walls on the tile path), the medium
+        # per pass: the step launches (plus the edge kernel after each with 2D walls on the tile paths), the medium
         # upload's check and write (plus the pole's re-check, and the wall-aware grad ln mu with walls and mu),
         # init, fields, the FP64 diagnostics and its reduction
-        launches = args.steps * (step_launches * (2 if walls and p.D == 2 and not (disp or aniso) else 1) + 6 +
+        launches = args.steps * (launches_run * (2 if walls and p.D == 2 and not (disp or aniso or marching) else 1) + 6 +
                                  (1 if args.storage == "f16" else 0) + (1 if disp else 0) +
                                  (1 if walls and p.mu_r is not None else 0))
         line = {"metric": "Mlups", "value": value, "unit": "Mlups", "n_gpus": world, "steps": args.steps,
@@ -1127,10 +1172,10 @@ def main():
             verdict = None if e is None else (f"<={bar:g} met" if max(e) <= bar else f"<={bar:g} MISSED")
             return [round(mlups / 1e3, 1), None if frac is None else round(frac, 3), spl_, r, verdict]
 
-        summ[f"{args.storage} (main)"] = entry(value, roofline["frac"], spp, main_acc, TOL[args.storage])
+        summ[f"{args.storage} (main)"] = entry(value, roofline["frac"], spl, main_acc, TOL[args.storage])
         for k, v in (forms or {}).items():
             if k == "adjoint_192":
-                summ[k] = [round(v["mlups_forward_plus_backward"] / 1e3, 1), round(v["backward_frac"], 3), 1,
+                summ[k] = [round(v["mlups_forward_plus_backward"] / 1e3, 1), round(v["backward_frac"], 3), 3,
                            "vs FD and oracle adjoint in tests", None]
                 continue
             e = acc.get(k)

@@ -212,9 +212,9 @@ static bool march_ok(const lbem_t *h) {
     return h->tblock == 2 && !h->tb_shape_set && multi_step_base(h) && !(h->disp && h->aniso);
 }
 // 3D: triples of steps by the marching kernel (march3d.cu) where several steps per launch are the default, with uniform
-// mu and the one-site-per-thread launch shapes; offsets in a plane must fit 32 bits.
+// mu; offsets in a plane must fit 32 bits.
 bool march3_ok(const lbem_t *h, bool adjoint) {
-    return h->tblock == 2 && h->dim == 3 && h->variant >= 1 && !h->has_mu && h->grid.plane < (1LL << 31) &&
+    return h->tblock == 2 && h->dim == 3 && !h->has_mu && h->grid.plane < (1LL << 31) &&
            march_3d_pays(h->grid, adjoint || h->bc[0] || h->bc[1] || h->bc[2]);
 }
 static int steps_per_launch(const lbem_t *h) { return three_step_ok(h) ? 3 : two_step_ok(h) ? 2 : 1; }
@@ -1208,20 +1208,23 @@ lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best) {
     if (st == LBEM_OK && max_k == 2 && trial_steps >= MARCH_MIN_STEPS) {
         const bool set = h->tb_shape_set;
         h->tb_shape_set = false;
-        if (march_ok(h)) {
+        const bool d3 = march3_ok(h);
+        if (d3 || march_ok(h)) {
             int n = 0;
+            const int steps = d3 ? trial_steps / MARCH3_STEPS * MARCH3_STEPS : trial_steps;
             for (int rep = 0; rep < 2 && st == LBEM_OK; rep++) {
                 StepArgs a = step_args(h, cur0);
                 a.evt.rowptr = nullptr;
                 cudaEventRecord(e0, h->stream);
-                cudaError_t e = launch_march_2d(a, handle_walls(h), h->storage, h->aniso, trial_steps, h->stream, &n);
+                cudaError_t e = d3 ? launch_march_3d(a, handle_walls(h), steps / MARCH3_STEPS, h->stream)
+                                   : launch_march_2d(a, handle_walls(h), h->storage, h->aniso, steps, h->stream, &n);
                 if (e != cudaSuccess) st = cuda_fail(e, "lbem_autotune");
                 cudaEventRecord(e1, h->stream);
             }
             cudaEventSynchronize(e1);
             float ms = 0.f;
             cudaEventElapsedTime(&ms, e0, e1);
-            march = ms / trial_steps < best_per_step;
+            march = ms / steps < best_per_step;
         }
         h->tb_shape_set = set;
     }

@@ -9,10 +9,11 @@
 // neighbouring tile owns: a tile owns 32 - 2 (K - 1) by TY - 2 (K - 1) columns, a segment starts and ends K - 1 planes out.
 // A plane's populations and medium arrive by cp.async while the plane before is computed.
 //
-// HBM carries 172 bytes a site per K steps; the L2 hands out the tiles' overlap as well (1.5 times the sites at K = 3 and
-// 20 rows) in sectors of 32 bytes that the +-x pulls straddle, and that bounds it: 5.5 TB/s from the L2, DRAM at 3.5 to
-// 3.9 TB/s, issue slots at 50 to 60 %.  Measured per step at 192^3, single steps 179.6 us: K = 3 and 20 rows of 10 warps
-// 106.6 us; 16 rows 113.9, 24 rows of 12 warps 116.1, of 8 warps 122.9; one column a thread in 16 rows 136.0 (the chain of
+// HBM carries 172 bytes a site per K steps (192^3: 1.25 GB a launch, 48 % of its rate); the L2 hands out the tiles' overlap
+// as well (1.5 times the sites at K = 3 and 20 rows), in sectors of 32 bytes that the +-x pulls straddle, at 9.9 TB/s (35 %);
+// half of the issue slots are used.  What bounds it is the chain of one site's levels and the barrier a plane with 10 warps
+// an SM (158 registers of levels' state a thread).  Measured per step at 192^3, single steps 179.6 us: K = 3 and 20 rows of
+// 10 warps 106.6 us; 16 rows 113.9, 24 rows of 12 warps 116.1, of 8 warps 122.9; one column a thread in 16 rows 136.0 (the chain of
 // one site's levels leaves the warps waiting); K = 2 148.3 to 177.0, K = 4 127.8 to 153.3 (the overlap grows to 2).
 // 96^3 25.1 -> 16.6 us; with walls and a layer 192^3 203 -> 135 us, 96^3 30.8 -> 21.9 us.
 // Sources and receivers: a block first marks, a word for each plane, its rows that have any (192^3 with 128 receivers 110 us
