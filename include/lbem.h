@@ -232,7 +232,7 @@ lbem_status lbem_set_dispersion(lbem_t *h, const float *wp2, const float *wr2, c
  * growth without sources), so a jump means an over-driven source or a corrupted state. */
 lbem_status lbem_set_watchdog(lbem_t *h, int every, double max_growth);
 
-/* Temporal blocking (2D; 16-bit storage needs uniform mu and nx % 4 == 0; otherwise ignored).  With
+/* Temporal blocking (2D: 16-bit storage needs uniform mu and nx % 4 == 0, otherwise ignored; 3D: see the end).  With
  * steps_per_pass = 2 (the default) lbem_step advances pairs of steps with one kernel that stages a tile plus
  * a two-site halo in shared memory and performs both steps there, so the state crosses HBM once per two steps
  * (44 instead of 88 bytes per site and step pair for FP32); an odd last step is a single step.  For FP32
@@ -265,10 +265,13 @@ lbem_status lbem_set_watchdog(lbem_t *h, int every, double max_growth);
  * no pass after it).  The results are the same bits again: those of single steps for FP32 storage, of launches of two
  * steps for 16-bit storage, whose state is rounded after every second step.  A tile shape >= 0 gives launches of two
  * steps.
+ * 3D: with steps_per_pass = 2 (the default) and uniform mu, steps run three per launch where that takes less time than
+ * single steps (not on small grids), walls and layers included, what is left over one by one; the same bits.  With 1, or
+ * a heterogeneous mu, every step is a single step.
  * LBEM_ERR_ARG for values outside the current handle's set. */
 lbem_status lbem_set_temporal_blocking(lbem_t *h, int steps_per_pass, int tile_shape);
 
-/* Steps per launch in effect (2 or 3 only where that kernel is enabled and applies), the tile shape (the one
+/* Steps per pass in effect (2 or 3 only where that kernel is enabled and applies in 2D; 1 in 3D), the tile shape (the one
  * launched when two steps per launch are in effect, else as set or autotuned) and the number of tile shapes of
  * the selected steps per pass; any pointer may be NULL. */
 lbem_status lbem_get_temporal_blocking(const lbem_t *h, int *steps_per_pass, int *tile_shape, int *nshapes);
@@ -386,14 +389,17 @@ lbem_status lbem_halo_in(lbem_t *h, int halo, const float *from_below, const flo
 
 /* Forward run that records what the adjoint needs: advances nsteps steps from
  * the current state (receivers record as in lbem_step) and keeps a copy of the
- * state every `checkpoint_every` steps in handle-owned device memory.  FP32
- * storage, uniform mu (LBEM_ERR_STATE otherwise). */
+ * state every `checkpoint_every` steps in handle-owned device memory; in 3D, where
+ * it takes no more memory than those copies and a segment's states together, the
+ * population sums of every step instead, and nothing is recomputed.  The memory
+ * serves the handle's next recorded run, if that is of a like size, and is freed
+ * with the handle.  FP32 storage, uniform mu (LBEM_ERR_STATE otherwise). */
 lbem_status lbem_forward_record(lbem_t *h, int nsteps, int checkpoint_every);
 
 /* Reverse-time adjoint of the last lbem_forward_record: given the cotangent of
  * the receiver traces dL/dtrace ([nrec][nsteps] floats, host or device), writes
  * dL/d eps_r ([nsite] floats, host or device).  Recomputes each checkpoint
- * segment forward, then runs the hand-written adjoint stream-collide kernel
+ * segment forward (unless every step was kept), then runs the hand-written adjoint stream-collide kernel
  * backwards through it; the gradient accumulates over time steps in FP64.
  * If grad_cL2 is not NULL it also receives dL/dc_L^2 ([nsite] doubles). */
 lbem_status lbem_adjoint(lbem_t *h, const float *trace_cot, float *grad_eps, double *grad_cL2);
@@ -405,8 +411,8 @@ lbem_status lbem_adjoint(lbem_t *h, const float *trace_cot, float *grad_eps, dou
  * *best (may be NULL) receives the chosen variant id.  Where two steps per
  * launch apply and are enabled (lbem_set_temporal_blocking), every tile shape
  * of that kernel is timed too; the fastest is kept, and two-step launches stay
- * on only if they beat the best single-step kernel.  The marching kernel (8 steps per launch) is timed beside them
- * where it applies; if it wins, the default without a tile shape is kept. */
+ * on only if they beat the best single-step kernel.  The marching kernel (2D and 3D) is timed beside them where
+ * it applies; if it wins, the default without a tile shape is kept. */
 lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best);
 lbem_status lbem_set_variant(lbem_t *h, int variant);
 lbem_status lbem_get_variant(const lbem_t *h, int *variant, int *nvariants);
@@ -414,7 +420,7 @@ lbem_status lbem_get_variant(const lbem_t *h, int *variant, int *nvariants);
 /* ---------------------------------------------------------------- batches of independent media */
 
 /* A batch steps n independent 2D FP32 handles (members, of any sizes) with one
- * kernel launch per step, or per pair of steps, over a flattened work table of
+ * kernel launch per step, per two or per eight, over a flattened work table of
  * all members; runs of steps are captured once into a CUDA graph and replayed.
  * Members keep their own medium, fields, sources, receivers and outputs (use
  * the calls above on them); all members must be at the same time t when
@@ -428,8 +434,10 @@ lbem_status lbem_get_variant(const lbem_t *h, int *variant, int *nvariants);
  * odd step count takes one single step first); 14, 15 advance two steps per
  * launch over the same packed copy by strip streaming (persistent CTAs take
  * units of 30 or 34 rows of a member's 128-column strip from a queue and stream
- * them in chunks of 4 or 3 rows through shared-memory stages).  Every variant
- * gives the same bits as each member stepped alone. */
+ * them in chunks of 4 or 3 rows through shared-memory stages); 16 (the default)
+ * marches 8 steps per launch over units of the members' own states, as lbem_step
+ * does on one grid.  Every variant gives the same bits as each member stepped
+ * alone. */
 lbem_status lbem_batch_create(int n, lbem_t *const *members, void *stream, lbem_batch_t **out);
 lbem_status lbem_batch_step(lbem_batch_t *b, int nsteps);
 /* Time every variant over trial_steps steps (members' states saved and restored) and keep the fastest; *best (may

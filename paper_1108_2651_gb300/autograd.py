@@ -3,7 +3,8 @@
 receiver_traces(eps, problem, ...) returns the receiver traces [nrec, nsteps]
 of a run from zero initial fields in the medium eps_r = eps (uniform mu);
 its backward calls lbem_adjoint, the reverse-time adjoint stream-collide
-kernel with checkpoint-and-recompute every `checkpoint_every` steps and the
+kernel with checkpoint-and-recompute every `checkpoint_every` steps (in 3D only
+where keeping every step's population sums would take more memory) and the
 gradient accumulated over time steps in FP64.  Any loss of the traces can be
 differentiated, e.g. the L2 misfit 1/2 sum (traces - obs)^2.
 """
