@@ -434,9 +434,9 @@ lbem_status lbem_get_variant(const lbem_t *h, int *variant, int *nvariants);
  * odd step count takes one single step first); 14, 15 advance two steps per
  * launch over the same packed copy by strip streaming (persistent CTAs take
  * units of 30 or 34 rows of a member's 128-column strip from a queue and stream
- * them in chunks of 4 or 3 rows through shared-memory stages); 16 (the default)
- * marches 8 steps per launch over units of the members' own states, as lbem_step
- * does on one grid.  Every variant gives the same bits as each member stepped
+ * them in chunks of 4 or 3 rows through shared-memory stages); 16 marches 8 steps
+ * per launch over units of the members' own states, as lbem_step does on one
+ * grid.  A new batch has variant 0.  Every variant gives the same bits as each member stepped
  * alone. */
 lbem_status lbem_batch_create(int n, lbem_t *const *members, void *stream, lbem_batch_t **out);
 lbem_status lbem_batch_step(lbem_batch_t *b, int nsteps);
