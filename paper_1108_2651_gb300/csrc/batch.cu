@@ -600,7 +600,6 @@ static lbem_status upload_unit_tables(lbem_batch_t *b, int shape) {
     if (ul.size() > (size_t)(1 << 30)) return fail(LBEM_ERR_ARG, "lbem_batch: too many units");
     if (b->units_cap < ul.size()) {
         cudaFree(b->d_units);
-    cudaFree(b->d_march);
         b->d_units = nullptr;
         b->units_cap = 0;
         if (cudaMalloc((void **)&b->d_units, sizeof(BatchUnit) * ul.size()) != cudaSuccess) {
@@ -956,6 +955,7 @@ void lbem_batch_destroy(lbem_batch_t *b) {
     cudaFree(b->d_args);
     cudaFree(b->d_tiles);
     cudaFree(b->d_units);
+    cudaFree(b->d_march);
     cudaFree(b->d_sched);
     cudaFree(b->d_r0);
     cudaFree(b->d_pack);
