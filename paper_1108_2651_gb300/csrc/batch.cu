@@ -708,15 +708,11 @@ static cudaError_t launch_batch(lbem_batch_t *b, int variant, int offset) {
         case -7: step2d_batch_lin<1><<<blocks, BLOCK, 0, b->stream>>>(b->d_members, b->d_wstart, b->d_map, nw, b->d_t0, offset); break;
         case -8: step2d_batch_lin<5><<<blocks, BLOCK, 0, b->stream>>>(b->d_members, b->d_wstart, b->d_map, nw, b->d_t0, offset); break;
         default: {
-            static int per_sm = 0, nsm = 0;
-            if (!per_sm) {
-                int dev = 0;
-                cudaGetDevice(&dev);
-                cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_batch_pipe, BLOCK, 0);
-                if (per_sm < 1) per_sm = 1;
-            }
-            const long long warps = (long long)per_sm * nsm * (BLOCK / 32);
+            static PerDevice<KernelFit> fits;
+            KernelFit fit;
+            const cudaError_t fe = kernel_fit(fits, step2d_batch_pipe, BLOCK, 0, &fit);
+            if (fe != cudaSuccess) return fe;
+            const long long warps = (long long)fit.per_sm * fit.nsm * (BLOCK / 32);
             const long long per_warp = (nw + warps - 1) / warps;
             const long long used = (nw + per_warp - 1) / per_warp;
             const unsigned pb = (unsigned)((used * 32 + BLOCK - 1) / BLOCK);

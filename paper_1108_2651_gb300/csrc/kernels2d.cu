@@ -243,17 +243,13 @@ __global__ void __launch_bounds__(BLOCK) step2d_pipe(StepArgs a) {
 
 template <int ST, bool MU>
 static cudaError_t launch_pipe(const StepArgs &a, cudaStream_t s) {
-    static int per_sm = 0, nsm = 0;  // resident blocks per SM of this instantiation, SM count
-    if (!per_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_pipe<ST, MU>, BLOCK, 0);
-        if (per_sm < 1) per_sm = 1;
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, step2d_pipe<ST, MU>, BLOCK, 0, &fit);
+    if (fe != cudaSuccess) return fe;
     const long long units = (long long)a.g.ny * (a.g.nchunk_pad / 32);
     long long blocks = (units * 32 + BLOCK - 1) / BLOCK;
-    blocks = blocks < (long long)per_sm * nsm ? blocks : (long long)per_sm * nsm;
+    blocks = blocks < (long long)fit.per_sm * fit.nsm ? blocks : (long long)fit.per_sm * fit.nsm;
     step2d_pipe<ST, MU><<<(unsigned)blocks, BLOCK, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -484,20 +480,14 @@ __global__ void __launch_bounds__(BLOCK) step2d_async(StepArgs a) {
 
 template <int ST, bool MU>
 static cudaError_t launch_async(const StepArgs &a, cudaStream_t s) {
-    static int per_sm = 0, nsm = 0;
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
     const size_t smem = (size_t)(BLOCK / 32) * KS * 32 * (SLOT + sizeof(ExSlot));
-    if (!per_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaError_t e = cudaFuncSetAttribute(step2d_async<ST, MU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_async<ST, MU>, BLOCK, smem);
-        if (per_sm < 1) per_sm = 1;
-    }
+    const cudaError_t fe = kernel_fit(fits, step2d_async<ST, MU>, BLOCK, smem, &fit);
+    if (fe != cudaSuccess) return fe;
     const long long units = (long long)a.g.ny * (a.g.nchunk_pad / 32);
     long long blocks = (units * 32 + BLOCK - 1) / BLOCK;
-    blocks = blocks < (long long)per_sm * nsm ? blocks : (long long)per_sm * nsm;
+    blocks = blocks < (long long)fit.per_sm * fit.nsm ? blocks : (long long)fit.per_sm * fit.nsm;
     step2d_async<ST, MU><<<(unsigned)blocks, BLOCK, smem, s>>>(a);
     return cudaGetLastError();
 }

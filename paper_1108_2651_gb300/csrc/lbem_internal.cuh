@@ -22,15 +22,44 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
 #include "../../include/lbem.h"
+#include "per_device.cuh"
 
 namespace lbk {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int BLOCK = 256;  // threads per block of the stencil kernels
+
+// What a launch needs to know of a kernel on the current device: its resident blocks per SM (at least 1) and the SMs.
+struct KernelFit {
+    int per_sm = 0, nsm = 0;
+};
+// Sets the kernel's dynamic shared memory (and, with carveout, all of L1 as shared memory) and asks for its fit, once
+// per device; `at` is the instantiation's own record.
+template <class Kernel>
+cudaError_t kernel_fit(PerDevice<KernelFit> &at, Kernel *k, int threads, size_t smem, KernelFit *fit,
+                       bool carveout = false) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)at.get(
+        dev,
+        [&](KernelFit &f) {
+            cudaError_t q = cudaDeviceGetAttribute(&f.nsm, cudaDevAttrMultiProcessorCount, dev);
+            if (q == cudaSuccess && smem)
+                q = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (q == cudaSuccess && carveout)
+                q = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+            if (q == cudaSuccess) q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f.per_sm, k, threads, smem);
+            f.per_sm = std::max(f.per_sm, 1);
+            return (int)q;
+        },
+        fit);
+}
 
 // ------------------------------------------------------------------ storage
 struct PopBuf {

@@ -903,23 +903,15 @@ template <int ST, int MED, bool WL, int K, int D>
 static cudaError_t launch_march(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches) {
     using Cfg = MarchCfg<ST, MED, K, D>;
     auto *k = march2d<ST, MED, WL, K, D>;
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, 32, Cfg::smem);
-        if (e != cudaSuccess) return e;
-        per_sm = std::max(n, 1);
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    cudaError_t fe = kernel_fit(fits, k, 32, Cfg::smem, &fit, true);
+    if (fe != cudaSuccess) return fe;
     MarchArgs m;
     m.a = a;
     m.w = w;
     m.nstrips = (a.g.nchunk + Cfg::W / 4 - 1) / (Cfg::W / 4);
-    const int cap = per_sm * nsm;
+    const int cap = fit.per_sm * fit.nsm;
     m.nl = m.nr = m.nsegx = m.he = m.hex = 0;
     if (WL && w.kind[0]) {  // strips whose columns (with the halo) reach a wall or its layer
         const int edge = std::max(w.nlayer, 1);

@@ -386,21 +386,15 @@ template <int K, int NW, int NR, bool WL, int MODE>
 static cudaError_t launch_march3(const StepArgs &a, const Walls &w, const Adj3 &adj, int nlaunch, cudaStream_t s) {
     constexpr int TY = NW * NR, smem = (2 * (K - 1) * 6 + 22 + (MODE == M3_ADJOINT ? 3 * K + 2 : 0)) * TY * 32 * 4;
     auto *k = march3d<K, NW, NR, WL, MODE>;
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, 32 * NW, smem);
-        if (e != cudaSuccess) return e;
-        per_sm = std::max(n, 1);
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, k, 32 * NW, smem, &fit);
+    if (fe != cudaSuccess) return fe;
     March3Args m;
     m.a = a;
     m.w = w;
     m.adj = adj;
-    plan3<K, TY>(a.g, per_sm * nsm, &m.ntx, &m.nty, &m.nseg);
+    plan3<K, TY>(a.g, fit.per_sm * fit.nsm, &m.ntx, &m.nty, &m.nseg);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;

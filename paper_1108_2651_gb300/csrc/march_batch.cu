@@ -19,18 +19,12 @@ __global__ void __launch_bounds__(32, 8) march2d_batch(const StepArgs *__restric
                                                                  (unsigned)__cvta_generic_to_shared(march_smem));
 }
 
+static PerDevice<KernelFit> batch_fits;
+
 static int resident_units() {
-    static int cap = 0;
-    if (!cap) {
-        int dev = 0, nsm = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(march2d_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, BatchCfg::smem);
-        cudaFuncSetAttribute(march2d_batch, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, march2d_batch, 32, BatchCfg::smem);
-        cap = std::max(1, n * nsm);
-    }
-    return cap;
+    KernelFit fit;
+    kernel_fit(batch_fits, march2d_batch, 32, BatchCfg::smem, &fit, true);
+    return std::max(1, fit.per_sm * fit.nsm);
 }
 
 // The units of members with these grids: segments of at most R rows, evenly cut, tall ones first, for the R whose units,
@@ -69,6 +63,9 @@ std::vector<BatchMarchUnit> batch_march_units(int n, const Grid *grids) {
 
 cudaError_t launch_batch_march(const StepArgs *args, const BatchMarchUnit *units, int nunits, const long long *t0p,
                                int toff, int steps, int par, cudaStream_t s) {
+    KernelFit fit;
+    const cudaError_t e = kernel_fit(batch_fits, march2d_batch, 32, BatchCfg::smem, &fit, true);
+    if (e != cudaSuccess) return e;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;

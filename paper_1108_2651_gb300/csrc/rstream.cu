@@ -234,17 +234,13 @@ __global__ void __launch_bounds__(128, MINB) step2d_rs2(StepArgs a, int nstrips,
 
 template <int MINB>
 static cudaError_t launch_rs(const StepArgs &a, cudaStream_t s) {
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_rs2<MINB>, 128, 0);
-        if (per_sm < 1) per_sm = 1;
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, step2d_rs2<MINB>, 128, 0, &fit);
+    if (fe != cudaSuccess) return fe;
     const int nstrips = (a.g.nx + 127) / 128;
     // one wave: about as many (strip, segment) warps as fit on the GPU at once, segments of at least 8 rows
-    const long long resident = (long long)per_sm * nsm * 4;
+    const long long resident = (long long)fit.per_sm * fit.nsm * 4;
     int nseg = (int)(resident / nstrips);
     if (nseg < 1) nseg = 1;
     int H = (a.g.ny + nseg - 1) / nseg;

@@ -757,17 +757,10 @@ static cudaError_t launch_ss(const StepArgs &a, cudaStream_t s) {
     constexpr int NT = (2 * TBY + 2) * 32;
     static_assert(MCH <= 32, "a unit's event flags are one 32-bit mask");
     if (!a.sched) return cudaErrorInvalidValue;
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(step2d_ss2<TBY, S, MINB, AN, MU>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::BYTES);
-        if (e != cudaSuccess) return e;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_ss2<TBY, S, MINB, AN, MU>, NT, Gm::BYTES);
-        if (per_sm < 1) per_sm = 1;
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, step2d_ss2<TBY, S, MINB, AN, MU>, NT, Gm::BYTES, &fit);
+    if (fe != cudaSuccess) return fe;
     CUtensorMap mIn, mCL, mIn4, mCL4, mDL, mDL4;
     memset(&mIn, 0, sizeof mIn);
     memset(&mCL, 0, sizeof mCL);
@@ -783,7 +776,7 @@ static cudaError_t launch_ss(const StepArgs &a, cudaStream_t s) {
     U.nstrip = (a.g.nx + SBX - 1) / SBX;
     U.H = MCH * TBY - 2;
     U.Hs = 2 * TBY - 2;
-    const long long slots = (long long)per_sm * nsm;
+    const long long slots = (long long)fit.per_sm * fit.nsm;
     const long long small_rows = (2 * slots + U.nstrip - 1) / U.nstrip * U.Hs;  // about two short units per CTA
     const long long big_runs = small_rows >= a.g.ny ? 0 : (a.g.ny - small_rows) / U.H;
     U.nbig = (int)(big_runs * U.nstrip);
@@ -1093,23 +1086,16 @@ static cudaError_t launch_bss(const StepArgs *args, const BatchUnit *units, int 
                               cudaStream_t s) {
     using Gm = SsGeom<TBY, S, true>;
     constexpr int NT = (2 * TBY + 2) * 32;
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(step2d_batch_ss2<TBY, S, MINB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::BYTES);
-        if (e != cudaSuccess) return e;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_batch_ss2<TBY, S, MINB>, NT, Gm::BYTES);
-        if (per_sm < 1) per_sm = 1;
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, step2d_batch_ss2<TBY, S, MINB>, NT, Gm::BYTES, &fit);
+    if (fe != cudaSuccess) return fe;
     CUtensorMap mA, mB, mCL;
     memset(&mA, 0, sizeof mA);
     memset(&mB, 0, sizeof mB);
     memset(&mCL, 0, sizeof mCL);
     if (!ss_batch_maps(pk, rows, TBY, &mA, &mB, &mCL)) return cudaErrorNotSupported;
-    const long long slots = (long long)per_sm * nsm;
+    const long long slots = (long long)fit.per_sm * fit.nsm;
     const int blocks = (int)(nunits < slots ? nunits : slots);
     if (blocks < 1) return cudaSuccess;
     step2d_batch_ss2<TBY, S, MINB>

@@ -715,20 +715,13 @@ static cudaError_t launch_batch_tb(const StepArgs *args, const BatchTile *tiles,
                                    const long long *t0p, int toff, int par, const BatchPacked &pk, long long rows,
                                    cudaStream_t s) {
     using Gm = TbGeom<TBY>;
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(step2d_batch_tb2<TBY, NT, MINB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::BYTES);
-        if (e != cudaSuccess) return e;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_batch_tb2<TBY, NT, MINB>, NT, Gm::BYTES);
-        if (per_sm < 1) per_sm = 1;
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, step2d_batch_tb2<TBY, NT, MINB>, NT, Gm::BYTES, &fit);
+    if (fe != cudaSuccess) return fe;
     CUtensorMap mA, mB, mCL;
     if (!make_batch_maps<TBY>(pk, rows, &mA, &mB, &mCL)) return cudaErrorNotSupported;
-    const long long slots = (long long)per_sm * nsm;
+    const long long slots = (long long)fit.per_sm * fit.nsm;
     const unsigned blocks = (unsigned)(ntiles < slots ? ntiles : slots);
     if (blocks == 0) return cudaSuccess;
     step2d_batch_tb2<TBY, NT, MINB><<<blocks, NT, Gm::BYTES, s>>>(args, tiles, ntiles, t0p, toff, par, pk, mA, mB, mCL);
@@ -1093,18 +1086,10 @@ static bool make_pole_maps(const StepArgs &a, PoleMaps<true> *pm) {
 template <int TBY, int NT, int MINB, bool MU = false, bool AN = false, bool POLE = false>
 static cudaError_t launch_tb(const StepArgs &a, cudaStream_t s) {
     using Gm = TbGeom<TBY, MU, POLE>;
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(step2d_tb2<TBY, NT, MINB, MU, AN, POLE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::BYTES);
-        if (e != cudaSuccess) return e;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_tb2<TBY, NT, MINB, MU, AN, POLE>, NT,
-                                                      Gm::BYTES);
-        if (per_sm < 1) per_sm = 1;
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, step2d_tb2<TBY, NT, MINB, MU, AN, POLE>, NT, Gm::BYTES, &fit);
+    if (fe != cudaSuccess) return fe;
     CUtensorMap mIn, mCL, mDL;
     PoleMaps<POLE> pm;
     memset(&mIn, 0, sizeof mIn);
@@ -1116,7 +1101,7 @@ static cudaError_t launch_tb(const StepArgs &a, cudaStream_t s) {
     const int use_tma = tma ? 1 : 0;
     const int ntx = (a.g.nx + TBX - 1) / TBX, nty = (a.g.ny + TBY - 1) / TBY;
     const int ntiles = ntx * nty;
-    const int blocks = ntiles < per_sm * nsm ? ntiles : per_sm * nsm;
+    const int blocks = ntiles < fit.per_sm * fit.nsm ? ntiles : fit.per_sm * fit.nsm;
     step2d_tb2<TBY, NT, MINB, MU, AN, POLE>
         <<<blocks, NT, Gm::BYTES, s>>>(a, mIn, mCL, mDL, pm, use_tma, ntx, nty, blocks / ntx, blocks % ntx);
     return cudaGetLastError();
@@ -1417,17 +1402,10 @@ __global__ void __launch_bounds__(NT, MINB)
 template <int TBY, int NT, int MINB>
 static cudaError_t launch_tb3(const StepArgs &a, cudaStream_t s) {
     using Gm = TbGeom3<TBY>;
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(step2d_tb3<TBY, NT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)Gm::BYTES);
-        if (e != cudaSuccess) return e;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_tb3<TBY, NT, MINB>, NT, Gm::BYTES);
-        if (per_sm < 1) per_sm = 1;
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, step2d_tb3<TBY, NT, MINB>, NT, Gm::BYTES, &fit);
+    if (fe != cudaSuccess) return fe;
     CUtensorMap mIn, mCL;
     memset(&mIn, 0, sizeof mIn);
     memset(&mCL, 0, sizeof mCL);
@@ -1435,7 +1413,7 @@ static cudaError_t launch_tb3(const StepArgs &a, cudaStream_t s) {
     const int use_tma = (a.g.ny >= TBY + 6 && make_maps<TBY + 2>(a, &mIn, &mCL)) ? 1 : 0;
     const int ntx = (a.g.nx + TBX - 1) / TBX, nty = (a.g.ny + TBY - 1) / TBY;
     const int ntiles = ntx * nty;
-    const int blocks = ntiles < per_sm * nsm ? ntiles : per_sm * nsm;
+    const int blocks = ntiles < fit.per_sm * fit.nsm ? ntiles : fit.per_sm * fit.nsm;
     step2d_tb3<TBY, NT, MINB><<<blocks, NT, Gm::BYTES, s>>>(a, mIn, mCL, use_tma, ntx, nty, blocks / ntx,
                                                             blocks % ntx);
     return cudaGetLastError();
@@ -1486,17 +1464,10 @@ static bool make_maps16(const StepArgs &a, CUtensorMap *mIn, CUtensorMap *mCL, C
 template <int ST, int TBY, int NT, int MINB>
 static cudaError_t launch_tb16(const StepArgs &a, cudaStream_t s) {
     using Gm = TbGeomH<ST, TBY>;
-    static int per_sm = 0, nsm = 0;
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(step2d_tb2h<ST, TBY, NT, MINB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::BYTES);
-        if (e != cudaSuccess) return e;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step2d_tb2h<ST, TBY, NT, MINB>, NT, Gm::BYTES);
-        if (per_sm < 1) per_sm = 1;
-    }
+    static PerDevice<KernelFit> fits;
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(fits, step2d_tb2h<ST, TBY, NT, MINB>, NT, Gm::BYTES, &fit);
+    if (fe != cudaSuccess) return fe;
     CUtensorMap mIn, mCL, mEx;
     memset(&mIn, 0, sizeof mIn);
     memset(&mCL, 0, sizeof mCL);
@@ -1504,7 +1475,7 @@ static cudaError_t launch_tb16(const StepArgs &a, cudaStream_t s) {
     const int use_tma = make_maps16<ST, TBY>(a, &mIn, &mCL, &mEx) ? 1 : 0;
     const int ntx = (a.g.nx + TBX - 1) / TBX, nty = (a.g.ny + TBY - 1) / TBY;
     const int ntiles = ntx * nty;
-    const int blocks = ntiles < per_sm * nsm ? ntiles : per_sm * nsm;
+    const int blocks = ntiles < fit.per_sm * fit.nsm ? ntiles : fit.per_sm * fit.nsm;
     step2d_tb2h<ST, TBY, NT, MINB><<<blocks, NT, Gm::BYTES, s>>>(a, mIn, mCL, mEx, use_tma, ntx, nty, blocks / ntx,
                                                                  blocks % ntx);
     return cudaGetLastError();

@@ -228,21 +228,15 @@ size_t edge_smem_bytes(int k, const std::vector<EdgeTile> &tiles, bool mu) {
 cudaError_t launch_edge_2d(const StepArgs &a, const Walls &w, const EdgeTile *d_tiles, int ntiles, size_t smem, int k,
                            bool aniso, cudaStream_t s) {
     if (ntiles == 0) return cudaSuccess;
-    static bool attr[3] = {false, false, false};
     const bool mu = a.med.dlnmu != nullptr;
     if (aniso && mu) return cudaErrorInvalidValue;  // an anisotropic medium has a uniform permeability
     const int v = aniso ? 2 : mu ? 1 : 0;
-    if (!attr[v]) {
-        const int max_bytes = (int)((sizeof(float) * edge_floats_per_site(true) + 3 * sizeof(int)) * EDGE_MAX_WINDOW);
-        cudaError_t e = v == 2   ? cudaFuncSetAttribute(edge2d<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        max_bytes)
-                        : v == 1 ? cudaFuncSetAttribute(edge2d<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        max_bytes)
-                                 : cudaFuncSetAttribute(edge2d<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        max_bytes);
-        if (e != cudaSuccess) return e;
-        attr[v] = true;
-    }
+    const size_t max_bytes = (sizeof(float) * edge_floats_per_site(true) + 3 * sizeof(int)) * EDGE_MAX_WINDOW;
+    static PerDevice<KernelFit> fits[3];
+    KernelFit fit;
+    const cudaError_t e = kernel_fit(fits[v], v == 2 ? edge2d<false, true> : v == 1 ? edge2d<true> : edge2d<false>,
+                                     EDGE_THREADS, max_bytes, &fit);
+    if (e != cudaSuccess) return e;
     if (v == 2) edge2d<false, true><<<ntiles, EDGE_THREADS, smem, s>>>(a, w, d_tiles, k);
     else if (v == 1) edge2d<true><<<ntiles, EDGE_THREADS, smem, s>>>(a, w, d_tiles, k);
     else edge2d<false><<<ntiles, EDGE_THREADS, smem, s>>>(a, w, d_tiles, k);
