@@ -412,7 +412,9 @@ lbem_status lbem_adjoint(lbem_t *h, const float *trace_cot, float *grad_eps, dou
  * launch apply and are enabled (lbem_set_temporal_blocking), every tile shape
  * of that kernel is timed too; the fastest is kept, and two-step launches stay
  * on only if they beat the best single-step kernel.  The marching kernel (2D and 3D) is timed beside them where
- * it applies; if it wins, the default without a tile shape is kept. */
+ * it applies (over trial_steps rounded up to a multiple of 24: whole launches); if it wins, the default without a tile
+ * shape is kept.  Where no launch of several steps applies to the medium at hand, steps_per_pass and the tile shape stay
+ * as they are. */
 lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best);
 lbem_status lbem_set_variant(lbem_t *h, int variant);
 lbem_status lbem_get_variant(const lbem_t *h, int *variant, int *nvariants);

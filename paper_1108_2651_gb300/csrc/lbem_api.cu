@@ -1171,11 +1171,13 @@ lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best) {
     // per step, single steps included
     float best_per_step = best_ms / trial_steps;
     int best_shape = h->tb_shape, best_tblock = 1;
+    bool multi = false;  // whether launches of several steps were timed: what was not keeps its setting
     const int max_k = h->tblock;
     for (int k = 2; k <= max_k && st == LBEM_OK; k++) {
         if (!multi_step_base(h) || (k == 3 && (h->storage != LBEM_F32 || h->has_mu))) continue;
         const int nl = trial_steps / k > 0 ? trial_steps / k : 1;
         const int nsh = k == 3 ? tb3_nshapes() : two_step_nshapes(h);
+        multi = true;
         for (int shape = 0; shape < nsh && st == LBEM_OK; shape++) {
             int cur = cur0;
             for (int rep = 0; rep < 2 && st == LBEM_OK; rep++) {
@@ -1203,15 +1205,17 @@ lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best) {
             }
         }
     }
-    // the marching kernel, where calls of this handle would run by it if no shape were kept
+    // the marching kernel, where calls of this handle would run by it if no shape were kept, over whole launches: 24 is
+    // a multiple of the steps of each (8, 6, 4 and, in 3D, 3), and a launch of fewer steps takes as long as a full one
     bool march = false;
-    if (st == LBEM_OK && max_k == 2 && trial_steps >= MARCH_MIN_STEPS) {
+    if (st == LBEM_OK && max_k == 2) {
         const bool set = h->tb_shape_set;
         h->tb_shape_set = false;
         const bool d3 = march3_ok(h);
         if (d3 || march_ok(h)) {
             int n = 0;
-            const int steps = d3 ? trial_steps / MARCH3_STEPS * MARCH3_STEPS : trial_steps;
+            const int steps = (trial_steps + 23) / 24 * 24;
+            multi = true;
             for (int rep = 0; rep < 2 && st == LBEM_OK; rep++) {
                 StepArgs a = step_args(h, cur0);
                 a.evt.rowptr = nullptr;
@@ -1237,9 +1241,11 @@ lbem_status lbem_autotune(lbem_t *h, int trial_steps, int *best) {
     cudaFree(save);
     if (st != LBEM_OK) return st;
     h->variant = best_v;
-    h->tb_shape = march ? 0 : best_shape;
-    h->tb_shape_set = !march;
-    h->tblock = march ? 2 : best_tblock;
+    if (multi) {
+        h->tb_shape = march ? 0 : best_shape;
+        h->tb_shape_set = !march;
+        h->tblock = march ? 2 : best_tblock;
+    }
     drop_graph(h);
     if (best) *best = best_v;
     return LBEM_OK;
