@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "lbem_internal.cuh"
+#include "march_units.cuh"
 
 namespace lbk {
 
@@ -208,8 +209,35 @@ static int two_step_shape(const lbem_t *h) {
 // two steps per launch are the default and no shape was chosen (but for a pole in an anisotropic medium).  Two steps
 // take one two-step launch as before.
 constexpr int MARCH_MIN_STEPS = 3;
+// Whether marching takes less time than launches of two steps with the handle's events.  A warp goes through the events
+// of a unit that holds more than its records (march_event_cost) one by one, 0.15 us each (a source 0.35), for all the rows
+// it marches; the tile and strip kernels go through a row's, 0.3 us each, many rows at a time, and lose 4 us a step
+// without events on 256^2, 6 on 1024^2, 44 on 4096^2.  Events that crowd rows of one unit therefore keep the launches of
+// two steps (us a step, those and marching: a block of 32^2 receivers on 1024^2 17 and 102, of 128^2 on 2048^2 83 and
+// 1057, one site in four on 256^2 32 and 107, a line of 1024 sources on 1024^2 with mu 297 and 365); few, scattered or a
+// line of receivers march (64 on a ring on 1024^2 10.6 and 3.7, 16384 at random on 2048^2 87 and 15, a line of 2048 there
+// 820 and 327).
+static bool march_events_ok(const lbem_t *h) {
+    if (h->nsrc < 2 && h->nev <= MARCH_RECORDS) return true;
+    if (h->march_events < 0) {
+        MarchUnits u;
+        if (launch_march_2d(step_args(h, h->cur), handle_walls(h), h->storage, h->aniso, 0, h->stream, nullptr, &u) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        std::vector<MarchEvent> ev;
+        ev.reserve(h->nev);
+        const int nx = h->grid.nx;
+        for (long long s : h->src_site) ev.push_back({(int)(s / nx), (int)(s % nx), true});
+        for (long long s : h->rec_site) ev.push_back({(int)(s / nx), (int)(s % nx), false});
+        const MarchEventCost c = march_event_cost(u, nx, h->grid.ny, event_bucket(nx), ev);
+        h->march_events = c.visits <= 2. * c.row + 24. + (double)h->nsite / 65536.;
+    }
+    return h->march_events != 0;
+}
 static bool march_ok(const lbem_t *h) {
-    return h->tblock == 2 && !h->tb_shape_set && multi_step_base(h) && !(h->disp && h->aniso);
+    return h->tblock == 2 && !h->tb_shape_set && multi_step_base(h) && !(h->disp && h->aniso) && march_events_ok(h);
 }
 // 3D: triples of steps by the marching kernel (march3d.cu) where several steps per launch are the default, with uniform
 // mu; offsets in a plane must fit 32 bits.
@@ -264,7 +292,7 @@ static cudaError_t enqueue_steps(const lbem_t *h, int cur, long long t0, int nst
             cur ^= 1;
         }
     }
-    if (march_ok(h) && nsteps >= MARCH_MIN_STEPS) {
+    if (nsteps >= MARCH_MIN_STEPS && march_ok(h)) {
         StepArgs a = step_args(h, cur);
         a.t = t0;
         int launches = 0;
@@ -356,6 +384,7 @@ static lbem_status rebuild_events(lbem_t *h) {
     gfree(h, h->d_ev);
     h->d_ev = nullptr;
     h->nev = (int)sorted.size();
+    h->march_events = -1;
     // the row pointers and, from the next multiple of 8 bytes, the rows' column masks: one array, one copy
     const size_t nrp = (size_t)(h->grid.nrows + 2) / 2 * 2;
     if (h->dim == 2) rowptr.resize(nrp + 2 * (size_t)h->grid.nrows, 0);
@@ -600,6 +629,7 @@ static lbem_status set_medium(lbem_t *h, const float *eps_r, const float *mu_r, 
     h->aniso_r = (float)r;
     h->aniso_mu = (float)mubar;
     h->has_medium = true;
+    h->march_events = -1;
     drop_graph(h);
     return LBEM_OK;
 }
@@ -840,6 +870,7 @@ lbem_status lbem_set_boundaries(lbem_t *h, const int kind[3], int layer, double 
     for (int a = 0; a < 3; a++) h->bc[a] = kind[a];
     h->layer = any ? layer : 0;
     h->gamma_max = any ? gamma_max : 0.0;
+    h->march_events = -1;
     drop_graph(h);
     if (h->has_mu) LBEM_CUDA(launch_medium_grad_walls(h, h->stream));  // grad ln mu at the walls
     if (!any) return LBEM_OK;
@@ -885,6 +916,7 @@ lbem_status lbem_set_dispersion(lbem_t *h, const float *wp2, const float *wr2, c
             *p = nullptr;
         }
         h->disp = false;
+        h->march_events = -1;
         drop_graph(h);
         return LBEM_OK;
     }
@@ -920,6 +952,7 @@ lbem_status lbem_set_dispersion(lbem_t *h, const float *wp2, const float *wr2, c
     for (float *p : {h->d_J, h->d_J2, h->d_P, h->d_P2}) LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * pl, h->stream));
     LBEM_CUDA(cudaStreamSynchronize(h->stream));
     h->disp = true;
+    h->march_events = -1;
     drop_graph(h);
     return LBEM_OK;
 }

@@ -532,6 +532,9 @@ struct lbem {
     std::vector<float> src_amp;
     std::vector<long long> rec_site;
     std::vector<int> rec_comp;
+    // whether the 2D marching kernel takes these events (lbem_api.cu, march_events_ok): -1 not looked at since the events
+    // or the medium changed
+    mutable int march_events = -1;
     // scratch
     double *d_partials = nullptr;
     int n_partials = 0;
@@ -619,13 +622,14 @@ cudaError_t launch_step_2d_rs2(const StepArgs &a, int shape, cudaStream_t s);
 // march_media.cu, march16.cu): enqueues the launches of nsteps steps from a.in, alternating between the two buffers;
 // *launches of them.  launch_march_2d chooses by the medium: FP32 with an isotropic medium (uniform or heterogeneous mu)
 // or an anisotropic tensor, walls and layers included, or a pole without walls, mu or tensor; 16-bit storage with uniform
-// mu and nx % 4 == 0, without walls.
+// mu and nx % 4 == 0, without walls.  With units, they say what those launches' units are instead (march_units.cuh).
+struct MarchUnits;
 cudaError_t launch_march_2d(const StepArgs &a, const Walls &w, int storage, bool aniso, int nsteps, cudaStream_t s,
-                            int *launches);
-cudaError_t launch_march_2d_an(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches);
-cudaError_t launch_march_2d_mu(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches);
-cudaError_t launch_march_2d_pole(const StepArgs &a, int nsteps, cudaStream_t s, int *launches);
-cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaStream_t s, int *launches);
+                            int *launches, MarchUnits *units = nullptr);
+cudaError_t launch_march_2d_an(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches, MarchUnits *units);
+cudaError_t launch_march_2d_mu(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches, MarchUnits *units);
+cudaError_t launch_march_2d_pole(const StepArgs &a, int nsteps, cudaStream_t s, int *launches, MarchUnits *units);
+cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaStream_t s, int *launches, MarchUnits *units);
 // 3D, MARCH3_STEPS steps per launch, uniform mu, walls and layers included (march3d.cu): nlaunch launches from a.in,
 // alternating between the two buffers
 constexpr int MARCH3_STEPS = 3;

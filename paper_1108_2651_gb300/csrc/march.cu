@@ -16,14 +16,14 @@
 namespace lbk {
 
 cudaError_t launch_march_2d(const StepArgs &a, const Walls &w, int storage, bool aniso, int nsteps, cudaStream_t s,
-                            int *launches) {
+                            int *launches, MarchUnits *units) {
     const bool walls = w.kind[0] || w.kind[1];
-    if (storage != LBEM_F32) return launch_march_2d_16(a, storage, nsteps, s, launches);
-    if (a.med.wp2) return launch_march_2d_pole(a, nsteps, s, launches);
-    if (aniso) return launch_march_2d_an(a, w, nsteps, s, launches);
-    if (a.med.dlnmu) return launch_march_2d_mu(a, w, nsteps, s, launches);
-    if (walls) return launch_march<LBEM_F32, MARCH_ISO, true, 8, 3>(a, w, nsteps, s, launches);
-    return launch_march<LBEM_F32, MARCH_ISO, false, 8, 3>(a, w, nsteps, s, launches);
+    if (storage != LBEM_F32) return launch_march_2d_16(a, storage, nsteps, s, launches, units);
+    if (a.med.wp2) return launch_march_2d_pole(a, nsteps, s, launches, units);
+    if (aniso) return launch_march_2d_an(a, w, nsteps, s, launches, units);
+    if (a.med.dlnmu) return launch_march_2d_mu(a, w, nsteps, s, launches, units);
+    if (walls) return launch_march<LBEM_F32, MARCH_ISO, true, 8, 3>(a, w, nsteps, s, launches, units);
+    return launch_march<LBEM_F32, MARCH_ISO, false, 8, 3>(a, w, nsteps, s, launches, units);
 }
 
 }  // namespace lbk

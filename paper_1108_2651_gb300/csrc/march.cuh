@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "lbem_internal.cuh"
+#include "march_units.cuh"
 
 namespace lbk {
 
@@ -119,14 +120,6 @@ struct MarchArgs {
     // last segments of a strip hold he (hex) rows (0: as the others)
     int nl, nr, nsegx, he, hex;
 };
-
-// The unit's column and row ranges: whole chunks of 4 columns and rows, evenly.
-__host__ __device__ __forceinline__ int march_cut(int k, int n, int of) { return (int)((long long)k * of / n); }
-// The first row of segment k of n, of ny rows, the first and the last segment of he rows (0: as the others).
-__host__ __device__ __forceinline__ int march_row(int k, int n, int ny, int he) {
-    if (he == 0 || k == 0 || k == n) return k == n ? ny : march_cut(k, n, ny);
-    return he + march_cut(k - 1, n - 2, ny - 2 * he);
-}
 
 template <int ST, int MED, int K, int D>
 struct MarchCfg {
@@ -758,7 +751,7 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
             float4 sh = z4, sig;
             bool src = false;
             if (MED == MARCH_MU) sh = mu_src(mr, g1, h2, g3, h4);
-            src = events(yl - j, j, h0, g1, h2, g3, h4, c, Pn, sh);
+            if (j < kp) src = events(yl - j, j, h0, g1, h2, g3, h4, c, Pn, sh);
             m_collide<MED>(h0, g1, h2, g3, h4, c, Pn, sh, r, ri, fs, n, sig);
             if (MED != MARCH_MU && src) source(c, sh, n);
             if (MED == MARCH_POLE) pole(mr, c, sig, Jn, Pn);
@@ -898,9 +891,10 @@ __global__ void __launch_bounds__(32, 8) march2d(const __grid_constant__ MarchAr
 // Launches of K steps, the last one of what is left.  One wave of units: as many segments as fill the GPU (a second
 // wave would leave it half empty), of at least two rows.  Each launch may start while the one before drains
 // (programmatic dependent launch; it waits for its input with griddepcontrol.wait): 128^2 8.2 us a launch against
-// 10.3 us, 1024^2 18 us against 20.5 us.
+// 10.3 us, 1024^2 18 us against 20.5 us.  With units, only says what they are.
 template <int ST, int MED, bool WL, int K, int D>
-static cudaError_t launch_march(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches) {
+static cudaError_t launch_march(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches,
+                                MarchUnits *units) {
     using Cfg = MarchCfg<ST, MED, K, D>;
     auto *k = march2d<ST, MED, WL, K, D>;
     static PerDevice<KernelFit> fits;
@@ -926,6 +920,17 @@ static cudaError_t launch_march(const StepArgs &a, const Walls &w, int nsteps, c
     if (WL && w.kind[1] && m.nseg >= 4) {
         const int reach = std::max(w.nlayer, 1) + K, he = std::max(reach, a.g.ny / m.nseg / 3 - (K - 1));
         if (2 * he + (m.nseg - 2) * 2 <= a.g.ny) m.he = he;
+    }
+    if (units) {
+        units->K = K;
+        units->H = Cfg::H;
+        units->nstrips = m.nstrips;
+        units->nseg = m.nseg;
+        units->nl = m.nl;
+        units->nr = m.nr;
+        units->nsegx = m.nsegx;
+        units->he = m.he;
+        return cudaSuccess;
     }
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -10,11 +10,11 @@
 
 namespace lbk {
 
-cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaStream_t s, int *launches) {
+cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaStream_t s, int *launches, MarchUnits *units) {
     const Walls w;
-    if (storage == LBEM_F16) return launch_march<LBEM_F16, MARCH_ISO, false, 8, 3>(a, w, nsteps, s, launches);
-    if (storage == LBEM_BF16) return launch_march<LBEM_BF16, MARCH_ISO, false, 8, 3>(a, w, nsteps, s, launches);
-    return launch_march<LBEM_I16B, MARCH_ISO, false, 4, 4>(a, w, nsteps, s, launches);
+    if (storage == LBEM_F16) return launch_march<LBEM_F16, MARCH_ISO, false, 8, 3>(a, w, nsteps, s, launches, units);
+    if (storage == LBEM_BF16) return launch_march<LBEM_BF16, MARCH_ISO, false, 8, 3>(a, w, nsteps, s, launches, units);
+    return launch_march<LBEM_I16B, MARCH_ISO, false, 4, 4>(a, w, nsteps, s, launches, units);
 }
 
 }  // namespace lbk

@@ -9,18 +9,18 @@
 
 namespace lbk {
 
-cudaError_t launch_march_2d_an(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches) {
-    if (w.kind[0] || w.kind[1]) return launch_march<LBEM_F32, MARCH_AN, true, 8, 3>(a, w, nsteps, s, launches);
-    return launch_march<LBEM_F32, MARCH_AN, false, 8, 3>(a, w, nsteps, s, launches);
+cudaError_t launch_march_2d_an(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches, MarchUnits *units) {
+    if (w.kind[0] || w.kind[1]) return launch_march<LBEM_F32, MARCH_AN, true, 8, 3>(a, w, nsteps, s, launches, units);
+    return launch_march<LBEM_F32, MARCH_AN, false, 8, 3>(a, w, nsteps, s, launches, units);
 }
 
-cudaError_t launch_march_2d_mu(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches) {
-    if (w.kind[0] || w.kind[1]) return launch_march<LBEM_F32, MARCH_MU, true, 6, 3>(a, w, nsteps, s, launches);
-    return launch_march<LBEM_F32, MARCH_MU, false, 6, 3>(a, w, nsteps, s, launches);
+cudaError_t launch_march_2d_mu(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches, MarchUnits *units) {
+    if (w.kind[0] || w.kind[1]) return launch_march<LBEM_F32, MARCH_MU, true, 6, 3>(a, w, nsteps, s, launches, units);
+    return launch_march<LBEM_F32, MARCH_MU, false, 6, 3>(a, w, nsteps, s, launches, units);
 }
 
-cudaError_t launch_march_2d_pole(const StepArgs &a, int nsteps, cudaStream_t s, int *launches) {
-    return launch_march<LBEM_F32, MARCH_POLE, false, 6, 3>(a, Walls(), nsteps, s, launches);
+cudaError_t launch_march_2d_pole(const StepArgs &a, int nsteps, cudaStream_t s, int *launches, MarchUnits *units) {
+    return launch_march<LBEM_F32, MARCH_POLE, false, 6, 3>(a, Walls(), nsteps, s, launches, units);
 }
 
 }  // namespace lbk
