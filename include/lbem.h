@@ -168,7 +168,7 @@ lbem_status lbem_set_receivers(lbem_t *h, int n, const long long *site, const in
  * 9-10), source (Eq. 3), equilibrium (Eq. 8), collision at tau = dt/2 (Eq. 17);
  * receivers sample the pre-collision fields.  One fused kernel launch per step,
  * or per two (three) steps where lbem_set_temporal_blocking enables it (two is
- * the default for 2D), or, for a call of at least 3 steps of a 2D grid that keeps
+ * the default for 2D), or, for a call of more than a few steps of a 2D grid that keeps
  * that default with no tile shape chosen, per 4 to 8 steps (see there), enqueued on the
  * stream (or replayed from a cached CUDA graph when enabled by lbem_set_graphs).
  * Requires a medium.  nsteps >= 0. */
@@ -258,9 +258,10 @@ lbem_status lbem_set_watchdog(lbem_t *h, int every, double max_growth);
  * sites), walls and layers included; a dispersive pole without walls or a mu array with shape 0 at 4 per SM;
  * both bit-identical to their single steps.  With a pole and walls (or a pole with a mu array), and for
  * steps_per_pass = 3, every step of these media is a single step.
- * With steps_per_pass = 2 and tile_shape = -1 (the default), a call of lbem_step of at least 3 steps runs several steps
+ * With steps_per_pass = 2 and tile_shape = -1 (the default), a call of lbem_step runs several steps
  * per launch by the marching kernel instead, wherever launches of two steps apply but for a pole in an anisotropic
- * medium: a warp walks a strip of columns down its rows with 8 time levels in flight (6 with a heterogeneous mu or a
+ * medium, if it has at least 3 steps (5 with LBEM_F16, LBEM_BF16 or walls; up to 7 on some grids) and its sources and
+ * receivers do not crowd a few rows and columns (shorter and crowded runs are faster by two): a warp walks a strip of columns down its rows with 8 time levels in flight (6 with a heterogeneous mu or a
  * pole, 4 with LBEM_I16B; the last launch of a call takes the steps left; walls and layers are applied on the way, with
  * no pass after it).  The results are the same bits again: those of single steps for FP32 storage, of launches of two
  * steps for 16-bit storage, whose state is rounded after every second step.  A tile shape >= 0 gives launches of two

@@ -205,10 +205,20 @@ static int two_step_shape(const lbem_t *h) {
     if (!h->tb_shape_set && big) return h->has_mu ? 2 : 7 + rs2_nshapes() + 1;
     return h->tblock == 2 && h->tb_shape < tb2_nshapes(h->storage, h->has_mu) ? h->tb_shape : 0;
 }
-// Whether calls of at least MARCH_MIN_STEPS steps run by the marching kernel (march.cu), up to 8 steps a launch: where
-// two steps per launch are the default and no shape was chosen (but for a pole in an anisotropic medium).  Two steps
-// take one two-step launch as before.
-constexpr int MARCH_MIN_STEPS = 3;
+// The fewest steps of a call that marching takes less time for than launches of two steps.  A launch of fewer steps than
+// the kernel's K computes all K levels, so a short call's launch takes almost the time of a full one.  Measured on 21 grids
+// from 64^2 to 4096^2 and 1 to 65536 rows (us a call, two-step launches and marching): three steps FP32 4096^2 230 and
+// 176, 1024^2 20.5 and 18.7, mu 24.6 and 18.5, a pole 32 and 24, block-int16 22.7 and 18.2, but on fewer than 8 rows and
+// very many columns, where a unit marches 2 rows and 2 (K - 1) more, 4 x 524288 41.0 and 45.6; with walls 1024^2 three
+// 41 and 47, four 45 and 50, five 64 and 57; with walls and a tensor three 33 and 51, five 58 and 62, six 74 and 67
+// (1025 x 2047: five 92 and 68); FP16, whose launches of two steps move half the bytes, 1024^2 three 18.6 and 21.1, 4096^2
+// four 181 and 203, five 249 and 205; BF16 likewise.
+static int march_min_steps(const lbem_t *h) {
+    const bool few_rows = h->grid.ny < 8 && h->grid.nx >= 1 << 18;
+    if (h->storage == LBEM_F16 || h->storage == LBEM_BF16) return few_rows ? 7 : 5;
+    if (h->walls() && !h->has_mu) return !h->aniso || h->nsite >= 1 << 21 ? 5 : 6;
+    return few_rows ? 4 : 3;
+}
 // Whether marching takes less time than launches of two steps with the handle's events.  A warp goes through the events
 // of a unit that holds more than its records (march_event_cost) one by one, 0.15 us each (a source 0.35), for all the rows
 // it marches; the tile and strip kernels go through a row's, 0.3 us each, many rows at a time, and lose 4 us a step
@@ -236,6 +246,9 @@ static bool march_events_ok(const lbem_t *h) {
     }
     return h->march_events != 0;
 }
+// Whether calls of at least march_min_steps steps run by the marching kernel (march.cu), up to 8 steps a launch: where two
+// steps per launch are the default and no shape was chosen (but for a pole in an anisotropic medium).  Shorter calls take
+// launches of two steps.
 static bool march_ok(const lbem_t *h) {
     return h->tblock == 2 && !h->tb_shape_set && multi_step_base(h) && !(h->disp && h->aniso) && march_events_ok(h);
 }
@@ -292,7 +305,7 @@ static cudaError_t enqueue_steps(const lbem_t *h, int cur, long long t0, int nst
             cur ^= 1;
         }
     }
-    if (nsteps >= MARCH_MIN_STEPS && march_ok(h)) {
+    if (nsteps >= march_min_steps(h) && march_ok(h)) {
         StepArgs a = step_args(h, cur);
         a.t = t0;
         int launches = 0;
