@@ -340,16 +340,14 @@ static cudaError_t enqueue_steps(const lbem_t *h, int cur, long long t0, int nst
             cur ^= 1;
         }
     }
-    if (march3_ok(h)) {
+    if (nsteps - n >= MARCH3_STEPS && march3_ok(h)) {
         const int K = MARCH3_STEPS, launches = (nsteps - n) / K;
-        if (launches > 0) {
-            StepArgs a = step_args(h, cur);
-            a.t = t0 + n;
-            cudaError_t e = launch_march_3d(a, handle_walls(h), launches, h->stream);
-            if (e != cudaSuccess) return e;
-            n += K * launches;
-            cur ^= launches & 1;
-        }
+        StepArgs a = step_args(h, cur);
+        a.t = t0 + n;
+        cudaError_t e = launch_march_3d(a, handle_walls(h), launches, h->stream);
+        if (e != cudaSuccess) return e;
+        n += K * launches;
+        cur ^= launches & 1;
     }
     for (; n < nsteps; n++) {
         StepArgs a = step_args(h, cur);

@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "march3_units.cuh"
 #include "site3d.cuh"
 
 namespace lbk {
@@ -36,8 +37,6 @@ struct March3Args {
     Adj3 adj;
     int ntx, nty, nseg;
 };
-
-constexpr int M3_PLANES = 512;  // the most planes a block marches
 
 __host__ __device__ __forceinline__ int cut3(int k, int n, int of) { return (int)((long long)k * of / n); }
 
@@ -362,25 +361,6 @@ __global__ void __launch_bounds__(32 * NW, 1) march3d(const __grid_constant__ Ma
     }
 }
 
-// The tiles, and the segments of planes for which the waves of blocks times the planes a block marches (its K - 1 at either
-// end included) are the fewest; returns those planes.
-template <int K, int TY>
-static long long plan3(const Grid &g, int wave, int *ntx, int *nty, int *nseg) {
-    constexpr int WX = 32 - 2 * (K - 1), WY = TY - 2 * (K - 1);
-    *ntx = (g.nx + WX - 1) / WX;
-    *nty = (g.ny + WY - 1) / WY;
-    const long long tiles = (long long)*ntx * *nty;
-    long long best = -1;
-    for (int n = (g.nz - 1) / (M3_PLANES - 2 * K) + 1; n <= g.nz; n++) {
-        const long long cost = (tiles * n + wave - 1) / wave * ((g.nz + n - 1) / n + 2 * (K - 1));
-        if (best < 0 || cost < best) {
-            best = cost;
-            *nseg = n;
-        }
-    }
-    return best;
-}
-
 // Each launch may start while the one before drains (it waits for its input with griddepcontrol.wait).
 template <int K, int NW, int NR, bool WL, int MODE>
 static cudaError_t launch_march3(const StepArgs &a, const Walls &w, const Adj3 &adj, int nlaunch, cudaStream_t s) {
@@ -394,7 +374,10 @@ static cudaError_t launch_march3(const StepArgs &a, const Walls &w, const Adj3 &
     m.a = a;
     m.w = w;
     m.adj = adj;
-    plan3<K, TY>(a.g, fit.per_sm * fit.nsm, &m.ntx, &m.nty, &m.nseg);
+    const March3Plan p = march3_plan(a.g.nx, a.g.ny, a.g.nz, K, TY, fit.per_sm * fit.nsm);
+    m.ntx = p.ntx;
+    m.nty = p.nty;
+    m.nseg = p.nseg;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -438,11 +421,11 @@ cudaError_t launch_march_3d_adj(const StepArgs &a, const Adj3 &adj, bool record,
 // A grid a little wider than a tile, say 30 x 24 x 96, pays for two tiles.
 bool march_3d_pays(const Grid &g, bool more) {
     constexpr int K = MARCH3_STEPS;
-    int nsm = 0, dev = 0, ntx, nty, nseg;
+    int nsm = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
         return false;
-    const double planes = (double)plan3<K, M3_WARPS * M3_COLS>(g, nsm, &ntx, &nty, &nseg);
+    const double planes = (double)march3_plan(g.nx, g.ny, g.nz, K, M3_WARPS * M3_COLS, nsm).planes;
     const double sites = (double)g.nx * g.ny * g.nz;
     return planes * (more ? 3.4 : 2.5) <= K * (3.5 + sites * (more ? 28.7e-6 : 25.4e-6));
 }
