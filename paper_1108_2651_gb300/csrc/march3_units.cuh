@@ -40,4 +40,15 @@ inline March3Plan march3_plan(int nx, int ny, int nz, int K, int TY, int wave) {
     return p;
 }
 
+// The time of a launch of the marching kernel and of a single step, measured on 22 grids from 32^3 to 192^3 and from 3 to
+// 131072 planes, rows or columns (more: with walls, with sigma written, and for the adjoint).  Marching takes 2.2 to 2.6 us
+// a plane of a wave of blocks (walls 3.0 to 3.4), a single step 27 ns a thousand elements of a plane, its rows' padding
+// included (a warp takes 32 of a row whatever it holds), but no launch less than 4.1 us: 3 x 250 x 460 34.0 us a launch
+// against three steps of 8.7 (walls 45.9, 11.1), 30 x 24 x 96 14.1 against 4.1, 48^3 14.5 against 6.1, 64^3 23.7 against 8.2
+// (walls 32.5, 10.1), 80^3 30.0 against 16.4 (walls 40.3, 18.4), 192^3 318 against 180 (walls 398, 187).
+inline double march3_us(const March3Plan &p, bool more) { return (double)p.planes * (more ? 3.35 : 2.4); }
+inline double single3_us(double plane, bool more) {
+    return std::max(4.1, (more ? 2. : 1.2) + plane * (more ? 27.5e-6 : 27e-6));
+}
+
 }  // namespace lbk

@@ -414,20 +414,15 @@ cudaError_t launch_march_3d_adj(const StepArgs &a, const Adj3 &adj, bool record,
                   : launch_march3<K, M3_WARPS, M3_COLS, false, M3_ADJOINT>(a, Walls(), adj, nlaunch, s);
 }
 
-// Whether K steps of the marching kernel take less time than K single ones.  Marching takes 2.5 us a plane of a wave of
-// blocks (3.4 with more to do: walls, sigma, the adjoint), a single step 3.5 us and 25.4 ns (28.7) per thousand sites,
-// measured on cubes of 24 to 192: 64^3 8.2 us a step either way, 48^3 5.1 against 6.2 us; with walls 64^3 11.4 against
-// 10.3 us, 80^3 14.3 against 20.5 us; 40 steps recorded and gone back 64^3 1.20 against 1.07 ms, 80^3 1.49 against 1.84 ms.
-// A grid a little wider than a tile, say 30 x 24 x 96, pays for two tiles.
+// Whether K steps of the marching kernel take less time than K single ones (march3_units.cuh has the estimate).
 bool march_3d_pays(const Grid &g, bool more) {
     constexpr int K = MARCH3_STEPS;
     int nsm = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
         return false;
-    const double planes = (double)march3_plan(g.nx, g.ny, g.nz, K, M3_WARPS * M3_COLS, nsm).planes;
-    const double sites = (double)g.nx * g.ny * g.nz;
-    return planes * (more ? 3.4 : 2.5) <= K * (3.5 + sites * (more ? 28.7e-6 : 25.4e-6));
+    const March3Plan p = march3_plan(g.nx, g.ny, g.nz, K, M3_WARPS * M3_COLS, nsm);
+    return march3_us(p, more) <= K * single3_us((double)g.plane, more);
 }
 
 }  // namespace lbk
