@@ -255,8 +255,12 @@ static bool march_ok(const lbem_t *h) {
 // 3D: triples of steps by the marching kernel (march3d.cu) where several steps per launch are the default, with uniform
 // mu; offsets in a plane must fit 32 bits.
 bool march3_ok(const lbem_t *h, bool adjoint) {
-    return h->tblock == 2 && h->dim == 3 && !h->has_mu && h->grid.plane < (1LL << 31) &&
-           march_3d_pays(h->grid, adjoint || h->bc[0] || h->bc[1] || h->bc[2]);
+    if (h->tblock != 2 || h->dim != 3 || h->has_mu || h->grid.plane >= (1LL << 31)) return false;
+    if (!h->march3_rows.empty()) {
+        h->march3_events = march_3d_events(h->grid, h->march3_rows);
+        h->march3_rows.clear();
+    }
+    return march_3d_pays(h->grid, adjoint || h->bc[0] || h->bc[1] || h->bc[2], h->march3_events);
 }
 static int steps_per_launch(const lbem_t *h) { return three_step_ok(h) ? 3 : two_step_ok(h) ? 2 : 1; }
 
@@ -396,6 +400,8 @@ static lbem_status rebuild_events(lbem_t *h) {
     h->d_ev = nullptr;
     h->nev = (int)sorted.size();
     h->march_events = -1;
+    h->march3_events = March3Events();
+    h->march3_rows = h->dim == 3 && h->nev ? rowptr : std::vector<int>();
     // the row pointers and, from the next multiple of 8 bytes, the rows' column masks: one array, one copy
     const size_t nrp = (size_t)(h->grid.nrows + 2) / 2 * 2;
     if (h->dim == 2) rowptr.resize(nrp + 2 * (size_t)h->grid.nrows, 0);

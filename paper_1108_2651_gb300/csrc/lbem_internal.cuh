@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "../../include/lbem.h"
+#include "march3_units.cuh"
 #include "per_device.cuh"
 
 namespace lbk {
@@ -535,6 +536,9 @@ struct lbem {
     // whether the 2D marching kernel takes these events (lbem_api.cu, march_events_ok): -1 not looked at since the events
     // or the medium changed
     mutable int march_events = -1;
+    // 3D: what they add to a marching launch and to a single step, from the events before each row (lbem_api.cu, march3_ok)
+    mutable lbk::March3Events march3_events;
+    mutable std::vector<int> march3_rows;  // empty: looked at, or no events
     // scratch
     double *d_partials = nullptr;
     int n_partials = 0;
@@ -634,7 +638,8 @@ cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaS
 // alternating between the two buffers
 constexpr int MARCH3_STEPS = 3;
 // whether it takes less time than single steps on this grid (more: with walls, with sigma written, and for the adjoint)
-bool march_3d_pays(const Grid &g, bool more);
+bool march_3d_pays(const Grid &g, bool more, const March3Events &ev);
+March3Events march_3d_events(const Grid &g, const std::vector<int> &rowptr);
 cudaError_t launch_march_3d(const StepArgs &a, const Walls &w, int nlaunch, cudaStream_t s);
 bool march3_ok(const lbem_t *h, bool adjoint = false);  // whether (adjoint) steps of this handle go to it
 // what the 3D adjoint records and accumulates (adjoint.cu)

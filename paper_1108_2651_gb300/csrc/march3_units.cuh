@@ -1,6 +1,7 @@
 // The 3D marching kernel's blocks (march3d.cu): host code, plain C++.
 #pragma once
 #include <algorithm>
+#include <vector>
 
 namespace lbk {
 
@@ -46,9 +47,86 @@ inline March3Plan march3_plan(int nx, int ny, int nz, int K, int TY, int wave) {
 // included (a warp takes 32 of a row whatever it holds), but no launch less than 4.1 us: 3 x 250 x 460 34.0 us a launch
 // against three steps of 8.7 (walls 45.9, 11.1), 30 x 24 x 96 14.1 against 4.1, 48^3 14.5 against 6.1, 64^3 23.7 against 8.2
 // (walls 32.5, 10.1), 80^3 30.0 against 16.4 (walls 40.3, 18.4), 192^3 318 against 180 (walls 398, 187).
-inline double march3_us(const March3Plan &p, bool more) { return (double)p.planes * (more ? 3.35 : 2.4); }
+inline double march3_us(const March3Plan &p, int nx, bool more) {
+    const double plane = more ? 3.35 : 2.4;
+    return (double)p.planes * (nx < 8 ? 1.65 * plane : plane);  // (460 x 250 x 3: 4.0 us a plane, walls 4.6)
+}
 inline double single3_us(double plane, bool more) {
     return std::max(4.1, (more ? 2. : 1.2) + plane * (more ? 27.5e-6 : 27e-6));
+}
+
+// What a handle's events (rowptr: those of row z ny + y before it) add to a launch of the marching kernel and to a single
+// step, in us.  A warp of a block goes through every event of each of its two rows that has one in the tile's columns, at
+// each of the K levels of a plane, while the block waits: 0.4 us a row and 0.09 us an event (64^3 with 16384 receivers at
+// random 29.0 us a step against 8.2 without, 10.3 by single steps; with 1024 11.6 and 8.3; 3 x 250 x 460 with 16384 69.9
+// and 16.5; 192^3 with 16384 139 and 184).  A single step has a warp a row: 0.15 us an event of the fullest row.
+struct March3Events {
+    double launch = 0., step = 0.;
+};
+inline March3Events march3_events_us(const March3Plan &p, int nx, int ny, int nz, int K, const std::vector<int> &rowptr) {
+    March3Events us;
+    struct Tile {      // of one plane
+        double hits = 0.;  // rows that have an event in one tile's columns, if a row's events lie evenly
+        int rows = 0, events = 0;
+    };
+    std::vector<Tile> row(p.nty);
+    std::vector<double> sum((size_t)p.nty * (nz + 1), 0.);  // [row of tiles][planes before]
+    int fullest = 0;
+    auto start = [&](int t) { return (int)((long long)t * ny / p.nty); };
+    for (int z = 0; z < nz; z++) {
+        const int *r = rowptr.data() + (long long)z * ny;
+        if (r[ny] == r[0]) {
+            for (int t = 0; t < p.nty; t++) sum[(size_t)t * (nz + 1) + z + 1] = sum[(size_t)t * (nz + 1) + z];
+            continue;
+        }
+        row.assign(p.nty, Tile());
+        int t = 0, y0 = 0, y1 = start(1);  // the tile of y and its rows
+        for (int y = 0; y < ny; y++) {
+            if (y >= y1) {
+                t++;
+                y0 = y1;
+                y1 = start(t + 1);
+            }
+            const int n = r[y + 1] - r[y];
+            if (n == 0) continue;
+            fullest = std::max(fullest, n);
+            auto add = [&](Tile &a) {
+                a.hits += std::min(1., n * 32. / nx);
+                a.rows++;
+                a.events += n;
+            };
+            add(row[t]);  // and the tiles that march it as one of their K - 1 rows at either side
+            if (p.nty > 1 && y - y0 < K - 1) add(row[t > 0 ? t - 1 : p.nty - 1]);
+            if (p.nty > 1 && y1 - y < K) add(row[t < p.nty - 1 ? t + 1 : 0]);
+        }
+        for (t = 0; t < p.nty; t++) {
+            const Tile &a = row[t];
+            const double most = a.hits < 1. ? a.hits : std::min(2., 1. + (a.hits - 1.) / 8.);  // of a warp's two rows
+            sum[(size_t)t * (nz + 1) + z + 1] =
+                sum[(size_t)t * (nz + 1) + z] + (a.rows ? most * (0.4 + 0.09 * a.events / a.rows) : 0.);
+        }
+    }
+    double worst = 0., all = 0.;  // over the rows of tiles and the segments
+    int len = 0;
+    for (int k = 0; k < p.nseg; k++) {  // a segment's planes and the K - 1 at either end
+        const int z0 = (int)((long long)k * nz / p.nseg), z1 = (int)((long long)(k + 1) * nz / p.nseg);
+        len = std::max(len, z1 - z0);
+        for (int t = 0; t < p.nty; t++) {
+            const double *s = sum.data() + (size_t)t * (nz + 1);
+            auto upto = [&](int z) {  // planes 0 .. z - 1, wrapped
+                const int q = z >= 0 ? z / nz : -((-z + nz - 1) / nz);
+                return q * s[nz] + s[z - q * nz];
+            };
+            const double v = upto(z1 + K - 1) - upto(z0 - (K - 1));
+            worst = std::max(worst, v);
+            all += v;
+        }
+    }
+    // one wave waits for the worst block, the others take the mean
+    const double waves = (double)p.planes / (len + 2 * (K - 1));
+    us.launch = K * (worst + (waves - 1.) * all / ((double)p.nty * p.nseg));
+    us.step = 0.15 * fullest;
+    return us;
 }
 
 }  // namespace lbk

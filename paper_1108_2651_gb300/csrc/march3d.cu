@@ -414,15 +414,28 @@ cudaError_t launch_march_3d_adj(const StepArgs &a, const Adj3 &adj, bool record,
                   : launch_march3<K, M3_WARPS, M3_COLS, false, M3_ADJOINT>(a, Walls(), adj, nlaunch, s);
 }
 
-// Whether K steps of the marching kernel take less time than K single ones (march3_units.cuh has the estimate).
-bool march_3d_pays(const Grid &g, bool more) {
-    constexpr int K = MARCH3_STEPS;
+// The plan on the current device (nseg 0: no device).
+static March3Plan device_plan(const Grid &g) {
+    March3Plan p;
     int nsm = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
-        return false;
-    const March3Plan p = march3_plan(g.nx, g.ny, g.nz, K, M3_WARPS * M3_COLS, nsm);
-    return march3_us(p, more) <= K * single3_us((double)g.plane, more);
+        p.nseg = 0;
+    else
+        p = march3_plan(g.nx, g.ny, g.nz, MARCH3_STEPS, M3_WARPS * M3_COLS, nsm);
+    return p;
+}
+
+// Whether K steps of the marching kernel take less time than K single ones (march3_units.cuh has the estimate).
+bool march_3d_pays(const Grid &g, bool more, const March3Events &ev) {
+    constexpr int K = MARCH3_STEPS;
+    const March3Plan p = device_plan(g);
+    return p.nseg > 0 && march3_us(p, g.nx, more) + ev.launch <= K * (single3_us((double)g.plane, more) + ev.step);
+}
+
+March3Events march_3d_events(const Grid &g, const std::vector<int> &rowptr) {
+    const March3Plan p = device_plan(g);
+    return p.nseg > 0 ? march3_events_us(p, g.nx, g.ny, g.nz, MARCH3_STEPS, rowptr) : March3Events();
 }
 
 }  // namespace lbk
