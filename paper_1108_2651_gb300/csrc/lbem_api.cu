@@ -260,7 +260,7 @@ bool march3_ok(const lbem_t *h, bool adjoint) {
         h->march3_events = march_3d_events(h->grid, h->march3_rows);
         h->march3_rows.clear();
     }
-    return march_3d_pays(h->grid, adjoint || h->bc[0] || h->bc[1] || h->bc[2], h->march3_events);
+    return march_3d_pays(h->grid, adjoint || h->bc[0] || h->bc[1] || h->bc[2], h->use_graphs && !adjoint, h->march3_events);
 }
 static int steps_per_launch(const lbem_t *h) { return three_step_ok(h) ? 3 : two_step_ok(h) ? 2 : 1; }
 

@@ -638,7 +638,7 @@ cudaError_t launch_march_2d_16(const StepArgs &a, int storage, int nsteps, cudaS
 // alternating between the two buffers
 constexpr int MARCH3_STEPS = 3;
 // whether it takes less time than single steps on this grid (more: with walls, with sigma written, and for the adjoint)
-bool march_3d_pays(const Grid &g, bool more, const March3Events &ev);
+bool march_3d_pays(const Grid &g, bool more, bool graphs, const March3Events &ev);
 March3Events march_3d_events(const Grid &g, const std::vector<int> &rowptr);
 cudaError_t launch_march_3d(const StepArgs &a, const Walls &w, int nlaunch, cudaStream_t s);
 bool march3_ok(const lbem_t *h, bool adjoint = false);  // whether (adjoint) steps of this handle go to it

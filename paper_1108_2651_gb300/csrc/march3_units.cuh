@@ -47,6 +47,8 @@ inline March3Plan march3_plan(int nx, int ny, int nz, int K, int TY, int wave) {
 // included (a warp takes 32 of a row whatever it holds), but no launch less than 4.1 us: 3 x 250 x 460 34.0 us a launch
 // against three steps of 8.7 (walls 45.9, 11.1), 30 x 24 x 96 14.1 against 4.1, 48^3 14.5 against 6.1, 64^3 23.7 against 8.2
 // (walls 32.5, 10.1), 80^3 30.0 against 16.4 (walls 40.3, 18.4), 192^3 318 against 180 (walls 398, 187).
+// In a CUDA graph a marching launch takes 2.1 us more than in a stream and a single step 0.7 us less (64^3 8.6 us a step by
+// marching against 7.5, 80^3 10.7 against 15.5).
 inline double march3_us(const March3Plan &p, int nx, bool more) {
     const double plane = more ? 3.35 : 2.4;
     return (double)p.planes * (nx < 8 ? 1.65 * plane : plane);  // (460 x 250 x 3: 4.0 us a plane, walls 4.6)

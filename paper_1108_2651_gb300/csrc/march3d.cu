@@ -427,10 +427,11 @@ static March3Plan device_plan(const Grid &g) {
 }
 
 // Whether K steps of the marching kernel take less time than K single ones (march3_units.cuh has the estimate).
-bool march_3d_pays(const Grid &g, bool more, const March3Events &ev) {
+bool march_3d_pays(const Grid &g, bool more, bool graphs, const March3Events &ev) {
     constexpr int K = MARCH3_STEPS;
     const March3Plan p = device_plan(g);
-    return p.nseg > 0 && march3_us(p, g.nx, more) + ev.launch <= K * (single3_us((double)g.plane, more) + ev.step);
+    return p.nseg > 0 && march3_us(p, g.nx, more) + (graphs ? 2.1 : 0.) + ev.launch <=
+                             K * (single3_us((double)g.plane, more) - (graphs ? 0.7 : 0.) + ev.step);
 }
 
 March3Events march_3d_events(const Grid &g, const std::vector<int> &rowptr) {
