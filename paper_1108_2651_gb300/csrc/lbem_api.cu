@@ -9,7 +9,6 @@
 #include <vector>
 
 #include "lbem_internal.cuh"
-#include "march_units.cuh"
 
 namespace lbk {
 
@@ -236,12 +235,7 @@ static bool march_events_ok(const lbem_t *h) {
             cudaGetLastError();
             return false;
         }
-        std::vector<MarchEvent> ev;
-        ev.reserve(h->nev);
-        const int nx = h->grid.nx;
-        for (long long s : h->src_site) ev.push_back({(int)(s / nx), (int)(s % nx), true});
-        for (long long s : h->rec_site) ev.push_back({(int)(s / nx), (int)(s % nx), false});
-        const MarchEventCost c = march_event_cost(u, nx, h->grid.ny, event_bucket(nx), ev);
+        const MarchEventCost c = march_event_cost(u, h->grid.nx, h->grid.ny, event_bucket(h->grid.nx), h->march_list);
         h->march_events = c.visits <= 2. * c.row + 24. + (double)h->nsite / 65536.;
     }
     return h->march_events != 0;
@@ -400,6 +394,10 @@ static lbem_status rebuild_events(lbem_t *h) {
     h->d_ev = nullptr;
     h->nev = (int)sorted.size();
     h->march_events = -1;
+    h->march_list.clear();
+    if (h->dim == 2) h->march_list.reserve(ev.size());
+    for (size_t i = 0; i < ev.size() && h->dim == 2; i++)
+        h->march_list.push_back({(int)rows[i], ev[i].x, ev[i].kind == 0});
     h->march3_events = March3Events();
     h->march3_rows = h->dim == 3 && h->nev ? rowptr : std::vector<int>();
     // the row pointers and, from the next multiple of 8 bytes, the rows' column masks: one array, one copy

@@ -28,6 +28,7 @@
 
 #include "../../include/lbem.h"
 #include "march3_units.cuh"
+#include "march_units.cuh"
 #include "per_device.cuh"
 
 namespace lbk {
@@ -536,6 +537,7 @@ struct lbem {
     // whether the 2D marching kernel takes these events (lbem_api.cu, march_events_ok): -1 not looked at since the events
     // or the medium changed
     mutable int march_events = -1;
+    mutable std::vector<lbk::MarchEvent> march_list;  // 2D: the events, in any order
     // 3D: what they add to a marching launch and to a single step, from the events before each row (lbem_api.cu, march3_ok)
     mutable lbk::March3Events march3_events;
     mutable std::vector<int> march3_rows;  // empty: looked at, or no events
@@ -627,7 +629,6 @@ cudaError_t launch_step_2d_rs2(const StepArgs &a, int shape, cudaStream_t s);
 // *launches of them.  launch_march_2d chooses by the medium: FP32 with an isotropic medium (uniform or heterogeneous mu)
 // or an anisotropic tensor, walls and layers included, or a pole without walls, mu or tensor; 16-bit storage with uniform
 // mu and nx % 4 == 0, without walls.  With units, they say what those launches' units are instead (march_units.cuh).
-struct MarchUnits;
 cudaError_t launch_march_2d(const StepArgs &a, const Walls &w, int storage, bool aniso, int nsteps, cudaStream_t s,
                             int *launches, MarchUnits *units = nullptr);
 cudaError_t launch_march_2d_an(const StepArgs &a, const Walls &w, int nsteps, cudaStream_t s, int *launches, MarchUnits *units);

@@ -30,12 +30,6 @@ struct MarchUnits {
     bool walled(int strip) const { return strip < nl || strip >= nstrips - nr; }
     int segs(int strip) const { return walled(strip) ? nsegx : nseg; }
     int row0(int strip, int k, int ny) const { return march_row(k, segs(strip), ny, walled(strip) ? 0 : he); }
-    int seg_of(int strip, int row, int ny) const {
-        int k = (int)((long long)row * segs(strip) / ny);
-        while (k + 1 < segs(strip) && row0(strip, k + 1, ny) <= row) k++;
-        while (k > 0 && row0(strip, k, ny) > row) k--;
-        return k;
-    }
 };
 
 struct MarchEvent {
@@ -53,9 +47,6 @@ struct MarchEventCost {
 inline MarchEventCost march_event_cost(const MarchUnits &u, int nx, int ny, int bucket, std::vector<MarchEvent> &ev) {
     MarchEventCost c;
     const int nchunk = (nx + 3) / 4;
-    std::sort(ev.begin(), ev.end(), [](const MarchEvent &a, const MarchEvent &b) {
-        return a.row != b.row ? a.row < b.row : a.source != b.source ? a.source : a.x < b.x;
-    });
     std::vector<unsigned long long> mask(ny, 0);
     std::vector<double> weight(ny, 0.);
     std::vector<int> count(ny, 0);
@@ -64,48 +55,62 @@ inline MarchEventCost march_event_cost(const MarchUnits &u, int nx, int ny, int 
         weight[e.row] += e.source ? 2.5 : 1.;
         c.row = std::max(c.row, ++count[e.row]);
     }
-    std::vector<int> first(u.nstrips + 1, 0);  // a strip's first unit
-    for (int s = 0; s < u.nstrips; s++) first[s + 1] = first[s] + u.segs(s);
+    std::vector<int> col(u.nstrips + 1, nx), first(u.nstrips + 1, 0);  // a strip's first column and first unit
+    for (int s = 0; s < u.nstrips; s++) {
+        col[s] = 4 * march_cut(s, u.nstrips, nchunk);
+        first[s + 1] = first[s] + u.segs(s);
+    }
+    std::vector<int> rows[2];  // the first rows of the segments of the strips without and with walls, and ny
+    for (int k = 0; k <= u.nseg; k++) rows[0].push_back(march_row(k, u.nseg, ny, u.he));
+    for (int k = 0; k <= u.nsegx; k++) rows[1].push_back(u.nsegx ? march_row(k, u.nsegx, ny, 0) : ny);
+    auto last_from = [](const std::vector<int> &v, int at) {  // the last of them that begins at or before `at`
+        const int n = (int)v.size() - 1;
+        int k = std::min((int)((double)at * n / v[n]), n - 1);  // (cut about evenly)
+        while (k + 1 < n && v[k + 1] <= at) k++;
+        while (k > 0 && v[k] > at) k--;
+        return k;
+    };
     std::vector<int> rec(first[u.nstrips], 0);
     const int out = u.K - 1;  // rows that a unit marches before and after its own
-    for (size_t i = 0; i < ev.size(); i++) {
-        const MarchEvent &e = ev[i];
-        int own = (int)((long long)(e.x / 4) * u.nstrips / nchunk);
-        while (own + 1 < u.nstrips && 4 * march_cut(own + 1, u.nstrips, nchunk) <= e.x) own++;
-        while (own > 0 && 4 * march_cut(own, u.nstrips, nchunk) > e.x) own--;
-        if (!e.source) {
-            rec[first[own] + u.seg_of(own, e.row, ny)]++;
-            continue;
-        }
-        const bool twice = i > 0 && ev[i - 1].source && ev[i - 1].row == e.row && ev[i - 1].x == e.x;
+    const auto sources = std::partition(ev.begin(), ev.end(), [](const MarchEvent &e) { return !e.source; });
+    for (auto e = ev.begin(); e != sources; ++e) {
+        const int s = last_from(col, e->x);
+        rec[first[s] + last_from(rows[u.walled(s)], e->row)]++;
+    }
+    std::sort(sources, ev.end(), [](const MarchEvent &a, const MarchEvent &b) {
+        return a.row != b.row ? a.row < b.row : a.x < b.x;
+    });
+    for (auto e = sources; e != ev.end(); ++e) {
+        const bool twice = e != sources && (e - 1)->row == e->row && (e - 1)->x == e->x;
+        const int own = last_from(col, e->x);
         // strips (56 to 112 columns wide, or one) whose 128 columns hold the source, once or, on a narrow grid, several times
         for (int d = -std::min(3, (u.nstrips - 1) / 2); d <= std::min(3, u.nstrips / 2); d++) {
             const int s = (own + d + u.nstrips) % u.nstrips;
-            int dx = (e.x - (4 * march_cut(s, u.nstrips, nchunk) - u.H)) % nx;
+            int dx = (e->x - (col[s] - u.H)) % nx;
             dx += dx < 0 ? nx : 0;
             const int copies = dx < 128 ? (127 - dx) / nx + 1 : 0;
             if (!copies) continue;
-            for (int y = e.row - (out + ny - 1) / ny * ny; y < ny + out; y += ny)  // the rows that wrap to it
-                for (int k = u.seg_of(s, std::min(std::max(y - out, 0), ny - 1), ny);
-                     k < u.segs(s) && u.row0(s, k, ny) - out <= y; k++)
-                    if (y < u.row0(s, k + 1, ny) + out) rec[first[s] + k] += twice ? MARCH_RECORDS + 1 : copies;
+            const std::vector<int> &r = rows[u.walled(s)];
+            for (int y = e->row - (out + ny - 1) / ny * ny; y < ny + out; y += ny)  // the rows that wrap to it
+                for (int k = last_from(r, std::min(std::max(y - out, 0), ny - 1)); k < u.segs(s) && r[k] - out <= y; k++)
+                    if (y < r[k + 1] + out) rec[first[s] + k] += twice ? MARCH_RECORDS + 1 : copies;
         }
     }
     for (int s = 0; s < u.nstrips; s++) {
+        const std::vector<int> &r = rows[u.walled(s)];
         unsigned long long cols = 0;  // the buckets of the strip's columns
         bool known = false;
         for (int k = 0; k < u.segs(s); k++) {
             if (rec[first[s] + k] <= MARCH_RECORDS) continue;
             for (int j = 0; j < 128 && !known; j++) {
-                const int x = (4 * march_cut(s, u.nstrips, nchunk) - u.H + j) % nx;
+                const int x = (col[s] - u.H + j) % nx;
                 cols |= 1ull << ((x < 0 ? x + nx : x) / bucket);
             }
             known = true;
             double v = 0.;
-            for (int y = u.row0(s, k, ny) - out; y < u.row0(s, k + 1, ny) + out; y++) {
-                const int row = ((y % ny) + ny) % ny;
+            int row = (((r[k] - out) % ny) + ny) % ny;
+            for (int y = r[k] - out; y < r[k + 1] + out; y++, row = row + 1 == ny ? 0 : row + 1)
                 if (mask[row] & cols) v += weight[row];
-            }
             c.visits = std::max(c.visits, v);
         }
     }
