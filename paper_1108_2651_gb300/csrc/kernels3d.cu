@@ -139,8 +139,12 @@ __global__ void __launch_bounds__(BLOCK) step3d(StepArgs a) {
 // With WL, pulls across walls follow wall_sign3 and the absorbing layer's
 // factor fx(x) fy(y) fz(z) scales the result.
 // With SIG, sigma of the state that the step starts from goes to sig[3][plane] (the adjoint's record).
+// Registers: uncapped 60, 63 with mu (4 blocks an SM); with walls or sigma 48 (5 blocks), which hold without spilling when
+// the sources' terms are added at every site of a grid with events and not behind a flag kept for the site: 192^3 with walls
+// 187 us against 202 with the flag (8 bytes spilled), 96^3 28.5 and 30.7; uncapped kernels capped too took 460 x 250 x 3
+// from 80 to 84 us.
 template <bool MU, bool WL = false, bool SIG = false>
-__global__ void __launch_bounds__(BLOCK, 5) step3d_site(StepArgs a, Walls w, float *sig) {
+__global__ void __launch_bounds__(BLOCK, WL || SIG ? 5 : 1) step3d_site(StepArgs a, Walls w, float *sig) {
     const Grid &G = a.g;
     int row, x;
     site_of(G, row, x);
@@ -212,7 +216,7 @@ __global__ void __launch_bounds__(BLOCK, 5) step3d_site(StepArgs a, Walls w, flo
         sig[2 * G.plane + o] = m.sz;
     }
     collide3d_free(h, cl);
-    if (src) source3d(h, cl, shx, shy, shz);  // (S^ = 0 would add -0)
+    if (WL || SIG ? MU || a.evt.rowptr : src) source3d(h, cl, shx, shy, shz);  // (S^ = 0 adds -0)
     float *out = static_cast<float *>(a.out.data);
     if (WL && (w.fx || w.fy || w.fz)) {
         const float f = __fmul_rn(__fmul_rn(w.fx ? w.fx[x] : 1.f, w.fy ? w.fy[y] : 1.f), w.fz ? w.fz[z] : 1.f);
