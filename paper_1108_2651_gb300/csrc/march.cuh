@@ -175,7 +175,8 @@ __device__ __forceinline__ float4 m_round4(const PopBuf &b, float4 v) {
             return __fmaf_rn(q, f, 0.f);
         };
         float4 r = make_float4(one(v.x), one(v.y), one(v.z), one(v.w));
-        if (!(m < 0x1p+100f)) r.x = r.y = r.z = r.w = __fmul_rn(32767.f, pow2f(112));
+        // huge or NaN: what reading back the saturated block gives, which is not 32767 2^112 (the decoder's product overflows)
+        if (!(m < 0x1p+100f)) r.x = r.y = r.z = r.w = i16x2_to_f2(0x7fff7fffu, i16b_factor(127)).x;
         return r;
     } else {
         uint2 r;
