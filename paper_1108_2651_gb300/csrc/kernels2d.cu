@@ -725,9 +725,10 @@ __device__ __forceinline__ float wall_sign(int kind) { return kind == 1 ? -1.f :
 // (with walls, where x + c_i lies beyond a wall, buf_i(x) is what site x pulls back: s g^(0)_opp(i)(x))
 // (anisotropic medium, ratio r = c_x / c_y: moving particles of axis x get (r/2)(Lambda + c_x B_y), of axis y
 // (1/(2r))(Lambda - c_y B_x), the rest one (w0/c^2) Lambda with w0 = 1 - c^2 (r + 1/r))
+// (16-bit storage, whose grids are periodic and isotropic)
 template <int ST>
 __global__ void __launch_bounds__(BLOCK) init2d(Grid G, PopBuf out, const float *cL2, const float *E, const float *B,
-                                                long long nsite, Walls w, float r) {
+                                                long long nsite) {
     using C = Codec<ST>;
     const long long tid = (long long)blockIdx.x * BLOCK + threadIdx.x;
     const int row = (int)(tid / G.nchunk_pad);
@@ -739,35 +740,21 @@ __global__ void __launch_bounds__(BLOCK) init2d(Grid G, PopBuf out, const float 
         for (int j = 0; j < 4; j++) {
             const int x = 4 * c + j;
             if (x >= G.nx) break;
-            int xs = x + cx[i], ys = row + cy[i], ie = i;
-            float sg = 1.f;
-            if (w.kind[0] && (xs < 0 || xs >= G.nx)) {
-                xs = x;
-                ie = opp2d(i);
-                sg = wall_sign(w.kind[0]);
-            } else if (w.kind[1] && (ys < 0 || ys >= G.ny)) {
-                ys = row;
-                ie = opp2d(i);
-                sg = wall_sign(w.kind[1]);
-            }
-            xs = (xs + G.nx) % G.nx;
-            ys = (ys + G.ny) % G.ny;
+            const int xs = (x + cx[i] + G.nx) % G.nx, ys = (row + cy[i] + G.ny) % G.ny;
             const long long sd = (long long)ys * G.nx + xs;
             const float cl = cL2[(long long)ys * G.pitch + xs];
             const float Lam = E ? -E[2 * nsite + sd] : 0.f;
             const float bx = B ? B[sd] : 0.f, by = B ? B[nsite + sd] : 0.f;
             // Eq. 8: g^(0)_i = (w_i / c_L^2) [Lambda + c_ix B_y - c_iy B_x]
-            float wc;
-            if (r == 1.f) wc = (ie == 0) ? (1.f - 2.f * cl) / cl : 0.5f;
-            else wc = (ie == 0) ? (1.f - (r + 1.f / r) * cl) / cl : (cx[ie] ? 0.5f * r : 0.5f / r);
-            set(v, j, sg * (wc * (Lam + cx[ie] * by - cy[ie] * bx)));
+            const float wc = i == 0 ? (1.f - 2.f * cl) / cl : 0.5f;
+            set(v, j, wc * (Lam + cx[i] * by - cy[i] * bx));
         }
         C::store4(out, i, row, c, v);
     }
 }
 
 // FP32: one site per thread, its neighbours' fields by coalesced loads, and the traces cleared alongside; bound by HBM
-// (20 bytes written a site, 16 read).  The sums and products are those above.  4096^2 294 -> 166 us (four sites a lane,
+// (20 bytes written a site, 16 read).  The sums and products are those above, with walls and a tensor besides.  4096^2 294 -> 166 us (four sites a lane,
 // remainders for every neighbour and strided loads before), 256^2 8.6 -> 4 us.
 template <bool WL>
 __global__ void __launch_bounds__(BLOCK) init2d_site(Grid G, float *out, const float *cL2, const float *E, const float *B,
@@ -822,17 +809,18 @@ cudaError_t launch_init_2d(const lbem_t *h, const float *E, const float *B, cuda
                 G, static_cast<float *>(o.data), h->cL2, E, B, h->nsite, w, r, h->d_traces,
                 h->d_traces ? (long long)h->nrec * h->cap : 0);
             break;
-        case LBEM_F16: init2d<LBEM_F16><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite, w, r); break;
-        case LBEM_BF16: init2d<LBEM_BF16><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite, w, r); break;
-        default: init2d<LBEM_I16B><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite, w, r); break;
+        case LBEM_F16: init2d<LBEM_F16><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite); break;
+        case LBEM_BF16: init2d<LBEM_BF16><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite); break;
+        default: init2d<LBEM_I16B><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite); break;
     }
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ field extraction (dense [3][nsite] outputs)
+// (16-bit storage)
 template <int ST>
 __global__ void __launch_bounds__(BLOCK) fields2d(Grid G, PopBuf in, const float *cL2, float *E, float *B,
-                                                  long long nsite, Walls w, const float *Pz, float r) {
+                                                  long long nsite) {
     using C = Codec<ST>;
     const int lane = threadIdx.x & 31;
     const long long wg = ((long long)blockIdx.x * BLOCK + threadIdx.x) >> 5;
@@ -847,23 +835,16 @@ __global__ void __launch_bounds__(BLOCK) fields2d(Grid G, PopBuf in, const float
     for (int j = 0; j < 4; j++) {
         const int x = 4 * c + j;
         if (x >= G.nx) break;
-        // pulls across a wall
-        if (w.kind[0] && x == 0) set(g[1], j, wall_sign(w.kind[0]) * C::load1(in, 3, row, x));
-        if (w.kind[0] && x == G.nx - 1) set(g[3], j, wall_sign(w.kind[0]) * C::load1(in, 1, row, x));
-        if (w.kind[1] && row == 0) set(g[2], j, wall_sign(w.kind[1]) * C::load1(in, 4, row, x));
-        if (w.kind[1] && row == G.ny - 1) set(g[4], j, wall_sign(w.kind[1]) * C::load1(in, 2, row, x));
         const long long sd = (long long)row * G.nx + x;
         const float s = ((get(g[0], j) + get(g[1], j)) + (get(g[2], j) + get(g[3], j))) + get(g[4], j);
         if (E) {
             E[sd] = 0.f;
             E[nsite + sd] = 0.f;
-            const float ez = -get(cl, j) * s;
-            E[2 * nsite + sd] = Pz ? __fsub_rn(ez, Pz[(long long)row * G.pitch + x]) : ez;  // E = D/eps_inf - P
+            E[2 * nsite + sd] = -get(cl, j) * s;
         }
-        if (B) {  // anisotropic medium: B_x = r (g_4 - g_2), B_y = (g_1 - g_3) / r
-            const float bx = get(g[4], j) - get(g[2], j), by = get(g[1], j) - get(g[3], j);
-            B[sd] = r == 1.f ? bx : __fmul_rn(r, bx);
-            B[nsite + sd] = r == 1.f ? by : __fmul_rn(__fdiv_rn(1.f, r), by);
+        if (B) {
+            B[sd] = get(g[4], j) - get(g[2], j);
+            B[nsite + sd] = get(g[1], j) - get(g[3], j);
             B[2 * nsite + sd] = 0.f;
         }
     }
@@ -889,9 +870,9 @@ __global__ void __launch_bounds__(BLOCK) fields2d_site(Grid G, const float *in, 
         const float ez = -__ldg(cL2 + o) * (((g[0] + g[1]) + (g[2] + g[3])) + g[4]);
         E[sd] = 0.f;
         E[nsite + sd] = 0.f;
-        E[2 * nsite + sd] = Pz ? __fsub_rn(ez, Pz[o]) : ez;
+        E[2 * nsite + sd] = Pz ? __fsub_rn(ez, Pz[o]) : ez;  // E = D/eps_inf - P
     }
-    if (B) {
+    if (B) {  // anisotropic medium: B_x = r (g_4 - g_2), B_y = (g_1 - g_3) / r
         const float bx = g[4] - g[2], by = g[1] - g[3];
         B[sd] = r == 1.f ? bx : __fmul_rn(r, bx);
         B[nsite + sd] = r == 1.f ? by : __fmul_rn(__fdiv_rn(1.f, r), by);
@@ -912,9 +893,9 @@ cudaError_t launch_fields_2d(const lbem_t *h, float *E, float *B, cudaStream_t s
             fields2d_site<<<(unsigned)(((long long)G.ny * G.pitch + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
                 G, static_cast<const float *>(in.data), h->cL2, E, B, h->nsite, w, Pz, r);
             break;
-        case LBEM_F16: fields2d<LBEM_F16><<<blocks, BLOCK, 0, s>>>(G, in, h->cL2, E, B, h->nsite, w, Pz, r); break;
-        case LBEM_BF16: fields2d<LBEM_BF16><<<blocks, BLOCK, 0, s>>>(G, in, h->cL2, E, B, h->nsite, w, Pz, r); break;
-        default: fields2d<LBEM_I16B><<<blocks, BLOCK, 0, s>>>(G, in, h->cL2, E, B, h->nsite, w, Pz, r); break;
+        case LBEM_F16: fields2d<LBEM_F16><<<blocks, BLOCK, 0, s>>>(G, in, h->cL2, E, B, h->nsite); break;
+        case LBEM_BF16: fields2d<LBEM_BF16><<<blocks, BLOCK, 0, s>>>(G, in, h->cL2, E, B, h->nsite); break;
+        default: fields2d<LBEM_I16B><<<blocks, BLOCK, 0, s>>>(G, in, h->cL2, E, B, h->nsite); break;
     }
     return cudaGetLastError();
 }

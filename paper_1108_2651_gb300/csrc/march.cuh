@@ -117,8 +117,8 @@ struct MarchArgs {
     int steps;            // 1 .. K
     int nstrips, nseg;    // units: strips of columns by segments of rows
     // Walls: the first nl and last nr strips hold walled columns or layers; they have nsegx segments, and the first and
-    // last segments of a strip hold he (hex) rows (0: as the others)
-    int nl, nr, nsegx, he, hex;
+    // last segments of the others he rows (0: as the rest)
+    int nl, nr, nsegx, he;
 };
 
 template <int ST, int MED, int K, int D>
@@ -633,13 +633,12 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
             set(n.p4, k, __fadd_rn(get(n.p4, k), Ty));
         }
     };
-    // One row, every level one row further.  EV: a row with events; its straight line only hands the quads of the lanes
-    // concerned to their places in shared memory, and (SRC: with sources, or in a launch of fewer than K steps) adds the
-    // sources' terms (S^ = 0 adds -0 and changes nothing); the records are gone through once, before and after.  With
-    // their code at every level the row was 20 KB that the instruction cache did not hold, 3 us against 0.5 us of a
-    // plain one.
+    // One row, every level one row further.  EV: a row with events, or in a launch of fewer than K steps; its straight line
+    // only hands the quads of the lanes concerned to their places in shared memory, and adds the sources' terms (S^ = 0
+    // adds -0 and changes nothing); the records are gone through once, before and after.  With their code at every level
+    // the row was 20 KB that the instruction cache did not hold, 3 us against 0.5 us of a plain one.
     auto row = [&](auto mode) {
-        constexpr bool EV = decltype(mode)::ev, SRC = EV;
+        constexpr bool EV = decltype(mode)::ev;
         const unsigned s = smem + st * SB + lane * (PS / 32);
         float4 g0, a1, g2, a3, g4, P = z4, J = z4;
         stage(s, g0, a1, g2, a3, g4, P, J);
@@ -647,7 +646,7 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
         unsigned levels = 0, recs = 0;  // EV: the levels to leave the line at, the records of the row's levels
         unsigned long long place = 0;   // the lane's place per level (6 bits, 32: none)
         if (EV) {
-            if (SRC && kp < K) levels = 1u << (kp - 1);
+            if (kp < K) levels = 1u << (kp - 1);
             recs = __ballot_sync(FULL, (unsigned)(yl - erow) < (unsigned)K);
 #pragma unroll 1
             for (unsigned b = recs; b; b &= b - 1) {
@@ -658,7 +657,7 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
                 if ((v.y & 31) == lane) {
                     const unsigned q = (unsigned)v.y >> 8;
                     place |= (unsigned long long)(32 | q) << (6 * j);
-                    if (SRC && !(v.y & 128))
+                    if (!(v.y & 128))
                         m_sts1(smem + Cfg::O_Q + q * Cfg::QB + 80 + ((v.y >> 5) & 3) * 4,
                                __fsub_rn(0.f, m_lds1(smem + Cfg::O_AMP + (l * K + j) * 4)));
                 }
@@ -688,14 +687,14 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
                     m_sts(q + 32, h2);
                     m_sts(q + 48, g3);
                     m_sts(q + 64, h4);
-                    if (SRC) S = m_lds(q + 80);
+                    S = m_lds(q + 80);
                     if (MED == MARCH_POLE) m_sts(q + 96, Pn);
                 }
-                if (SRC && MED == MARCH_MU)
+                if (MED == MARCH_MU)
                     sh = make_float4(__fadd_rn(sh.x, S.x), __fadd_rn(sh.y, S.y), __fadd_rn(sh.z, S.z), __fadd_rn(sh.w, S.w));
             }
             m_collide<MED>(h0, g1, h2, g3, h4, c, Pn, sh, r, ri, fs, n, sig);
-            if (SRC && MED != MARCH_MU && leave) source(c, S, n);
+            if (EV && MED != MARCH_MU && leave) source(c, S, n);
             if (MED == MARCH_POLE) pole(mr, c, sig, Jn, Pn);
             if (WL) layer(yl - j, n);
             // 16-bit storage: the state is rounded after every second step (and as it is stored)
@@ -710,12 +709,12 @@ __device__ __forceinline__ void march_unit(const StepArgs &a, const Walls &w, in
                 PP[j] = Po;
                 JJ[j] = Jo;
             }
-            if (SRC && leave && j < K - 1 && j == kp - 1) store(yl - j, n, Pn, Jn);
+            if (EV && leave && j < K - 1 && j == kp - 1) store(yl - j, n, Pn, Jn);
             o = n;
             Po = Pn;
             Jo = Jn;
         }
-        if (!SRC || kp == K) store(yl - (K - 1), o, Po, Jo);
+        if (!EV || kp == K) store(yl - (K - 1), o, Po, Jo);
         if (EV) {  // the receivers
 #pragma unroll 1
             for (unsigned b = recs; b; b &= b - 1) {
@@ -867,8 +866,8 @@ __global__ void __launch_bounds__(32, 8) march2d(const __grid_constant__ MarchAr
         if (blockIdx.x < nbx) {
             const int seg = blockIdx.x / nx, k = blockIdx.x - seg * nx;
             strip = k < m.nl ? k : m.nstrips - nx + k;
-            y0 = march_row(seg, m.nsegx, G.ny, m.hex);
-            y1 = march_row(seg + 1, m.nsegx, G.ny, m.hex);
+            y0 = march_cut(seg, m.nsegx, G.ny);
+            y1 = march_cut(seg + 1, m.nsegx, G.ny);
         } else {
             const int b = blockIdx.x - nbx, n = m.nstrips - nx, seg = b / n;
             strip = m.nl + b - seg * n;
@@ -907,7 +906,7 @@ static cudaError_t launch_march(const StepArgs &a, const Walls &w, int nsteps, c
     m.w = w;
     m.nstrips = (a.g.nchunk + Cfg::W / 4 - 1) / (Cfg::W / 4);
     const int cap = fit.per_sm * fit.nsm;
-    m.nl = m.nr = m.nsegx = m.he = m.hex = 0;
+    m.nl = m.nr = m.nsegx = m.he = 0;
     if (WL && w.kind[0]) {  // strips whose columns (with the halo) reach a wall or its layer
         const int edge = std::max(w.nlayer, 1);
         auto x0 = [&](int k) { return 4 * march_cut(k, m.nstrips, a.g.nchunk) - Cfg::H; };
