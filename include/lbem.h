@@ -260,14 +260,14 @@ lbem_status lbem_set_watchdog(lbem_t *h, int every, double max_growth);
  * steps_per_pass = 3, every step of these media is a single step.
  * With steps_per_pass = 2 and tile_shape = -1 (the default), a call of lbem_step runs several steps
  * per launch by the marching kernel instead, wherever launches of two steps apply but for a pole in an anisotropic
- * medium, if it has at least 3 steps (5 with LBEM_F16, LBEM_BF16 or walls; up to 7 on some grids) and its sources and
+ * medium, if it has at least 3 steps (up to 7 with LBEM_F16, LBEM_BF16, walls or very long rows) and its sources and
  * receivers do not crowd a few rows and columns (shorter and crowded runs are faster by two): a warp walks a strip of columns down its rows with 8 time levels in flight (6 with a heterogeneous mu or a
  * pole, 4 with LBEM_I16B; the last launch of a call takes the steps left; walls and layers are applied on the way, with
  * no pass after it).  The results are the same bits again: those of single steps for FP32 storage, of launches of two
  * steps for 16-bit storage, whose state is rounded after every second step.  A tile shape >= 0 gives launches of two
  * steps.
  * 3D: with steps_per_pass = 2 (the default) and uniform mu, steps run three per launch where that takes less time than
- * single steps (not on small grids), walls and layers included, what is left over one by one; the same bits.  With 1, or
+ * single steps (not on small or flat grids, nor with very many receivers), walls and layers included, what is left over one by one; the same bits.  With 1, or
  * a heterogeneous mu, every step is a single step.
  * LBEM_ERR_ARG for values outside the current handle's set. */
 lbem_status lbem_set_temporal_blocking(lbem_t *h, int steps_per_pass, int tile_shape);

@@ -206,17 +206,21 @@ static int two_step_shape(const lbem_t *h) {
 }
 // The fewest steps of a call that marching takes less time for than launches of two steps.  A launch of fewer steps than
 // the kernel's K computes all K levels, so a short call's launch takes almost the time of a full one.  Measured on 21 grids
-// from 64^2 to 4096^2 and 1 to 65536 rows (us a call, two-step launches and marching): three steps FP32 4096^2 230 and
-// 176, 1024^2 20.5 and 18.7, mu 24.6 and 18.5, a pole 32 and 24, block-int16 22.7 and 18.2, but on fewer than 8 rows and
-// very many columns, where a unit marches 2 rows and 2 (K - 1) more, 4 x 524288 41.0 and 45.6; with walls 1024^2 three
-// 41 and 47, four 45 and 50, five 64 and 57; with walls and a tensor three 33 and 51, five 58 and 62, six 74 and 67
-// (1025 x 2047: five 92 and 68); FP16, whose launches of two steps move half the bytes, 1024^2 three 18.6 and 21.1, 4096^2
-// four 181 and 203, five 249 and 205; BF16 likewise.
+// from 64^2 to 4096^2 and 1 to 65536 rows (us a call, two-step launches and marching).  Three steps: FP32 4096^2 230 and
+// 176, 1024^2 20.5 and 18.7, mu 24.6 and 18.5, a pole 32 and 24, block-int16 22.7 and 18.2; but with fewer than 8 rows of
+// very many columns, where a unit marches 2 rows and 2 (K - 1) more, 4 x 524288 41.0 and 45.6.  Walls: 256^2 three 27.8 and
+// 20.1, but about 1024^2 three 41 and 47, four 45 and 50, five 64 and 57 (1025 x 2047 three 59 and 54); with a tensor 1024^2
+// three 33 and 51, five 58 and 62, six 74 and 67, 4096^2 four 254 and 270, five 377 and 274, 256^2 three 20.5 and 21.4, four
+// 32 and 28.  FP16, whose launches of two steps move half the bytes: 1024^2 three 18.6 and 21.1, 4096^2 four 181 and 203,
+// five 249 and 205, 4 x 524288 six 86 and 85; but narrower than a tile of 128 columns 65536 x 16 three 117 and 88.  BF16
+// likewise.
 static int march_min_steps(const lbem_t *h) {
-    const bool few_rows = h->grid.ny < 8 && h->grid.nx >= 1 << 18;
-    if (h->storage == LBEM_F16 || h->storage == LBEM_BF16) return few_rows ? 7 : 5;
-    if (h->walls() && !h->has_mu) return !h->aniso || h->nsite >= 1 << 21 ? 5 : 6;
-    return few_rows ? 4 : 3;
+    const long long nx = h->grid.nx, ny = h->grid.ny, n = nx * ny;
+    const bool long_rows = ny < 8 && nx >= 1 << 18, large = nx >= 512 && ny >= 100 && n >= 1 << 19;
+    if (h->storage == LBEM_F16 || h->storage == LBEM_BF16) return nx <= 128 || n <= 1 << 14 ? 3 : long_rows ? 7 : 5;
+    if (h->walls() && h->aniso) return ny <= 32 ? 3 : !large ? 4 : n < 1 << 21 ? 6 : 5;
+    if (h->walls()) return large && n <= 1 << 21 && !h->has_mu ? 5 : 3;
+    return long_rows && h->storage == LBEM_F32 && !h->has_mu && !h->disp ? 4 : 3;
 }
 // Whether marching takes less time than launches of two steps with the handle's events.  A warp goes through the events
 // of a unit that holds more than its records (march_event_cost) one by one, 0.15 us each (a source 0.35), for all the rows
