@@ -803,12 +803,15 @@ cudaError_t launch_init_2d(const lbem_t *h, const float *E, const float *B, cuda
     const Walls w = handle_walls(h);
     const float r = h->aniso_r;
     switch (h->storage) {
-        case LBEM_F32:
-            (w.kind[0] || w.kind[1] ? init2d_site<true> : init2d_site<false>)<<<
-                (unsigned)(((long long)G.ny * G.pitch + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
-                G, static_cast<float *>(o.data), h->cL2, E, B, h->nsite, w, r, h->d_traces,
-                h->d_traces ? (long long)h->nrec * h->cap : 0);
+        case LBEM_F32: {
+            const unsigned site_blocks = (unsigned)(((long long)G.ny * G.pitch + BLOCK - 1) / BLOCK);
+            long long ntr;
+            const cudaError_t e = traces_to_clear(h, site_blocks, s, &ntr);
+            if (e != cudaSuccess) return e;
+            (w.kind[0] || w.kind[1] ? init2d_site<true> : init2d_site<false>)<<<site_blocks, BLOCK, 0, s>>>(
+                G, static_cast<float *>(o.data), h->cL2, E, B, h->nsite, w, r, h->d_traces, ntr);
             break;
+        }
         case LBEM_F16: init2d<LBEM_F16><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite); break;
         case LBEM_BF16: init2d<LBEM_BF16><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite); break;
         default: init2d<LBEM_I16B><<<blocks, BLOCK, 0, s>>>(G, o, h->cL2, E, B, h->nsite); break;

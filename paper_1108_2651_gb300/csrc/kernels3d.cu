@@ -316,10 +316,12 @@ static Walls walls_of(const lbem_t *h) {
 cudaError_t launch_init_3d(const lbem_t *h, const float *E, const float *B, cudaStream_t s) {
     const Grid &G = h->grid;
     const Walls w = walls_of(h);
-    (w.kind[0] || w.kind[1] || w.kind[2] ? init3d<true> : init3d<false>)<<<
-        (unsigned)(((long long)G.nrows * G.pitch + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
-        G, static_cast<float *>(h->buf[h->cur].data), h->cL2, E, B, h->nsite, w, h->d_traces,
-        h->d_traces ? (long long)h->nrec * h->cap : 0);
+    const unsigned blocks = (unsigned)(((long long)G.nrows * G.pitch + BLOCK - 1) / BLOCK);
+    long long ntr;
+    const cudaError_t e = traces_to_clear(h, blocks, s, &ntr);
+    if (e != cudaSuccess) return e;
+    (w.kind[0] || w.kind[1] || w.kind[2] ? init3d<true> : init3d<false>)<<<blocks, BLOCK, 0, s>>>(
+        G, static_cast<float *>(h->buf[h->cur].data), h->cL2, E, B, h->nsite, w, h->d_traces, ntr);
     return cudaGetLastError();
 }
 

@@ -711,7 +711,16 @@ int batch_ss2_chunks(int shape);  // chunks of a full unit
 cudaError_t launch_batch_ss2(const StepArgs *args, const BatchUnit *units, int nunits, int *sched, const long long *t0p,
                              int toff, int par, const BatchPacked &pk, long long rows, int shape, cudaStream_t s);
 // The initial state from dense fields (null: zero); the FP32 kernels also clear the receivers' traces (ntr floats; 16-bit
-// storage leaves them to the caller).
+// storage leaves them to the caller): *ntr, those that a kernel of `blocks` blocks clears alongside.  More than 256 a thread
+// are cleared by a memset before it (16^2 with 4096 traces of 1000 samples 128 us in the kernel, 15 by memset; 64^2 with
+// 1024 of them, 250 a thread, 8.7 and 12.9).
+inline cudaError_t traces_to_clear(const lbem_t *h, unsigned blocks, cudaStream_t s, long long *ntr) {
+    *ntr = h->d_traces ? (long long)h->nrec * h->cap : 0;
+    if (*ntr <= 256LL * BLOCK * blocks) return cudaSuccess;
+    const size_t bytes = sizeof(float) * (size_t)*ntr;
+    *ntr = 0;
+    return cudaMemsetAsync(h->d_traces, 0, bytes, s);
+}
 cudaError_t launch_init_2d(const lbem_t *h, const float *E, const float *B, cudaStream_t s);
 cudaError_t launch_fields_2d(const lbem_t *h, float *E, float *B, cudaStream_t s);
 cudaError_t launch_diag_2d(const lbem_t *h, double *partials, int nblocks, cudaStream_t s);
