@@ -13,8 +13,10 @@ are larger than L2, so no flush is needed between steps.
 Metric: Mlups (10^6 lattice-site updates per second) = sites x 5000 / time.
 A launch moves 44 algorithmic bytes per site (5 populations read + 5 written
 in FP32, plus c_L^2), whether it advances one step or eight: single steps and
-pairs are bound by HBM bandwidth, the marching kernel by the issue of its
-arithmetic.
+pairs are bound by HBM bandwidth, the marching kernel by latency: with two
+warps a scheduler it waits for rows from HBM, for shared memory and for its
+own dependent arithmetic, and fills no unit (HBM and shared memory about
+70 % each, issue slots 45 %).
 
 --impl reference times the FP64 CPU oracle (test infrastructure) on a
 bounded sample of the same workload.  With torchrun (N > 1) the path shards:
@@ -67,10 +69,11 @@ def batch_kernel(variant):
 
 
 def steps_per_launch(p, storage, spp, tile_shape_set=False):
-    """Steps that one launch of lbem_step advances: with the two-step default and no tile shape chosen, those of the
-    marching kernel for the workload's medium and storage; else the steps per pass that were set."""
+    """Steps that one launch of lbem_step advances on this file's workloads: with the two-step default and no tile shape
+    chosen, those of the marching kernel for the workload's medium and storage; else the steps per pass that were set.
+    (3D: smaller boxes than 80^3 may take single steps, whichever the library finds the faster.)"""
     if p.D == 3:
-        return 3 if spp == 2 and p.mu_r is None else 1
+        return 3 if spp == 2 and p.mu_r is None and min(p.shape) >= 80 else 1
     pole, tensor = p.wp2 is not None, getattr(p, "aniso", None) is not None
     if spp != 2 or tile_shape_set or (pole and (tensor or p.mu_r is not None or any(p.bc))):
         return spp
