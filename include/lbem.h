@@ -220,7 +220,8 @@ lbem_status lbem_get_boundaries(const lbem_t *h, int kind[3], int *layer, double
  * single steps.  The update J <- ((1 - gamma/2) J - wr2 P + wp2 E) / (1 + gamma/2) runs with three per-site
  * coefficients formed once here in FP64 (no division per step).  The handle holds second J and P planes (every launch
  * writes J and P to the planes paired with its output
- * population buffer); lbem_set_fields starts the pole at rest (D = E); lbem_save_state
+ * population buffer; without room for the second J the handle steps by launches of one and two steps, J in place);
+ * lbem_set_fields starts the pole at rest (D = E); lbem_save_state
  * appends J and P (lbem_info's state_bytes counts them).  Batches and the
  * adjoint take non-dispersive handles only.  Synchronises the stream. */
 lbem_status lbem_set_dispersion(lbem_t *h, const float *wp2, const float *wr2, const float *gamma);

@@ -248,7 +248,8 @@ static bool march_events_ok(const lbem_t *h) {
 // steps per launch are the default and no shape was chosen (but for a pole in an anisotropic medium).  Shorter calls take
 // launches of two steps.
 static bool march_ok(const lbem_t *h) {
-    return h->tblock == 2 && !h->tb_shape_set && multi_step_base(h) && !(h->disp && h->aniso) && march_events_ok(h);
+    return h->tblock == 2 && !h->tb_shape_set && multi_step_base(h) && !(h->disp && (h->aniso || !h->d_J2)) &&
+           march_events_ok(h);
 }
 // 3D: triples of steps by the marching kernel (march3d.cu) where several steps per launch are the default, with uniform
 // mu; offsets in a plane must fit 32 bits.
@@ -705,7 +706,7 @@ lbem_status lbem_set_fields(lbem_t *h, const float *E, const float *B) {
         LBEM_CUDA(cudaMemsetAsync(h->d_traces, 0, sizeof(float) * (size_t)h->nrec * h->cap, h->stream));
     if (h->disp) {  // the pole starts at rest: D = E
         for (float *p : {h->d_J, h->d_J2, h->d_P, h->d_P2})
-            LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * (size_t)h->grid.plane, h->stream));
+            if (p) LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * (size_t)h->grid.plane, h->stream));
     }
     drop_graph(h);
     return LBEM_OK;
@@ -960,15 +961,28 @@ lbem_status lbem_set_dispersion(lbem_t *h, const float *wp2, const float *wr2, c
                                          " sites with a parameter not finite and >= 0, or wp^2 + wr^2 > 4 w0");
     const size_t pl = (size_t)h->grid.plane;  // stored as planes with the grid's pitch (padding zero)
     if (!h->d_wp2) {
-        for (float **p : {&h->d_wp2, &h->d_wr2, &h->d_gam, &h->d_J, &h->d_J2, &h->d_P, &h->d_P2, &h->d_pc, &h->d_pb,
-                          &h->d_pa})
-            LBEM_CUDA(gmalloc(h, (void **)p, sizeof(float) * pl, "dispersive pole"));
+        float **planes[] = {&h->d_wp2, &h->d_wr2, &h->d_gam, &h->d_J, &h->d_P, &h->d_P2, &h->d_pc, &h->d_pb, &h->d_pa};
+        cudaError_t e = cudaSuccess;
+        for (float **p : planes)
+            if (e == cudaSuccess) e = gmalloc(h, (void **)p, sizeof(float) * pl, "dispersive pole");
+        if (e != cudaSuccess) {  // all or none: d_wp2 stands for the rest
+            for (float **p : planes) {
+                gfree(h, *p);
+                *p = nullptr;
+            }
+            cudaGetLastError();
+            return cuda_fail(e, "lbem_set_dispersion");
+        }
+        // the marching kernel reads J at sites that other units advance, so it needs a second plane; without room for one
+        // the launches of one and two steps update J in place
+        if (gmalloc(h, (void **)&h->d_J2, sizeof(float) * pl, "dispersive pole") != cudaSuccess) cudaGetLastError();
     }
     const float *src[3] = {dp, dr, dg};
     float *dst[3] = {h->d_wp2, h->d_wr2, h->d_gam};
     for (int k = 0; k < 3; k++) LBEM_CUDA(launch_to_plane(h, src[k], dst[k], h->stream));
     LBEM_CUDA(launch_pole_coefficients(h, h->stream));
-    for (float *p : {h->d_J, h->d_J2, h->d_P, h->d_P2}) LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * pl, h->stream));
+    for (float *p : {h->d_J, h->d_J2, h->d_P, h->d_P2})
+        if (p) LBEM_CUDA(cudaMemsetAsync(p, 0, sizeof(float) * pl, h->stream));
     LBEM_CUDA(cudaStreamSynchronize(h->stream));
     h->disp = true;
     h->march_events = -1;

@@ -579,7 +579,7 @@ struct lbem {
           *d_P2 = nullptr;
     float *d_pc = nullptr, *d_pb = nullptr, *d_pa = nullptr;  // pole_update's coefficients (pole_coefficients)
     float *pole_P(int c) const { return c ? d_P2 : d_P; }
-    float *pole_J(int c) const { return c ? d_J2 : d_J; }
+    float *pole_J(int c) const { return c && d_J2 ? d_J2 : d_J; }  // (one plane, in place, where there was no room for two)
     bool disp = false;
     // anisotropic medium (lbem_set_medium_aniso): r = sqrt(mu_xx / mu_yy), mubar = sqrt(mu_xx mu_yy)
     bool aniso = false;

@@ -340,8 +340,8 @@ __device__ __forceinline__ void tb_step_a(const StepArgs &a, const float *IN, co
             constexpr int JPL = TbGeom<TBY, false, true>::JS_PL;
             pp.P = lds4(PS + py * TW + c);
             pp.J = pp.wp = pp.wr = pp.gm = make_float4(0.f, 0.f, 0.f, 0.f);
-            // lanes past nx (rows past ny) of a ragged last tile work on wrapped sites: their pole results only ever
-            // reach the row padding or are dropped
+            // lanes past nx (rows past ny) of a ragged last tile work on wrapped sites, whose J another tile may be
+            // writing where the handle has one plane: their pole results only ever reach the row padding or are dropped
             if (own) {
                 const float *js = JS + (py - 1) * TBX + 4 * lane;
                 pp.J = lds4(js);
