@@ -15,7 +15,7 @@
 // an SM (158 registers of levels' state a thread).  Measured per step at 192^3, single steps 179.6 us: K = 3 and 20 rows of
 // 10 warps 106.6 us; 16 rows 113.9, 24 rows of 12 warps 116.1, of 8 warps 122.9; one column a thread in 16 rows 136.0 (the chain of
 // one site's levels leaves the warps waiting); K = 2 148.3 to 177.0, K = 4 127.8 to 153.3 (the overlap grows to 2).
-// 96^3 25.1 -> 16.6 us; with walls and a layer 192^3 203 -> 135 us, 96^3 30.8 -> 21.9 us.
+// 96^3 25.1 -> 16.6 us; with walls and a layer 192^3 187 -> 135 us, 96^3 28.4 -> 21.9 us.
 // Sources and receivers: a block first marks, a word for each plane, its rows that have any (192^3 with 128 receivers 110 us
 // a step; with the row pointers looked up in the loop 123 us, most of it without an event in sight).
 // Each site update is collide3d_free, as in the single-step kernels, so the results are bit-identical to theirs.
