@@ -2,6 +2,7 @@
 // the device that was current when they were set or asked for: with one copy for the process, a handle on a second device
 // launched kernels without the attribute that their shared memory needs.
 #pragma once
+#include <atomic>
 #include <mutex>
 
 namespace lbk {
@@ -10,7 +11,7 @@ template <class T>
 class PerDevice {
     static constexpr int MAX = 64;
     std::mutex mu_;
-    bool have_[MAX] = {};
+    std::atomic<bool> have_[MAX] = {};  // val_ is written before, and not again
     T val_[MAX] = {};
 
   public:
@@ -19,13 +20,15 @@ class PerDevice {
     template <class Make>
     int get(int dev, Make make, T *out) {
         if (dev < 0 || dev >= MAX) return make(*out);
-        std::lock_guard<std::mutex> lock(mu_);
-        if (!have_[dev]) {
-            T v{};
-            const int e = make(v);
-            if (e != 0) return e;
-            val_[dev] = v;
-            have_[dev] = true;
+        if (!have_[dev].load(std::memory_order_acquire)) {
+            std::lock_guard<std::mutex> lock(mu_);
+            if (!have_[dev].load(std::memory_order_relaxed)) {
+                T v{};
+                const int e = make(v);
+                if (e != 0) return e;
+                val_[dev] = v;
+                have_[dev].store(true, std::memory_order_release);
+            }
         }
         *out = val_[dev];
         return 0;
